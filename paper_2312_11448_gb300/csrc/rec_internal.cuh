@@ -67,6 +67,13 @@ struct DevScalars {
   float Gf;          // G = (1 - C) lambda + C beta e_alpha
   float Ghi, Glo;    // G as a double-float pair
   float wscale;      // S1s / tally_total (0 without tallies)
+  // compact velocity copy of the march (rec_velq.cuh): the velocity that maps to
+  // 127, km/s (0: no usable copy), and the largest speed
+  float vq_u, vq_v;
+  // running maxima of the allocation's first pass as ordered bits (weight, velocity
+  // component, squared speed) and what was invalid (bit 0 weight, bit 1 velocity); 0 between calls
+  unsigned long long mx_w;
+  unsigned int mx_u, mx_v2, mx_bad;
 };
 
 // Batched contexts (several boxes in one context, one launch per phase for
@@ -93,6 +100,8 @@ struct BoxDev {
   uint32_t n, lg, nt, p2;  // side, log2 side (power of two), super-tiles per axis, side is a power of two
   uint64_t mn, mn2;        // multipliers ceil(2^64/n), ceil(2^64/n^2) of the exact divisions (n >= 2)
   uint32_t tlg;            // log2 of the super-tile side in use
+  uint32_t vbx;            // brick bits of the compact velocity copy
+  uint32_t* velq;          // compact velocity copy (rec_velq.cuh), NULL: none
   uint64_t npk;        // packets requested per transport
   uint64_t pk0;        // first packet of the box in the batch packet space (multiple of 64)
   uint32_t ablk0;      // first allocation block
@@ -151,6 +160,7 @@ struct rec_ctx {
   unsigned long long* bcap;  // march-queue bucket capacities / offsets [super-tiles]
   unsigned long long* bfill; // packets queued per bucket [super-tiles]
   unsigned long long* cpre;  // first march chunk of each bucket [super-tiles + 1]
+  uint32_t* velq = nullptr;  // compact velocity copy of the march (rec_velq.cuh); NULL: no memory for it
   unsigned long long* partQ; // allocation block sums / offsets [alloc blocks]
   void* quant;               // emission-profile table (float or double) [n_quantiles]
   int grid;                  // blocks of the streaming passes
@@ -263,6 +273,8 @@ void enqueue_newton_passes(rec_ctx* c, DevScalars* sc, const StepCoef& k, const 
 // rec_transport.cu
 cudaError_t launch_transport(rec_ctx* c, int step, double z, rec_stats* st);
 cudaError_t launch_transport_batch(rec_ctx* c, int step, double z, rec_stats* st);
+// Blocks of the single-box allocation passes.
+int alloc_blocks_single(int64_t n3);
 void transport_limits(bool mixed, bool batch, int* emit_max, int* march_max);
 // Largest march grid (blocks per SM) of the region-sweep march.
 int sweep_march_limit(bool mixed);

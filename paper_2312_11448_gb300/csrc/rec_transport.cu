@@ -34,6 +34,7 @@
 
 #include "rec_internal.cuh"
 #include "rec_reduce.cuh"
+#include "rec_velq.cuh"
 
 namespace rec {
 namespace {
@@ -192,30 +193,110 @@ template <> struct Draws<double> {
 };
 
 // ---- allocation -------------------------------------------------------------------
-// The maximum is taken in the working precision (exact for any precision), so
-// the binary32 form issues no binary64 instruction per cell.
-template <class R>
-__global__ void __launch_bounds__(kPassThreads) k_alloc_max(const R* emis, int64_t n3, DevScalars* sc, double* part) {
-  R m = (R)0;
+// Velocity components for the compact copy (rec_velq.cuh), which the march's bound
+// uses.  Binary64: bits moved to binary32 without the binary64 pipe, toward
+// zero for the copy and one unit up for the maxima; the ends of binary32's
+// range map to its smallest normal number and to infinity.
+__device__ __forceinline__ float velq_value(float v) { return v; }
+__device__ __forceinline__ float velq_upper(float v) { return fabsf(v); }
+__device__ __forceinline__ uint32_t velq_abs_bits(double v) {
+  const uint32_t hi = (uint32_t)__double2hiint(v) & 0x7fffffffu;
+  if (hi >= 0x47e00000u) return 0x7f800000u;
+  if (hi < 0x38100000u) return 0x00800000u;
+  return __funnelshift_l((uint32_t)__double2loint(v), hi, 3) + 0x40000000u;
+}
+__device__ __forceinline__ float velq_value(double v) {
+  return __uint_as_float(velq_abs_bits(v) | ((uint32_t)__double2hiint(v) & 0x80000000u));
+}
+__device__ __forceinline__ float velq_upper(double v) { return __uint_as_float(velq_abs_bits(v) + 1u); }
+
+// Largest |component| and squared speed of a velocity vector, running maxima;
+// anything not finite marks the box as unusable for the compact copy.
+struct VelMax {
+  float u = 0.0f, v2 = 0.0f;
   int bad = 0;
+  template <class V>
+  __device__ __forceinline__ void add(const V& U) {
+    const float x = velq_upper(U.x), y = velq_upper(U.y), z = velq_upper(U.z);
+    bad |= !(x < 3e38f) || !(y < 3e38f) || !(z < 3e38f);
+    u = fmaxf(u, fmaxf(x, fmaxf(y, z)));
+    v2 = fmaxf(v2, x * x + y * y + z * z);
+  }
+};
+// Bits of a non-negative number; as unsigned integers they order like the numbers.
+__device__ __forceinline__ uint64_t order_bits(float v) { return __float_as_uint(v) & 0x7fffffffu; }
+__device__ __forceinline__ uint64_t order_bits(double v) {
+  return (uint64_t)__double_as_longlong(v) & 0x7fffffffffffffffull;
+}
+__device__ __forceinline__ float from_order_bits(uint64_t b, float) { return __uint_as_float((uint32_t)b); }
+__device__ __forceinline__ double from_order_bits(uint64_t b, double) { return __longlong_as_double((long long)b); }
+
+// Largest weight and velocity of a block into the box's running maxima: warp
+// maxima by integer reductions of the ordered bits (a maximum in binary64 would go
+// through the slow pipe five times per value), one atomic maximum per block and value.
+// bad: bit 0 an invalid weight, bit 1 a velocity that is not finite.
+template <int NTH>
+__device__ __forceinline__ void block_maxima(DevScalars* sc, uint64_t w, const VelMax& vm, bool bad) {
+  __shared__ uint32_t sm[NTH / 32][5];
+  const unsigned full = 0xffffffffu;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  auto max64 = [&](uint32_t hi, uint32_t lo, uint32_t* h, uint32_t* l) {
+    *h = __reduce_max_sync(full, hi);
+    *l = __reduce_max_sync(full, hi == *h ? lo : 0u);
+  };
+  uint32_t h, l;
+  max64((uint32_t)(w >> 32), (uint32_t)w, &h, &l);
+  const uint32_t u = __reduce_max_sync(full, __float_as_uint(vm.u));
+  const uint32_t v2 = __reduce_max_sync(full, __float_as_uint(vm.v2));
+  const uint32_t b = __reduce_or_sync(full, (bad ? 1u : 0u) | (vm.bad ? 2u : 0u));
+  __syncthreads();  // sm may still be read by a previous call
+  if (lane == 0) { sm[warp][0] = h; sm[warp][1] = l; sm[warp][2] = u; sm[warp][3] = v2; sm[warp][4] = b; }
+  __syncthreads();
+  if (warp == 0) {
+    const bool in = lane < NTH / 32;
+    max64(in ? sm[lane][0] : 0u, in ? sm[lane][1] : 0u, &h, &l);
+    const uint32_t bu = __reduce_max_sync(full, in ? sm[lane][2] : 0u);
+    const uint32_t bv = __reduce_max_sync(full, in ? sm[lane][3] : 0u);
+    const uint32_t bb = __reduce_or_sync(full, in ? sm[lane][4] : 0u);
+    if (lane == 0) {
+      atomicMax(&sc->mx_w, ((unsigned long long)h << 32) | l);
+      atomicMax(&sc->mx_u, bu);
+      atomicMax(&sc->mx_v2, bv);
+      if (bb) atomicOr(&sc->mx_bad, bb);
+    }
+  }
+}
+// The box's maxima once every block has added its own (one thread); ready for the next call.
+template <class R>
+__device__ __forceinline__ void take_maxima(DevScalars* sc, float kappa) {
+  const uint32_t bad = __ldcg(&sc->mx_bad);
+  sc->rmax = bad & 1u ? 0.0 : (double)from_order_bits(__ldcg(&sc->mx_w), (R)0);  // invalid weights: emit nothing
+  sc->flags &= ~(2 | 4 | 16);                                                    // transport flags describe this call only
+  if (bad & 1u) sc->flags |= 4;
+  sc->vq_u = velq_scale(__uint_as_float(__ldcg(&sc->mx_u)), (bad & 2u) != 0u, kappa);
+  sc->vq_v = sqrtf(__uint_as_float(__ldcg(&sc->mx_v2))) * 1.00001f;
+  sc->mx_w = 0;
+  sc->mx_u = sc->mx_v2 = sc->mx_bad = 0;
+}
+
+// Reads the emission weights once (their maximum, exact in the working precision)
+// and the velocities once (the scale of their compact copy).
+template <class R>
+__global__ void __launch_bounds__(kPassThreads) k_alloc_max(const R* emis, const typename Vec4<R>::T* vel, int64_t n3,
+                                                            float kappa, DevScalars* sc) {
+  R m = (R)0;
+  bool bad = false;
+  VelMax vm;
   for (int64_t i = (int64_t)blockIdx.x * kPassThreads + threadIdx.x; i < n3; i += (int64_t)gridDim.x * kPassThreads) {
     const R r = emis[i];
-    if (!(r >= (R)0) || isinf(r)) bad = 1;
-    else m = fmax(m, r);
+    if (!(r >= (R)0) || isinf(r)) bad = true;
+    else m = m < r ? r : m;
+    vm.add(vel[i]);
   }
-  bad = __syncthreads_or(bad);
-  double bm = block_max<kPassThreads>((double)m);
-  if (threadIdx.x == 0) {
-    part[(size_t)blockIdx.x * kMaxSums + 0] = bm;
-    part[(size_t)blockIdx.x * kMaxSums + 1] = bad ? 1.0 : 0.0;
-  }
+  block_maxima<kPassThreads>(sc, order_bits(m), vm, bad);
   if (!last_block_done(&sc->counter)) return;
-  double mx = combine_max<kPassThreads>(part, gridDim.x, kMaxSums, 0);
-  double anybad = combine_max<kPassThreads>(part, gridDim.x, kMaxSums, 1);
   if (threadIdx.x == 0) {
-    sc->rmax = anybad > 0.0 ? 0.0 : mx;  // invalid weights: emit nothing
-    sc->flags &= ~(2 | 4 | 16);          // transport flags describe this call only
-    if (anybad > 0.0) sc->flags |= 4;
+    take_maxima<R>(sc, kappa);
     sc->counter = 0;
   }
 }
@@ -302,41 +383,62 @@ inline Tiles make_tiles(int n, int tile) {
   return t;
 }
 
-// The allocation kernels give each thread kAllocItems consecutive cells.
-template <class R>
-__device__ __forceinline__ void load_items(const R* p, int64_t c0, int64_t n3, R (&v)[kAllocItems]) {
-  if (c0 + kAllocItems <= n3 && (reinterpret_cast<uintptr_t>(p) & 15u) == 0) {
+// Compact copy of the velocities of AT * IT consecutive cells (one block).
+template <class R, int IT, class V>
+__device__ __forceinline__ void velq_write(const V* vel, int64_t n3, int64_t c0, float u, uint32_t* velq, uint32_t bx,
+                                           const Tiles& tl) {
+  if (!velq || !(u > 0.0f)) return;
+  const float qs = 127.0f / u;
+#pragma unroll 4
+  for (int k = 0; k < IT; ++k) {
+    const int64_t i = c0 + (int64_t)k * AT + threadIdx.x;
+    if (i >= n3) break;
+    const V U = vel[i];
+    uint32_t ix, iy, iz;
+    tl.template coords<false>((uint32_t)i, &ix, &iy, &iz);
+    velq[velq_x(ix) | velq_y(iy, bx) | velq_z(iz, bx)] =
+        velq_pack(velq_value(U.x), velq_value(U.y), velq_value(U.z), qs);
+  }
+}
+
+// The allocation kernels give each thread IT consecutive cells.
+template <class R, int IT>
+__device__ __forceinline__ void load_items(const R* p, int64_t c0, int64_t n3, R (&v)[IT]) {
+  if (IT >= 4 && c0 + IT <= n3 && (reinterpret_cast<uintptr_t>(p) & 15u) == 0) {
     if (sizeof(R) == 4) {
       const float4* q = reinterpret_cast<const float4*>(p + c0);
 #pragma unroll
-      for (int k = 0; k < kAllocItems / 4; ++k) {
+      for (int k = 0; k < IT / 4; ++k) {
         float4 t = q[k];
         v[4 * k] = (R)t.x; v[4 * k + 1] = (R)t.y; v[4 * k + 2] = (R)t.z; v[4 * k + 3] = (R)t.w;
       }
     } else {
       const double2* q = reinterpret_cast<const double2*>(p + c0);
 #pragma unroll
-      for (int k = 0; k < kAllocItems / 2; ++k) {
+      for (int k = 0; k < IT / 2; ++k) {
         double2 t = q[k];
         v[2 * k] = (R)t.x; v[2 * k + 1] = (R)t.y;
       }
     }
   } else {
 #pragma unroll
-    for (int k = 0; k < kAllocItems; ++k) v[k] = (c0 + k < n3) ? p[c0 + k] : (R)0;
+    for (int k = 0; k < IT; ++k) v[k] = (c0 + k < n3) ? p[c0 + k] : (R)0;
   }
 }
 
-template <class R>
-__global__ void __launch_bounds__(AT) k_alloc_sum(const R* emis, int64_t n3, uint64_t n_packets, Stream strm,
-                                                  DevScalars* sc, unsigned long long* partQ, uint32_t* P) {
+template <class R, int IT>
+__global__ void __launch_bounds__(AT) k_alloc_sum(const R* emis, const typename Vec4<R>::T* vel, int64_t n3,
+                                                  uint64_t n_packets, Stream strm, DevScalars* sc,
+                                                  unsigned long long* partQ, uint32_t* P, uint32_t* velq, uint32_t vbx,
+                                                  Tiles tl) {
   const R rmax = (R)sc->rmax;
+  velq_write<R, IT>(vel, n3, (int64_t)blockIdx.x * (AT * IT), sc->vq_u, velq, vbx, tl);
   uint64_t acc = 0;
   if (rmax > (R)0) {
-    R v[kAllocItems];
-    load_items<R>(emis, (int64_t)blockIdx.x * kAllocChunk + (int64_t)threadIdx.x * kAllocItems, n3, v);
+    R v[IT];
+    load_items<R, IT>(emis, (int64_t)blockIdx.x * (AT * IT) + (int64_t)threadIdx.x * IT, n3, v);
 #pragma unroll
-    for (int k = 0; k < kAllocItems; ++k) acc += quantised<R>(v[k], rmax);
+    for (int k = 0; k < IT; ++k) acc += quantised<R>(v[k], rmax);
   }
   uint64_t incl;
   uint64_t tot = block_scan_incl(acc, &incl);
@@ -413,36 +515,35 @@ __device__ __forceinline__ uint64_t div_small(uint64_t t, uint64_t S, uint64_t m
 // cell of packet 32 w (each cell writes the multiples of 32 in its packet
 // range, so a warp of 32 consecutive packets finds its first cell with one
 // load) and the packets per super-tile (the capacity of its march-queue bucket).
-template <class R>
+template <class R, int IT>
 __device__ __forceinline__ void alloc_prefix_block(const R* emis, int64_t n3, uint64_t n_packets, uint64_t S,
                                                    uint64_t u, R rmax, uint64_t pre_block, int64_t c0, uint32_t* P,
                                                    uint32_t* first, const Tiles& tl, uint32_t bk0,
                                                    unsigned long long* bcap) {
-  uint64_t Q[kAllocItems];
+  uint64_t Q[IT];
   uint64_t acc = 0;
   {
-    R v[kAllocItems];
-    load_items<R>(emis, c0, n3, v);
+    R v[IT];
+    load_items<R, IT>(emis, c0, n3, v);
 #pragma unroll
-    for (int k = 0; k < kAllocItems; ++k) {
+    for (int k = 0; k < IT; ++k) {
       Q[k] = (rmax > (R)0 && c0 + k < n3) ? quantised<R>(v[k], rmax) : 0;
       acc += Q[k];
     }
   }
   uint64_t incl;
   block_scan_incl(acc, &incl);
-  if (c0 >= n3) return;
-  uint32_t out[kAllocItems];
+  uint32_t out[IT];
+  uint32_t bk = 0xffffffffu, bcount = 0;  // packets of the thread's last super-tile
   if (S == 0) {
 #pragma unroll
-    for (int k = 0; k < kAllocItems; ++k) out[k] = 0u;
+    for (int k = 0; k < IT; ++k) out[k] = 0u;
   } else {
     uint64_t rem;
     uint32_t pk = sys_floor(n_packets, pre_block + incl - acc, u, S, &rem);
-    uint32_t bk = 0xffffffffu, bcount = 0;
     const uint64_t minv = ~0ull / S;
 #pragma unroll
-    for (int k = 0; k < kAllocItems; ++k) {
+    for (int k = 0; k < IT; ++k) {
       out[k] = pk;
       const uint64_t t = rem + n_packets * Q[k];  // < S + 2^63 <= 2^64
       const uint64_t dq = div_small(t, S, minv, &rem);
@@ -459,25 +560,29 @@ __device__ __forceinline__ void alloc_prefix_block(const R* emis, int64_t n3, ui
       }
       pk = p1;
     }
-    if (bcount) atomicAdd(&bcap[bk], (unsigned long long)bcount);
   }
-  if (c0 + kAllocItems <= n3 && (reinterpret_cast<uintptr_t>(P + c0) & 15u) == 0) {
+  // the lanes of a warp are mostly in one super-tile: one addition per warp and super-tile
+  const unsigned same = __match_any_sync(0xffffffffu, bk);
+  const uint32_t sum = __reduce_add_sync(same, bcount);
+  if (sum && (int)(threadIdx.x & 31) == __ffs(same) - 1) atomicAdd(&bcap[bk], (unsigned long long)sum);
+  if (c0 >= n3) return;
+  if (IT >= 4 && c0 + IT <= n3 && (reinterpret_cast<uintptr_t>(P + c0) & 15u) == 0) {
     uint4* q = reinterpret_cast<uint4*>(P + c0);
 #pragma unroll
-    for (int k = 0; k < kAllocItems / 4; ++k) q[k] = make_uint4(out[4 * k], out[4 * k + 1], out[4 * k + 2], out[4 * k + 3]);
+    for (int k = 0; k < IT / 4; ++k) q[k] = make_uint4(out[4 * k], out[4 * k + 1], out[4 * k + 2], out[4 * k + 3]);
   } else {
 #pragma unroll
-    for (int k = 0; k < kAllocItems; ++k)
+    for (int k = 0; k < IT; ++k)
       if (c0 + k < n3) P[c0 + k] = out[k];
   }
 }
 
-template <class R>
+template <class R, int IT>
 __global__ void __launch_bounds__(AT) k_alloc_prefix(const R* emis, int64_t n3, uint64_t n_packets, DevScalars* sc,
                                                      const unsigned long long* partQ, uint32_t* P, uint32_t* first,
                                                      Tiles tl, unsigned long long* bcap) {
-  const int64_t c0 = (int64_t)blockIdx.x * kAllocChunk + (int64_t)threadIdx.x * kAllocItems;
-  alloc_prefix_block<R>(emis, n3, n_packets, sc->sumQ, sc->alloc_u, (R)sc->rmax, partQ[blockIdx.x], c0, P, first, tl,
+  const int64_t c0 = (int64_t)blockIdx.x * (AT * IT) + (int64_t)threadIdx.x * IT;
+  alloc_prefix_block<R, IT>(emis, n3, n_packets, sc->sumQ, sc->alloc_u, (R)sc->rmax, partQ[blockIdx.x], c0, P, first, tl,
                         0u, bcap);
 }
 
@@ -584,6 +689,10 @@ struct TransportArgs {
   uint64_t rq_part;                // entries one part holds
   uint32_t halo;                   // region of a bucket: its super-tile and halo cells around it; 0: no limit
   int resumed;                     // the queue holds full states of an earlier sweep (3 vectors per entry)
+  // compact velocity copy (rec_velq.cuh) and its index masks
+  const uint32_t* velq;
+  VelqMasks vm;
+  uint32_t vbx;
 };
 
 // Loads of the packet prefix and coarse index: the read-only path, or through
@@ -1134,76 +1243,201 @@ __global__ void __launch_bounds__(TT, emit_occupancy<R>()) k_emit(TransportArgs<
 // the warps advance through the super-tile buckets together and the cells
 // they touch stay close in memory; each warp refills its idle lanes from its
 // current chunk, so that lanes stay busy whatever the spread of path lengths.
-// Cells a lane marches per round between two votes of its warp.  The walk of
-// the traversal does not depend on the velocities, so a round first steps the
-// traversal through its cells and gathers their velocities together, then runs
-// the resonance tests in order: the lane waits on memory once per round rather
-// than once per cell.  The arithmetic of every cell is the same as one cell at
-// a time; only the order of the loads changes.
-#ifndef REC_MARCH_AHEAD
-#define REC_MARCH_AHEAD 4
-#endif
-template <class R> struct MarchAhead { static constexpr int value = sizeof(R) == 4 ? REC_MARCH_AHEAD : 2; };
+//
+// A lane walks kMarchAhead cells per round.  For every cell it asks the bound of
+// rec_velq.cuh, one 32-bit word of the compact velocity copy and one integer dot
+// product, whether the packet can be absorbed there at all; a cell whose
+// threshold exceeds any possible dot product is not even loaded.  A lane with
+// a candidate cell parks.  Once `refill` lanes of a warp are parked or idle, the
+// parked ones read the exact velocity of their candidate and take the exact
+// resonance test (tally and done, or on to the rest of the round), and the idle
+// ones take new packets, so that both run with many lanes at once.
+constexpr int kMarchAhead = 4;
 
 // Resident blocks per SM of the march (register budget per thread; a batch
 // keeps the box of each lane's packet in registers).
 template <class R, bool MB, bool RS = false> constexpr int march_occupancy() {
-  return RS ? (sizeof(R) == 4 ? 3 : 2)
-            : (MB ? 3 : (sizeof(R) == 4 ? (MarchAhead<R>::value > 4 ? 3 : MarchAhead<R>::value > 2 ? 4 : 5) : 3));
+  return RS ? (sizeof(R) == 4 ? 3 : 2) : (MB ? 3 : (sizeof(R) == 4 ? 4 : 3));
+}
+
+// The exit distance in binary32 for the bound: binary64 truncates toward zero
+// (its bits moved, 2^-23 relative).  Every exit distance is a normal binary32
+// number: at least 2^-53 (offset in the cell times tDelta >= 1), at most sqrt(3) per
+// crossing (one direction cosine is at least 1/sqrt(3)) times the crossing cap.
+__device__ __forceinline__ float bound_exit(float s) { return s; }
+__device__ __forceinline__ float bound_exit(double s) {
+  return __uint_as_float(__funnelshift_l((uint32_t)__double2loint(s), (uint32_t)__double2hiint(s), 3) + 0x40000000u);
+}
+
+// Word of a cell whose threshold some dot product may reach; predicated, not
+// branched around.
+__device__ __forceinline__ void load_word(uint32_t& w, const uint32_t* q, uint32_t cell, int thr, int top) {
+  asm("{\n\t.reg .pred p;\n\t.reg .u64 a;\n\t"
+      "setp.le.s32 p, %3, %4;\n\t"
+      "mad.wide.u32 a, %2, 4, %1;\n\t"
+      "@p ld.global.nc.u32 %0, [a];\n\t}"
+      : "+r"(w)
+      : "l"(q), "r"(cell), "r"(thr), "r"(top));
+}
+
+// One cell of the walk: returns the exit distance (the nearest face, ties
+// broken x < y < z) and steps across that face: its next distance, and its part
+// of the word index (an addition with a mask, which wraps power-of-two sides).
+// The three axes are predicated instructions, written out: as selects they
+// cost twice as many, and the march is bound by instruction issue.
+__device__ __forceinline__ float walk_step(float& tMx, float& tMy, float& tMz, float tDx, float tDy, float tDz,
+                                           uint32_t& X, uint32_t& Y, uint32_t& Z, uint32_t Sx, uint32_t Sy,
+                                           uint32_t Sz, uint32_t mx, uint32_t my, uint32_t mz) {
+  float s;
+  asm("{\n\t.reg .pred px, py, pz;\n\t"
+      "min.f32 %0, %1, %2, %3;\n\t"
+      "setp.eq.f32 px, %1, %0;\n\t"
+      "setp.eq.and.f32 py|pz, %2, %0, !px;\n\t"
+      "@px add.rn.f32 %1, %1, %7;\n\t"
+      "@py add.rn.f32 %2, %2, %8;\n\t"
+      "@pz add.rn.f32 %3, %3, %9;\n\t"
+      "@px add.u32 %4, %4, %10;\n\t"
+      "@py add.u32 %5, %5, %11;\n\t"
+      "@pz add.u32 %6, %6, %12;\n\t"
+      "@px and.b32 %4, %4, %13;\n\t"
+      "@py and.b32 %5, %5, %14;\n\t"
+      "@pz and.b32 %6, %6, %15;\n\t}"
+      : "=&f"(s), "+f"(tMx), "+f"(tMy), "+f"(tMz), "+r"(X), "+r"(Y), "+r"(Z)
+      : "f"(tDx), "f"(tDy), "f"(tDz), "r"(Sx), "r"(Sy), "r"(Sz), "r"(mx), "r"(my), "r"(mz));
+  return s;
+}
+// Binary64: face distances are positive or +inf, so their bits order as
+// integers and no comparison goes to the slow binary64 pipe; the addition is the
+// walk's only binary64 operation.
+__device__ __forceinline__ double walk_step(double& tMx, double& tMy, double& tMz, double tDx, double tDy, double tDz,
+                                            uint32_t& X, uint32_t& Y, uint32_t& Z, uint32_t Sx, uint32_t Sy,
+                                            uint32_t Sz, uint32_t mx, uint32_t my, uint32_t mz) {
+  const long long a = __double_as_longlong(tMx), b = __double_as_longlong(tMy), c = __double_as_longlong(tMz);
+  const bool px = a <= b && a <= c, py = !px && b <= c, pz = !px && !py;
+  const double s = __longlong_as_double(px ? a : (py ? b : c));
+  const double t = __dadd_rn(s, px ? tDx : (py ? tDy : tDz));
+  if (px) { tMx = t; X = (X + Sx) & mx; }
+  if (py) { tMy = t; Y = (Y + Sy) & my; }
+  if (pz) { tMz = t; Z = (Z + Sz) & mz; }
+  return s;
+}
+// Sides that are no power of two: the last cell in the direction of travel
+// (end) steps to the first one (last ^ end, since one of the two is offset 0),
+// set up beforehand as an addition, since the mask would not wrap there.
+template <class R>
+__device__ __forceinline__ R walk_step_any(R& tMx, R& tMy, R& tMz, R tDx, R tDy, R tDz, uint32_t& X, uint32_t& Y,
+                                           uint32_t& Z, uint32_t Sx, uint32_t Sy, uint32_t Sz, uint32_t mx,
+                                           uint32_t my, uint32_t mz, uint32_t Ex, uint32_t Ey, uint32_t Ez,
+                                           uint32_t lx, uint32_t ly, uint32_t lz) {
+  const uint32_t x0 = X, y0 = Y, z0 = Z;
+  const R s = walk_step(tMx, tMy, tMz, tDx, tDy, tDz, X, Y, Z, Sx, Sy, Sz, mx, my, mz);
+  // one axis moved; from its end the masked step left a wrong offset
+  if (X != x0 && x0 == Ex) X = lx ^ Ex;
+  if (Y != y0 && y0 == Ey) Y = ly ^ Ey;
+  if (Z != z0 && z0 == Ez) Z = lz ^ Ez;
+  return s;
 }
 
 __device__ __forceinline__ void transport_end_batch(const BoxDev* bxs, int B, const unsigned long long* bfill,
                                                     rec_stats* st);
 
-// P2: the box side is a power of two (cell index by shifts and masks).
+// P2: the box side is a power of two (periodic wrap by masks).
 // MB: batched context; the lanes of a warp may hold packets of different boxes.
 template <class R, bool P2, bool MB, bool RS = false>
 __global__ void __launch_bounds__(TT, (march_occupancy<R, MB, RS>())) k_march(TransportArgs<R> a, const BoxDev* bxs,
                                                                               int B, const BoxStep* bst,
                                                                               rec_stats* st) {
   static_assert(!RS || (P2 && !MB), "region sweeps: single box of power-of-two side");
+  static_assert(!MB || !P2, "a batch mixes sides");
   using V = typename Vec4<R>::T;
+  constexpr int kA = kMarchAhead;
   const int lane = threadIdx.x & 31;
   const uint32_t n = (uint32_t)a.n;
-  const uint32_t lg = P2 ? (uint32_t)(__ffs((int)n) - 1) : 0u;
-  // region sweeps: bucket of the open chunk and of the lane's packet (its
-  // super-tile), 0xffffffff for a packet that marches without a limit
-  uint32_t cbk = 0, lbk = 0;
-  bool rqp = false;  // the lane's packet leaves its region: queue it again
+  // region sweeps: bucket of the open chunk (its super-tile); path length at
+  // which the lane's packet leaves the region around it (+inf: no limit)
+  uint32_t cbk = 0;
+  float leave = 0.0f;
   __shared__ BoxCounters cnt;
   if (MB) box_counters_clear(cnt, B);
-  // box of the lane's packet (batch) and of the open chunk
-  const V* lvel = a.vel;
-  uint32_t* ltally = a.tally;
-  uint32_t ln = n;
-  R lkappa = a.kappa;
+  // box of the lane's packet and of the open chunk
   int lbox = -1, cbox = 0;
-  const V* cvel = a.vel;
-  uint32_t* ctally = a.tally;
-  uint32_t cn = n;
-  R ckappa = a.kappa;
+  const uint32_t* q = a.velq;
+  VelqMasks lm = a.vm;
+  uint32_t bx = a.vbx, ln = n;
+  uint32_t lastx = 0, lasty = 0, lastz = 0;
+  R lkappa = a.kappa;
+  VelqBox vb;
+  if (!MB) {
+    vb = velq_box(a.velq ? a.sc->vq_u : 0.0f, a.sc->vq_v, (float)a.kappa);
+    lastx = velq_x(n - 1u); lasty = velq_y(n - 1u, bx); lastz = velq_z(n - 1u, bx);
+  }
   const uint64_t n_chunks = a.cpre[a.nb];
-  uint64_t chunk = 0;
-  uint64_t pos = 0, end = 0;  // queue slots [pos, end) left in the current chunk
-  bool have = false;          // a chunk is open
+  uint64_t pos = 0, end = 0;  // queue slots [pos, end) left in the open chunk
   bool more = n_chunks > 0;
-  bool active = false;
-  uint32_t cell = 0;
-  Ray<R> r;
-  r.kc = 0;
-  V Uc;
+  bool active = false, parked = false;
+  // the packet: cell (three parts of the word index), face distances, steps, resonance
+  uint32_t X = 0, Y = 0, Z = 0, Sx = 0, Sy = 0, Sz = 0, Ex = 0, Ey = 0, Ez = 0, kc = 0;
+  R tMx = 0, tMy = 0, tMz = 0, tDx = 0, tDy = 0, tDz = 0, knx = 0, kny = 0, knz = 0, u0 = 0;
+  VelqPacket vp;
+  vp.m = 0; vp.c1 = vp.c2 = 0.0f; vp.top = 0;
+  // the last round: cells, exit distances, words, first cell not yet cleared
+  uint32_t cl[kA] = {}, qw[kA] = {}, kfrom = 0;
+  R se[kA] = {};
   uint64_t my_abs = 0, my_cap = 0, my_cross = 0;
   for (;;) {
-    unsigned idle = __ballot_sync(0xffffffffu, !active);
-    if (more && __popc(idle) >= a.refill) {
+    const unsigned stop = __ballot_sync(0xffffffffu, !active || parked);
+    bool fresh = false;  // region sweeps: a round was completed, check the region
+    if (__popc(stop) >= a.refill || stop == 0xffffffffu) {
+      // exact test of the parked lanes' first candidate cell
+      if (parked) {
+        uint32_t cand = 0;
+#pragma unroll
+        for (int k = 0; k < kA; ++k) {
+          const int thr = __float_as_int(fmaf(-bound_exit(se[k]), vp.c1, vp.c2));
+          if (velq_dot(qw[k], vp.m, kVelqBiasBits) >= thr || kc - (uint32_t)(kA - k) >= kMaxCrossings) cand |= 1u << k;
+        }
+        cand &= 0xffffffffu << kfrom;
+        if (cand == 0) {
+          parked = false;
+          fresh = true;
+        } else {
+          const uint32_t k = (uint32_t)__ffs((int)cand) - 1u;
+          uint32_t c = cl[0];
+          R s = se[0];
+#pragma unroll
+          for (int i = 1; i < kA; ++i)
+            if (k == (uint32_t)i) { c = cl[i]; s = se[i]; }
+          uint32_t ix, iy, iz;
+          velq_coords(c, bx, &ix, &iy, &iz);
+          const uint32_t lin = (iz * ln + iy) * ln + ix;
+          const V* vel = MB ? (const V*)bxs[lbox].vel4 : a.vel;
+          const V U = vel[lin];
+          Ray<R> r;
+          r.knx = knx; r.kny = kny; r.knz = knz;
+          // resonance in the cell at path length u0 - kappa n.U: absorb unless beyond its exit
+          const uint32_t kcell = kc - (uint32_t)kA + k;  // crossings before this cell
+          const bool hit = Ar<R>::sub(u0, doppler(r, U)) <= s;
+          if (hit || kcell >= kMaxCrossings) {
+            active = parked = false;
+            my_cross += kcell - 1;  // crossings up to this cell; the first was counted at emission
+            if (hit) { atomicAdd((MB ? bxs[lbox].tally : a.tally) + lin, 1u); ++my_abs; }
+            else ++my_cap;
+          } else {
+            kfrom = k + 1u;
+            parked = (cand >> kfrom) != 0u;
+            fresh = !parked;
+          }
+        }
+      }
       // refill idle lanes in lane order from the warp's chunks
+      unsigned idle = __ballot_sync(0xffffffffu, !active);
       while (idle && more) {
-        if (!have || pos >= end) {
+        if (pos >= end) {
           // next chunk in queue order, shared by all warps: the warps in flight
           // stay on neighbouring chunks, so their rays start close together
           unsigned long long nc = 0;
           if (lane == 0) nc = atomicAdd(&a.sc->march_next, 1ull);
-          chunk = __shfl_sync(0xffffffffu, nc, 0);
+          const uint64_t chunk = __shfl_sync(0xffffffffu, nc, 0);
           if (chunk >= n_chunks) { more = false; break; }
           // bucket of this chunk: last b with cpre[b] <= chunk (uniform over the warp)
           uint32_t lo = 0, hi = (uint32_t)a.nb;
@@ -1215,137 +1449,126 @@ __global__ void __launch_bounds__(TT, (march_occupancy<R, MB, RS>())) k_march(Tr
           const uint64_t k0 = (chunk - __ldg(a.cpre + lo)) * a.chunk;
           pos = a.boff[lo] + k0;
           end = pos + min((uint64_t)a.chunk, (uint64_t)(a.bfill[lo] - k0));
-          have = true;
           if (RS) cbk = lo;
-          if (MB) {  // box of this bucket: last b with bk0 <= lo
-            cbox = last_le(B, lo, [&](int i) { return bxs[i].bk0; });
-            cvel = (const V*)bxs[cbox].vel4;
-            ctally = bxs[cbox].tally;
-            cn = bxs[cbox].n;
-            ckappa = (R)bst[cbox].kappa;
-          }
+          if (MB) cbox = last_le(B, lo, [&](int i) { return bxs[i].bk0; });  // last b with bk0 <= lo
         }
         const uint32_t take = (uint32_t)min((uint64_t)__popc(idle), end - pos);
         const uint32_t rank = __popc(idle & ((1u << lane) - 1u));
         if (((idle >> lane) & 1u) && rank < take) {
           const uint64_t slot = pos + rank;
           constexpr int QV = QueueVecs<R>::value;
-          if (RS) lbk = cbk;
-          if (RS && a.resumed) {
-            // a full state queued again by an earlier sweep
-            const V q0v = a.queue[3 * slot], q1v = a.queue[3 * slot + 1], q2v = a.queue[3 * slot + 2];
-            cell = to_bits<R>(q0v.x);
-            r.ix = cell & (n - 1u); r.iy = (cell >> lg) & (n - 1u); r.iz = cell >> (2u * lg);
-            r.tMx = q0v.y; r.tMy = q0v.z; r.tMz = q0v.w;
-            r.sx = q1v.x < (R)0 ? -1 : 1; r.tDx = fabs(q1v.x);
-            r.sy = q1v.y < (R)0 ? -1 : 1; r.tDy = fabs(q1v.y);
-            r.sz = q1v.z < (R)0 ? -1 : 1; r.tDz = fabs(q1v.z);
-            r.u0 = q1v.w;
-            r.knx = q2v.x; r.kny = q2v.y; r.knz = q2v.z;
-            r.kc = to_bits<R>(q2v.w);
-            Uc = lvel[cell];
-            active = true;
-          } else {
-          const V q0v = a.queue[QV * slot], q1v = a.queue[QV * slot + 1];
           if (MB) {
             if (lbox != cbox) {  // counters of the previous box to shared memory
               if (lbox >= 0) box_counters_add(cnt, lbox, my_abs, my_cap, my_cross);
               my_abs = my_cap = my_cross = 0;
               lbox = cbox;
+              const BoxDev& d = bxs[lbox];
+              ln = d.n;
+              bx = d.vbx;
+              lm = velq_masks(ln, bx, false);
+              q = d.velq;
+              lkappa = (R)bst[lbox].kappa;
+              lastx = velq_x(ln - 1u); lasty = velq_y(ln - 1u, bx); lastz = velq_z(ln - 1u, bx);
+              vb = velq_box(q ? d.sc->vq_u : 0.0f, d.sc->vq_v, (float)lkappa);
             }
-            lvel = cvel;
-            ltally = ctally;
-            ln = cn;
-            lkappa = ckappa;
           }
-          cell = to_bits<R>(q0v.x);
-          if (P2) {
-            r.ix = cell & (n - 1u); r.iy = (cell >> lg) & (n - 1u); r.iz = cell >> (2u * lg);
-          } else if (MB) {
-            r.ix = cell % ln; r.iy = (cell / ln) % ln; r.iz = cell / (ln * ln);
+          uint32_t cell;
+          int sx, sy, sz;
+          if (RS && a.resumed) {
+            // a full state queued again by an earlier sweep
+            const V q0v = a.queue[3 * slot], q1v = a.queue[3 * slot + 1], q2v = a.queue[3 * slot + 2];
+            cell = to_bits<R>(q0v.x);
+            tMx = q0v.y; tMy = q0v.z; tMz = q0v.w;
+            sx = q1v.x < (R)0 ? -1 : 1; tDx = fabs(q1v.x);
+            sy = q1v.y < (R)0 ? -1 : 1; tDy = fabs(q1v.y);
+            sz = q1v.z < (R)0 ? -1 : 1; tDz = fabs(q1v.z);
+            u0 = q1v.w;
+            knx = q2v.x; kny = q2v.y; knz = q2v.z;
+            kc = to_bits<R>(q2v.w);
           } else {
-            a.tl.template coords<false>(cell, &r.ix, &r.iy, &r.iz);
+            const V q0v = a.queue[QV * slot], q1v = a.queue[QV * slot + 1];
+            cell = to_bits<R>(q0v.x);
+            tMx = q0v.y; tMy = q0v.z; tMz = q0v.w;
+            u0 = q1v.w;
+            if (QV == 2) {  // tDelta and kappa n exactly as the emission formed them
+              axis_setup<R>(q1v.x, &tDx, &sx);
+              axis_setup<R>(q1v.y, &tDy, &sy);
+              axis_setup<R>(q1v.z, &tDz, &sz);
+              knx = Ar<R>::mul(lkappa, q1v.x); kny = Ar<R>::mul(lkappa, q1v.y); knz = Ar<R>::mul(lkappa, q1v.z);
+            } else {
+              const V q2v = a.queue[QV * slot + 2];
+              sx = q1v.x < (R)0 ? -1 : 1; tDx = fabs(q1v.x);
+              sy = q1v.y < (R)0 ? -1 : 1; tDy = fabs(q1v.y);
+              sz = q1v.z < (R)0 ? -1 : 1; tDz = fabs(q1v.z);
+              knx = q2v.x; kny = q2v.y; knz = q2v.z;
+            }
+            kc = 1;  // the step out of the home cell
           }
-          r.tMx = q0v.y; r.tMy = q0v.z; r.tMz = q0v.w;
-          r.u0 = q1v.w;
-          if (QV == 2) {  // tDelta and kappa n exactly as the emission formed them
-            axis_setup<R>(q1v.x, &r.tDx, &r.sx);
-            axis_setup<R>(q1v.y, &r.tDy, &r.sy);
-            axis_setup<R>(q1v.z, &r.tDz, &r.sz);
-            r.knx = Ar<R>::mul(lkappa, q1v.x); r.kny = Ar<R>::mul(lkappa, q1v.y); r.knz = Ar<R>::mul(lkappa, q1v.z);
+          uint32_t ix, iy, iz;
+          if (MB) {
+            const BoxDev& d = bxs[lbox];
+            Tiles{d.n, d.nt, d.lg, d.mn, d.mn2, d.tlg}.template coords<false>(cell, &ix, &iy, &iz);
           } else {
-            const V q2v = a.queue[QV * slot + 2];
-            r.sx = q1v.x < (R)0 ? -1 : 1; r.tDx = fabs(q1v.x);
-            r.sy = q1v.y < (R)0 ? -1 : 1; r.tDy = fabs(q1v.y);
-            r.sz = q1v.z < (R)0 ? -1 : 1; r.tDz = fabs(q1v.z);
-            r.knx = q2v.x; r.kny = q2v.y; r.knz = q2v.z;
+            a.tl.template coords<P2>(cell, &ix, &iy, &iz);
           }
-          r.kc = 1;  // the step out of the home cell
-          Uc = lvel[cell];
+          X = velq_x(ix); Y = velq_y(iy, bx); Z = velq_z(iz, bx);
+          if (RS) {
+            // the region: the bucket's super-tile widened by the halo (periodic:
+            // offsets from its low corner modulo n).  Along an axis the packet leaves
+            // after the cells that are left of it in the direction of travel.
+            leave = __int_as_float(0x7f800000);
+            if (a.halo) {
+              const uint32_t tlg = a.tl.tlg, ntl = a.tl.lg - tlg, ntm = (1u << ntl) - 1u, m = n - 1u;
+              const uint32_t far = (1u << tlg) + 2u * a.halo - 1u;
+              const uint32_t rx = (ix - (((cbk & ntm) << tlg) - a.halo)) & m;
+              const uint32_t ry = (iy - ((((cbk >> ntl) & ntm) << tlg) - a.halo)) & m;
+              const uint32_t rz = (iz - (((cbk >> (2u * ntl)) << tlg) - a.halo)) & m;
+              leave = fminf(leave, (float)tMx + (float)(sx > 0 ? far - rx : rx) * (float)tDx);
+              leave = fminf(leave, (float)tMy + (float)(sy > 0 ? far - ry : ry) * (float)tDy);
+              leave = fminf(leave, (float)tMz + (float)(sz > 0 ? far - rz : rz) * (float)tDz);
+            }
+          }
+          Sx = sx > 0 ? 0u - lm.x : 0u - 1u;
+          Sy = sy > 0 ? 0u - lm.y : 0u - 2u;
+          Sz = sz > 0 ? 0u - lm.z : 0u - 4u;
+          if (!P2) { Ex = sx > 0 ? lastx : 0u; Ey = sy > 0 ? lasty : 0u; Ez = sz > 0 ? lastz : 0u; }
+          vp = velq_packet(vb, (float)knx, (float)kny, (float)knz, (float)u0);
           active = true;
-          }
         }
-        // lanes taken this round leave the idle set (the lowest `take` idle lanes)
-        unsigned taken = 0, m = idle;
-        for (uint32_t t = 0; t < take; ++t) { unsigned bb = m & (0u - m); taken |= bb; m ^= bb; }
-        idle &= ~taken;
         pos += take;
+        idle = __ballot_sync(0xffffffffu, !active);
       }
     }
     if (!__any_sync(0xffffffffu, active)) break;  // no packet left in the warp
-    if (active) {
-      // one round of kA cells: cell 0 is the current one (velocity in Uc); the
-      // walk records each cell's exit distance and gathers the velocity of the
-      // cell after it, then the cells are tested in order
-      constexpr int kA = MarchAhead<R>::value;
-      R se[kA];
-      V Un[kA];
-      uint32_t cl[kA + 1];
-      cl[0] = cell;
-      const uint32_t kc0 = r.kc;
+    if (active && !parked && !(RS && fresh)) {
+      // one round: walk kA cells, loading the words that matter, then ask the bound
 #pragma unroll
       for (int k = 0; k < kA; ++k) {
-        bool ax0, ax1, ax2;
-        se[k] = dda_exit(r, &ax0, &ax1, &ax2);
-        dda_advance<R, P2>(r, ax0, ax1, ax2, se[k], ln);
-        cl[k + 1] = P2 ? (((r.iz << lg) | r.iy) << lg) | r.ix : (r.iz * ln + r.iy) * ln + r.ix;
-        Un[k] = lvel[cl[k + 1]];
+        cl[k] = X | Y | Z;
+        if (P2)
+          se[k] = walk_step(tMx, tMy, tMz, tDx, tDy, tDz, X, Y, Z, Sx, Sy, Sz, lm.x, lm.y, lm.z);
+        else
+          se[k] = walk_step_any(tMx, tMy, tMz, tDx, tDy, tDz, X, Y, Z, Sx, Sy, Sz, lm.x, lm.y, lm.z, Ex, Ey, Ez, lastx,
+                                lasty, lastz);
+        load_word(qw[k], q, cl[k], __float_as_int(fmaf(-bound_exit(se[k]), vp.c1, vp.c2)), vp.top);
       }
-      int res = 0;
-      uint32_t kend = 0, cend = 0;
+      kc += kA;
+      kfrom = 0;
+      parked = kc > kMaxCrossings;
 #pragma unroll
-      for (int k = 0; k < kA; ++k) {
-        const R dc = doppler(r, k == 0 ? Uc : Un[k - 1]);
-        if (res == 0) {
-          // resonance in cell k at path length u0 - kappa n.U: absorb unless beyond its exit
-          if (Ar<R>::sub(r.u0, dc) <= se[k]) { res = 1; kend = (uint32_t)k; cend = cl[k]; }
-          else if (kc0 + (uint32_t)k >= kMaxCrossings) { res = 2; kend = (uint32_t)k; }
-        }
-      }
-      if (res == 0) {
-        cell = cl[kA];
-        Uc = Un[kA - 1];
-        if (RS && a.halo && lbk != 0xffffffffu) {
-          // still inside the super-tile of its bucket widened by the halo?
-          // (periodic: offsets from the region's low corner modulo n)
-          const uint32_t tlg = a.tl.tlg, ntl = lg - tlg, ntm = (1u << ntl) - 1u, m = n - 1u;
-          const uint32_t span = (1u << tlg) + 2u * a.halo;
-          const uint32_t ox = (((lbk & ntm) << tlg) - a.halo) & m;
-          const uint32_t oy = ((((lbk >> ntl) & ntm) << tlg) - a.halo) & m;
-          const uint32_t oz = (((lbk >> (2u * ntl)) << tlg) - a.halo) & m;
-          if (((r.ix - ox) & m) >= span || ((r.iy - oy) & m) >= span || ((r.iz - oz) & m) >= span) {
-            rqp = true;
-            active = false;
-          }
-        }
-      } else {
-        active = false;
-        my_cross += kc0 + kend - 1;  // crossings up to the last cell; the first was counted at emission
-        if (res == 1) { atomicAdd(ltally + cend, 1u); ++my_abs; }
-        else ++my_cap;
-      }
+      for (int k = 0; k < kA; ++k)
+        parked |= velq_dot(qw[k], vp.m, kVelqBiasBits) >= __float_as_int(fmaf(-bound_exit(se[k]), vp.c1, vp.c2));
+      fresh = !parked;
     }
     if (RS) {
+      bool rqp = false;  // the lane's packet left its region: queue it again
+      uint32_t cell = 0;
+      if (fresh && bound_exit(se[kA - 1]) >= leave) {
+        rqp = true;
+        uint32_t ix, iy, iz;
+        velq_coords(X | Y | Z, bx, &ix, &iy, &iz);
+        cell = (((iz << a.tl.lg) | iy) << a.tl.lg) | ix;
+      }
       // packets that left their region: appended to the second queue as full
       // states (the current cell is the next to test), counted in the bucket
       // of the super-tile they have reached
@@ -1362,24 +1585,20 @@ __global__ void __launch_bounds__(TT, (march_occupancy<R, MB, RS>())) k_march(Tr
         const uint64_t slot = (uint64_t)part * a.rq_part + k;
         if (stored) {
           V q0v, q1v, q2v;
-          q0v.x = bits_to<R>(cell); q0v.y = r.tMx; q0v.z = r.tMy; q0v.w = r.tMz;
-          q1v.x = r.sx < 0 ? -r.tDx : r.tDx; q1v.y = r.sy < 0 ? -r.tDy : r.tDy; q1v.z = r.sz < 0 ? -r.tDz : r.tDz;
-          q1v.w = r.u0;
-          q2v.x = r.knx; q2v.y = r.kny; q2v.z = r.knz; q2v.w = bits_to<R>(r.kc);
+          q0v.x = bits_to<R>(cell); q0v.y = tMx; q0v.z = tMy; q0v.w = tMz;
+          q1v.x = copysign(tDx, knx); q1v.y = copysign(tDy, kny); q1v.z = copysign(tDz, knz); q1v.w = u0;
+          q2v.x = knx; q2v.y = kny; q2v.z = knz; q2v.w = bits_to<R>(kc);
           a.rq[3 * slot] = q0v;
           a.rq[3 * slot + 1] = q1v;
           a.rq[3 * slot + 2] = q2v;
+          active = false;
         }
         const unsigned sm = __ballot_sync(0xffffffffu, stored);
         const uint32_t bk = stored ? a.tl.template at<true>(cell) : 0xffffffffu;
         const unsigned gm = __match_any_sync(0xffffffffu, bk) & sm;
         if (stored && lane == __ffs(gm) - 1) atomicAdd(&a.rcount[bk], (unsigned long long)__popc(gm));
-        if (rqp && !stored) {  // the second queue is full: this packet marches on without a limit
-          active = true;
-          lbk = 0xffffffffu;
-        }
+        if (rqp && !stored) leave = __int_as_float(0x7f800000);  // the second queue is full: march on without a limit
         if (__any_sync(0xffffffffu, rqp && !stored) && lane == 0) atomicOr(&a.sc->flags, 16);
-        rqp = false;
       }
     }
   }
@@ -1501,6 +1720,23 @@ __global__ void k_transport_end(DevScalars* sc, rec_stats* st) {
   }
 }
 
+// Consecutive cells per thread of the single-box allocation: few for small
+// boxes, whose time is one thread's serial chain (quotients, remainders) on a
+// part of the chip, many for large ones, where the passes stream and the
+// prefix's 128-bit division is shared.  Whole passes with 16 cells per thread
+// against the rule's: 32^3 FP64 step 250 / 217 us, 100^3 transport 326 / 318 us.
+int alloc_items(int64_t n3) { return n3 <= (1 << 17) ? 1 : (n3 <= (1 << 21) ? 4 : kAllocItems); }
+
+template <class R, int IT>
+void alloc_launch(rec_ctx* c, int blocks, const typename Vec4<R>::T* vel, const Stream& s, const Tiles& tl, int nb) {
+  const R* emis = (const R*)c->box.emis;
+  const uint64_t npk = c->box.n_packets;
+  k_alloc_sum<R, IT><<<blocks, AT, 0, c->stream>>>(emis, vel, c->n3, npk, s, c->sc, c->partQ, c->P, c->velq,
+                                                   velq_bits((uint32_t)c->box.n), tl);
+  cudaMemsetAsync(c->bcap, 0, sizeof(unsigned long long) * nb, c->stream);
+  k_alloc_prefix<R, IT><<<blocks, AT, 0, c->stream>>>(emis, c->n3, npk, c->sc, c->partQ, c->P, c->first, tl, c->bcap);
+}
+
 template <class R>
 cudaError_t run_transport(rec_ctx* c, int step, double z, rec_stats* st) {
   const rec_box& b = c->box;
@@ -1509,18 +1745,18 @@ cudaError_t run_transport(rec_ctx* c, int step, double z, rec_stats* st) {
   const rec_tuning& tu = c->tune;
   const Tiles tl = make_tiles(b.n, tu.tile);
   const int nb = (int)(tl.nt * tl.nt * tl.nt);
-  {
-    GroupTimer t(c, kTAlloc, 4);
-    k_alloc_max<R><<<c->grid, kPassThreads, 0, c->stream>>>((const R*)b.emis, c->n3, c->sc, c->part);
-    k_alloc_sum<R><<<c->alloc_blocks, AT, 0, c->stream>>>((const R*)b.emis, c->n3, b.n_packets, s, c->sc,
-                                                          c->partQ, c->P);
-    cudaMemsetAsync(c->bcap, 0, sizeof(unsigned long long) * nb, c->stream);
-    k_alloc_prefix<R><<<c->alloc_blocks, AT, 0, c->stream>>>((const R*)b.emis, c->n3, b.n_packets, c->sc,
-                                                             c->partQ, c->P, c->first, tl, c->bcap);
-    k_bucket_offsets<<<1, 1024, 0, c->stream>>>(c->bcap, c->bfill, nb);
-  }
   double kappa, cth;
   transport_scalars(c->cosmo, b.n, z, &kappa, &cth);
+  {
+    GroupTimer t(c, kTAlloc, 4);
+    const typename Vec4<R>::T* vel = (const typename Vec4<R>::T*)b.vel4;
+    k_alloc_max<R><<<c->grid, kPassThreads, 0, c->stream>>>((const R*)b.emis, vel, c->n3, (float)kappa, c->sc);
+    const int it = alloc_items(c->n3), ab = c->alloc_blocks;
+    if (it == 1) alloc_launch<R, 1>(c, ab, vel, s, tl, nb);
+    else if (it == 4) alloc_launch<R, 4>(c, ab, vel, s, tl, nb);
+    else alloc_launch<R, kAllocItems>(c, ab, vel, s, tl, nb);
+    k_bucket_offsets<<<1, 1024, 0, c->stream>>>(c->bcap, c->bfill, nb);
+  }
   TransportArgs<R> a;
   a.P = c->P;
   a.first = c->first;
@@ -1550,6 +1786,9 @@ cudaError_t run_transport(rec_ctx* c, int step, double z, rec_stats* st) {
   a.rq_part = 0;
   a.halo = 0;
   a.resumed = 0;
+  a.velq = c->velq;
+  a.vbx = velq_bits((uint32_t)b.n);
+  a.vm = velq_masks((uint32_t)b.n, a.vbx, p2);
   {
     GroupTimer t(c, kTEmit, 2);
     const int eb = c->sm_count * tu.emit_blocks_per_sm;
@@ -1596,6 +1835,11 @@ cudaError_t run_transport(rec_ctx* c, int step, double z, rec_stats* st) {
 
 // ---- batched contexts: every phase is one launch over all boxes ------------------
 
+// Transport scalars of every box, a kernel parameter.
+struct BoxStepArgs {
+  BoxStep s[kMaxBoxes];
+};
+
 // Allocation blocks: kAllocChunk cells of one box each; box of block g = last b
 // with ablk0 <= g.
 __device__ __forceinline__ int alloc_box(const BoxDev* bxs, int B, uint32_t g) {
@@ -1605,56 +1849,37 @@ __device__ __forceinline__ int alloc_box(const BoxDev* bxs, int B, uint32_t g) {
 // Allocation phases of a batch as functions of the allocation block g of ng
 // (blockIdx.x of a per-phase launch, or a virtual block of the persistent one).
 template <class R>
-__device__ __forceinline__ void alloc_max_batch(const BoxDev* bxs, int B, DevScalars* gsc, double* part, uint32_t g,
-                                                uint32_t ng) {
+__device__ __forceinline__ void alloc_max_batch(const BoxDev* bxs, const BoxStepArgs& bs, int B, DevScalars* gsc,
+                                                uint32_t g, uint32_t ng) {
+  using V = typename Vec4<R>::T;
   const int b = alloc_box(bxs, B, g);
   const BoxDev& d = bxs[b];
   const int64_t c0 = (int64_t)(g - d.ablk0) * kAllocChunk + (int64_t)threadIdx.x * kAllocItems;
   R v[kAllocItems];
-  load_items<R>((const R*)d.emis, c0, d.n3, v);
+  load_items<R, kAllocItems>((const R*)d.emis, c0, d.n3, v);
   R m = (R)0;
-  int bad = 0;
+  bool bad = false;
 #pragma unroll
   for (int k = 0; k < kAllocItems; ++k) {
     if (c0 + k >= d.n3) continue;
     const R r = v[k];
-    if (!(r >= (R)0) || isinf(r)) bad = 1;
-    else m = fmax(m, r);
+    if (!(r >= (R)0) || isinf(r)) bad = true;
+    else m = m < r ? r : m;
   }
-  bad = __syncthreads_or(bad);
-  double bm = block_max<AT>((double)m);
-  if (threadIdx.x == 0) {
-    part[(size_t)g * kMaxSums + 0] = bm;
-    part[(size_t)g * kMaxSums + 1] = bad ? 1.0 : 0.0;
+  VelMax vm;
+  for (int k = 0; k < kAllocItems; ++k) {
+    const int64_t i = (int64_t)(g - d.ablk0) * kAllocChunk + (int64_t)k * AT + threadIdx.x;
+    if (i < d.n3) vm.add(((const V*)d.vel4)[i]);
   }
+  block_maxima<AT>(d.sc, order_bits(m), vm, bad);
   if (!last_block_done(&gsc->counter, ng)) return;
-  // one warp per box: maximum over the box's blocks
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int i = warp; i < B; i += AT / 32) {
-    const uint32_t g0 = bxs[i].ablk0;
-    const uint32_t g1 = (i + 1 < B) ? bxs[i + 1].ablk0 : ng;
-    double mx = 0.0, anybad = 0.0;
-    for (uint32_t g = g0 + lane; g < g1; g += 32) {
-      mx = fmax(mx, __ldcg(part + (size_t)g * kMaxSums));
-      anybad = fmax(anybad, __ldcg(part + (size_t)g * kMaxSums + 1));
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-      anybad = fmax(anybad, __shfl_xor_sync(0xffffffffu, anybad, o));
-    }
-    if (lane == 0) {
-      DevScalars* sc = bxs[i].sc;
-      sc->rmax = anybad > 0.0 ? 0.0 : mx;
-      sc->flags &= ~(2 | 4 | 16);
-      if (anybad > 0.0) sc->flags |= 4;
-    }
-  }
+  for (int i = threadIdx.x; i < B; i += AT) take_maxima<R>(bxs[i].sc, (float)(R)bs.s[i].kappa);
   if (threadIdx.x == 0) gsc->counter = 0;
 }
 template <class R>
-__global__ void __launch_bounds__(AT) k_alloc_max_batch(const BoxDev* bxs, int B, DevScalars* gsc, double* part) {
-  alloc_max_batch<R>(bxs, B, gsc, part, blockIdx.x, gridDim.x);
+__global__ void __launch_bounds__(AT) k_alloc_max_batch(const BoxDev* bxs, BoxStepArgs bs, int B,
+                                                        DevScalars* gsc) {
+  alloc_max_batch<R>(bxs, bs, B, gsc, blockIdx.x, gridDim.x);
 }
 
 template <class R>
@@ -1663,11 +1888,13 @@ __device__ __forceinline__ void alloc_sum_batch(const BoxDev* bxs, int B, uint32
   const int b = alloc_box(bxs, B, g);
   const BoxDev& d = bxs[b];
   const R rmax = (R)__ldcg(&d.sc->rmax);
+  velq_write<R, kAllocItems>((const typename Vec4<R>::T*)d.vel4, d.n3, (int64_t)(g - d.ablk0) * kAllocChunk, __ldcg(&d.sc->vq_u),
+                d.velq, d.vbx, Tiles{d.n, d.nt, d.lg, d.mn, d.mn2, d.tlg});
   uint64_t acc = 0;
   if (rmax > (R)0) {
     const int64_t c0 = (int64_t)(g - d.ablk0) * kAllocChunk + (int64_t)threadIdx.x * kAllocItems;
     R v[kAllocItems];
-    load_items<R>((const R*)d.emis, c0, d.n3, v);
+    load_items<R, kAllocItems>((const R*)d.emis, c0, d.n3, v);
 #pragma unroll
     for (int k = 0; k < kAllocItems; ++k) acc += quantised<R>(v[k], rmax);
   }
@@ -1726,7 +1953,7 @@ __device__ __forceinline__ void alloc_prefix_batch(const BoxDev* bxs, int B, con
   const BoxDev& d = bxs[b];
   const DevScalars* sc = d.sc;
   const int64_t c0 = (int64_t)(g - d.ablk0) * kAllocChunk + (int64_t)threadIdx.x * kAllocItems;
-  alloc_prefix_block<R>((const R*)d.emis, d.n3, d.npk, __ldcg(&sc->sumQ), __ldcg(&sc->alloc_u), (R)__ldcg(&sc->rmax),
+  alloc_prefix_block<R, kAllocItems>((const R*)d.emis, d.n3, d.npk, __ldcg(&sc->sumQ), __ldcg(&sc->alloc_u), (R)__ldcg(&sc->rmax),
                         __ldcg(&partQ[g]), c0, d.P, d.first, Tiles{d.n, d.nt, d.lg, d.mn, d.mn2, d.tlg}, d.bk0, bcap);
 }
 template <class R>
@@ -1835,9 +2062,6 @@ __global__ void __launch_bounds__(TT, 4) k_emit_batch(TransportArgs<R> a, const 
   emit_batch_body<R, false>(a, bxs, bst, B, tot_pk);
 }
 
-struct BoxStepArgs {
-  BoxStep s[kMaxBoxes];
-};
 __global__ void k_set_box_step(BoxStepArgs p, BoxStep* out, int B) {
   for (int b = threadIdx.x; b < B; b += blockDim.x) out[b] = p.s[b];
 }
@@ -1880,14 +2104,14 @@ __global__ void k_transport_end_batch(const BoxDev* bxs, int B, const unsigned l
 template <class R>
 __global__ void __launch_bounds__(AT, 4) k_batch_front(TransportArgs<R> a, const BoxDev* bxs, BoxStep* bst,
                                                        BoxStepArgs bs, int B, uint32_t k0, uint32_t k1,
-                                                       DevScalars* gsc, double* part, unsigned long long* partQ,
-                                                       unsigned long long* cpre, uint32_t n_ablk, uint64_t tot_pk,
+                                                       DevScalars* gsc, unsigned long long* partQ, unsigned long long* cpre,
+                                                       uint32_t n_ablk, uint64_t tot_pk,
                                                        uint32_t limit) {
   if (blockIdx.x == 0)
     for (int b = threadIdx.x; b < B; b += AT) bst[b] = bs.s[b];
   for (int i = blockIdx.x * AT + threadIdx.x; i < a.nb; i += gridDim.x * AT) a.boff[i] = 0ull;
   if (blockIdx.x == 0 && threadIdx.x == 0) gsc->march_next = ~0ull >> 1;  // no march work until the chunks exist
-  for (uint32_t g = blockIdx.x; g < n_ablk; g += gridDim.x) alloc_max_batch<R>(bxs, B, gsc, part, g, n_ablk);
+  for (uint32_t g = blockIdx.x; g < n_ablk; g += gridDim.x) alloc_max_batch<R>(bxs, bs, B, gsc, g, n_ablk);
   if (!grid_barrier(&gsc->bar, &gsc->flags, limit)) return;
   for (uint32_t g = blockIdx.x; g < n_ablk; g += gridDim.x) alloc_sum_batch<R>(bxs, B, k0, k1, gsc, partQ, g, n_ablk);
   if (!grid_barrier(&gsc->bar, &gsc->flags, limit)) return;
@@ -1935,7 +2159,6 @@ cudaError_t run_transport_batch(rec_ctx* c, int step, double z, rec_stats* st) {
     const BoxDev* bxs = c->bx;
     BoxStep* bst = c->bstep;
     DevScalars* gsc = c->gsc;
-    double* part = c->part;
     unsigned long long* partQ = c->partQ;
     unsigned long long* cpre = c->cpre;
     uint32_t n_ablk = (uint32_t)c->tot_ablk;
@@ -1943,14 +2166,14 @@ cudaError_t run_transport_batch(rec_ctx* c, int step, double z, rec_stats* st) {
     uint32_t limit = c->wait_limit;
     int Bv = B;
     uint32_t k0v = k0, k1v = k1;
-    void* args[] = {&a, &bxs, &bst, &bs, &Bv, &k0v, &k1v, &gsc, &part, &partQ, &cpre, &n_ablk, &tot_pk, &limit};
+    void* args[] = {&a, &bxs, &bst, &bs, &Bv, &k0v, &k1v, &gsc, &partQ, &cpre, &n_ablk, &tot_pk, &limit};
     cudaError_t e = cudaLaunchCooperativeKernel((void*)k_batch_front<R>, c->batch_front_grid, AT, args, 0, c->stream);
     if (e != cudaSuccess) return e;
   } else {
     {
       GroupTimer t(c, kTAlloc, 5);
       k_set_box_step<<<1, kMaxBoxes, 0, c->stream>>>(bs, c->bstep, B);
-      k_alloc_max_batch<R><<<c->tot_ablk, AT, 0, c->stream>>>(c->bx, B, c->gsc, c->part);
+      k_alloc_max_batch<R><<<c->tot_ablk, AT, 0, c->stream>>>(c->bx, bs, B, c->gsc);
       k_alloc_sum_batch<R><<<c->tot_ablk, AT, 0, c->stream>>>(c->bx, B, k0, k1, c->gsc, c->partQ);
       cudaMemsetAsync(c->bcap, 0, sizeof(unsigned long long) * nb, c->stream);
       k_alloc_prefix_batch<R><<<c->tot_ablk, AT, 0, c->stream>>>(c->bx, B, c->partQ, c->bcap);
@@ -1972,6 +2195,11 @@ cudaError_t run_transport_batch(rec_ctx* c, int step, double z, rec_stats* st) {
 }
 
 }  // namespace
+
+int alloc_blocks_single(int64_t n3) {
+  const int64_t cells = (int64_t)AT * alloc_items(n3);
+  return (int)((n3 + cells - 1) / cells);
+}
 
 // Largest resident blocks per SM of the emission and the march (their
 // launch bounds), for the checks of rec_set_tuning.
