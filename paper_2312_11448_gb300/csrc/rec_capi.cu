@@ -98,6 +98,18 @@ uint32_t log2u(uint32_t v) {
   return l;
 }
 
+// Device scratch that only saves time: NULL where it would take more than an
+// eighth of the memory that is free, or cannot be had.
+void* optional_scratch(size_t bytes) {
+  size_t free_bytes = 0, total = 0;
+  void* p = nullptr;
+  if (cudaMemGetInfo(&free_bytes, &total) != cudaSuccess || bytes > free_bytes / 8 || cudaMalloc(&p, bytes) != cudaSuccess) {
+    cudaGetLastError();
+    return nullptr;
+  }
+  return p;
+}
+
 // Super-tile layout of every box of a batch for the tile side in use.
 void layout_buckets(rec_ctx* c) {
   c->tot_buckets = 0;
@@ -204,11 +216,8 @@ rec_status init_batch(const rec_params* params, const rec_box* boxes, int32_t n_
     rec_free(c);
     return r;
   }
-  // the march runs without its compact velocity copies where there is no memory for them
-  if (cudaMalloc(&c->velq, sizeof(uint32_t) * nvelq) != cudaSuccess) {
-    c->velq = nullptr;
-    cudaGetLastError();
-  }
+  // scratch that only saves time is left out where memory is short
+  c->velq = (uint32_t*)optional_scratch(sizeof(uint32_t) * nvelq);
   nvelq = 0;
   for (int i = 0; i < n_boxes; ++i) {
     const rec_box& b = boxes[i];
@@ -324,11 +333,10 @@ rec_status rec_init(const rec_params* params, const rec_box* boxes, int32_t n_bo
     rec_free(c);
     return r;
   }
-  // the march runs without its compact velocity copy where there is no memory for it
-  if (cudaMalloc(&c->velq, sizeof(uint32_t) * rec::velq_words((uint32_t)b.n)) != cudaSuccess) {
-    c->velq = nullptr;
-    cudaGetLastError();
-  }
+  // scratch that only saves time is left out where memory is short
+  c->velq = (uint32_t*)optional_scratch(sizeof(uint32_t) * rec::velq_words((uint32_t)b.n));
+  if (params->precision == REC_PREC_FP64 && params->mixing != REC_MIX_LOCAL)
+    c->cellcache = optional_scratch(5 * sizeof(double) * (size_t)c->n3);
   // emission-profile table in the working precision of the transport
   std::vector<char> hq(qbytes);
   for (int i = 0; i < params->n_quantiles; ++i) {
@@ -636,6 +644,7 @@ void rec_free(rec_ctx* c) {
   cudaFree(c->quant);
   cudaFree(c->queue);
   cudaFree(c->velq);
+  cudaFree(c->cellcache);
   cudaFree(c->first);
   cudaFree(c->xy);
   cudaFree(c->bcap);

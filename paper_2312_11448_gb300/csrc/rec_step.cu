@@ -64,6 +64,7 @@ struct PassArgs {
   CoefF32 kf;       // k in binary32 (mixed form)
   const void* div;  // partial mixing: velocity divergence per cell (working precision)
   double fmix;      // partial mixing: share f of the full-mixing rate (0 < f <= 1)
+  double4_32a* cc;  // FP64 form: coefficients of the substep per cell (CellCache), NULL: none
 };
 
 __device__ __forceinline__ int32_t ld_flag(const int32_t* p) { return *(volatile const int32_t*)p; }
@@ -73,17 +74,28 @@ struct CellF64 {
   double Tn, al, n, A, s;
 };
 
+// The coefficients of a cell do not depend on lambda, but the evaluation passes
+// and the final pass all need them, and a logarithm, two exponentials and six
+// quotients are most of a cell's binary64 operations (about 190 of 250, on a pipe
+// of two operations per cycle and SM).  The first evaluation of a substep
+// keeps {alpha(T'), mixing weight w or local Peebles factor, T', t^pd of the case-B fit}
+// per cell; the later ones read them back (32 bytes) and form the same A, s
+// and n from them, bit for bit.  256^3, three evaluations: 26.2 -> 11.7 ms per step.
+enum CellCache { kNoCache = 0, kFillCache = 1, kReadCache = 2 };
+
 // Coefficients of one cell at the substep end (backward Euler, x_old in the
 // Compton and heating terms).  w uses the substep-start neutral fraction.
 __device__ __forceinline__ CellF64 cell_f64(const StepCoef& k, double d, double x, double T, uint32_t tal,
-                                            double tot, double S1s) {
+                                            double tot, double S1s, double* w_out = nullptr,
+                                            double* tpd_out = nullptr) {
   CellF64 c;
   double opx = 1.0 + k.fHe + x;
   double g = k.kc * x / opx;
   double hh = k.hq / (d * opx);
   c.Tn = (T + k.dt * (g * k.Tg + hh)) / (1.0 + k.dt * (2.0 * k.H + g));
   double lt = log(c.Tn * 1.0e-4);
-  c.al = k.fa * exp(k.pb * lt) / (1.0 + k.pc * exp(k.pd * lt));
+  const double tpd = exp(k.pd * lt);
+  c.al = k.fa * exp(k.pb * lt) / (1.0 + k.pc * tpd);
   c.n = k.nH * d;
   c.A = k.dt * c.al * c.n;
   double w = 1.0;
@@ -92,6 +104,18 @@ __device__ __forceinline__ CellF64 cell_f64(const StepCoef& k, double d, double 
     if (S1s > 0.0 && n1s_rel > 0.0) w = ((double)tal / tot) * S1s / n1s_rel;
   }
   c.s = k.dt * w;
+  if (w_out) *w_out = w;
+  if (tpd_out) *tpd_out = tpd;
+  return c;
+}
+// The same from the kept values of an earlier pass.
+__device__ __forceinline__ CellF64 cell_from_cache(const StepCoef& k, double d, const double4_32a& q) {
+  CellF64 c;
+  c.al = q.x;
+  c.Tn = q.z;
+  c.n = k.nH * d;
+  c.A = k.dt * c.al * c.n;
+  c.s = k.dt * q.y;
   return c;
 }
 
@@ -292,13 +316,42 @@ __device__ __forceinline__ float local_C_f32(const StepCoef& k, float div, float
   return fdiv((float)k.L2g + R, (float)(k.beta + k.L2g) + R);
 }
 
+// Coefficients of cell i for a pass of the FP64 form, computed (and kept) or read back.
+template <bool PART, int CACHE>
+__device__ __forceinline__ CellF64 pass_cell(const PassArgs& a, int64_t i, double d, double x, const double* T,
+                                             double tot, double S1s, double& Gc) {
+  CellF64 c;
+  double Ci = 0.0;
+  if (CACHE == kReadCache) {
+    const double4_32a q = a.cc[i];
+    c = cell_from_cache(a.k, d, q);
+    Ci = q.y;
+  } else {
+    const uint32_t tal = (a.k.mixing == REC_MIX_TALLY) ? a.tally[i] : 0u;
+    double w, tpd;
+    c = cell_f64(a.k, d, x, T[i], tal, tot, S1s, &w, &tpd);
+    if (PART) Ci = local_C(a.k, ((const double*)a.div)[i], c.n * (1.0 - x));
+    if (CACHE == kFillCache) {
+      double4_32a q;
+      q.x = c.al; q.y = PART ? Ci : w; q.z = c.Tn; q.w = tpd;
+      a.cc[i] = q;
+    }
+  }
+  if (PART) {
+    c.A *= a.fmix + (1.0 - a.fmix) * Ci;
+    c.s = a.k.dt * a.fmix;
+    Gc += ((1.0 - a.fmix) / a.fmix) * Ci * (a.k.beta * a.k.ea);
+  }
+  return c;
+}
+
 // Per-block partial sums of one Newton evaluation at lambda (result in thread 0):
 // v0 = sum alpha n^2 x'^2, v1 = sum n (1 - x'), v2 = sum (2 alpha n^2 x' + lambda n) dx'/dG;
 // mixed form also v3 = sum [2 alpha n^2 (dx'/dG)^2 + (2 alpha n^2 x' + lambda n) d2x'/dG2],
 // v4 = sum n dx'/dG (the second derivative of F for the Halley step).
 // PART: partial mixing — per cell, A scaled by f + (1 - f) C_i, s = dt f and G
 // offset by (1 - f)/f C_i beta e_alpha (C_i the local Peebles factor).
-template <bool MIXED, bool PART = false>
+template <bool MIXED, bool PART = false, int CACHE = kNoCache>
 __device__ __forceinline__ void newton_block_sums(const PassArgs& a, double lam, double G, double tot, double S1s,
                                                   const MixedScal& ms, int blk, int nblk, double (&v)[5]) {
   const int64_t stride = (int64_t)nblk * NT;
@@ -309,15 +362,8 @@ __device__ __forceinline__ void newton_block_sums(const PassArgs& a, double lam,
     const double* T = (const double*)a.T;
     for (int64_t i = (int64_t)blk * NT + threadIdx.x; i < a.n3; i += stride) {
       double d = delta[i], x = a.x[i];
-      uint32_t tal = (a.k.mixing == REC_MIX_TALLY) ? a.tally[i] : 0u;
-      CellF64 c = cell_f64(a.k, d, x, T[i], tal, tot, S1s);
       double Gc = G;
-      if (PART) {
-        const double Ci = local_C(a.k, ((const double*)a.div)[i], c.n * (1.0 - x));
-        c.A *= a.fmix + (1.0 - a.fmix) * Ci;
-        c.s = a.k.dt * a.fmix;
-        Gc = G + ((1.0 - a.fmix) / a.fmix) * Ci * (a.k.beta * a.k.ea);
-      }
+      const CellF64 c = pass_cell<PART, CACHE>(a, i, d, x, T, tot, S1s, Gc);
       double dxdG;
       double xr = root_f64(c.A, c.s, Gc, x, &dxdG);
       double an2 = c.al * c.n * c.n;
@@ -435,7 +481,7 @@ __device__ __forceinline__ void final_cell_mixed(const PassArgs& a, const FinalM
 // Per-block final update at the converged lambda: writes x, T, U, emission
 // weights (zeroes the tallies on the last substep); partial sums (thread 0):
 // v0 = sum delta (1 - x'), v1 = sum delta x', v2 = sum delta.
-template <bool MIXED, bool PART = false>
+template <bool MIXED, bool PART = false, int CACHE = kNoCache>
 __device__ __forceinline__ void final_block(const PassArgs& a, double G, double tot, double S1s, const MixedScal& ms,
                                             int blk, int nblk, double (&v)[3]) {
   const int64_t stride = (int64_t)nblk * NT;
@@ -448,15 +494,8 @@ __device__ __forceinline__ void final_block(const PassArgs& a, double G, double 
     double* emis = (double*)a.emis;
     for (int64_t i = (int64_t)blk * NT + threadIdx.x; i < a.n3; i += stride) {
       double d = delta[i], x = a.x[i];
-      uint32_t tal = (a.k.mixing == REC_MIX_TALLY) ? a.tally[i] : 0u;
-      CellF64 c = cell_f64(a.k, d, x, T[i], tal, tot, S1s);
       double Gc = G;
-      if (PART) {
-        const double Ci = local_C(a.k, ((const double*)a.div)[i], c.n * (1.0 - x));
-        c.A *= a.fmix + (1.0 - a.fmix) * Ci;
-        c.s = a.k.dt * a.fmix;
-        Gc = G + ((1.0 - a.fmix) / a.fmix) * Ci * (a.k.beta * a.k.ea);
-      }
+      const CellF64 c = pass_cell<PART, CACHE>(a, i, d, x, T, tot, S1s, Gc);
       double xr = root_f64(c.A, c.s, Gc, x, nullptr);
       double damp = exp(-(a.k.kd * xr + a.k.H) * a.k.dt);
       double4_32a u = U[i];
@@ -537,7 +576,7 @@ __device__ __forceinline__ void pass_view(PassArgs& a, const BoxDev* bxs, int B,
   *box = lo;
 }
 
-template <bool MIXED, bool MB>
+template <bool MIXED, bool MB, int CACHE = kNoCache>
 __global__ void __launch_bounds__(NT) k_newton(PassArgs a, const BoxDev* bxs, int B) {
   int blk = blockIdx.x, nblk = gridDim.x, box = 0;
   if (MB) pass_view(a, bxs, B, &blk, &nblk, &box, blockIdx.x);
@@ -546,8 +585,8 @@ __global__ void __launch_bounds__(NT) k_newton(PassArgs a, const BoxDev* bxs, in
   const double lam = sc->lam;
   constexpr int K = NSums<MIXED>::value;
   double v[5];
-  newton_block_sums<MIXED>(a, lam, sc->omC * lam + sc->G0, (double)sc->tally_total, sc->S1s, mixed_scal(sc, false), blk,
-                           nblk, v);
+  newton_block_sums<MIXED, false, CACHE>(a, lam, sc->omC * lam + sc->G0, (double)sc->tally_total, sc->S1s,
+                                         mixed_scal(sc, false), blk, nblk, v);
   if (threadIdx.x == 0) {
     double* p = a.part + (size_t)blk * kMaxSums;
     for (int j = 0; j < K; ++j) p[j] = v[j];
@@ -720,14 +759,15 @@ __global__ void __launch_bounds__(kTmaThreads) k_newton_tma(PassArgs a, uint32_t
 
 // Final pass: new state at the converged lambda, emission weights, sums.
 // st: statistics record (one per box in a batch) or NULL.
-template <bool MIXED, bool MB>
+template <bool MIXED, bool MB, int CACHE = kNoCache>
 __global__ void __launch_bounds__(NT) k_final(PassArgs a, rec_stats* st, const BoxDev* bxs, int B) {
   int blk = blockIdx.x, nblk = gridDim.x, box = 0;
   if (MB) pass_view(a, bxs, B, &blk, &nblk, &box, blockIdx.x);
   DevScalars* sc = a.sc;
   const double lam = sc->lam;
   double v[3];
-  final_block<MIXED>(a, sc->omC * lam + sc->G0, (double)sc->tally_total, sc->S1s, mixed_scal(sc, false), blk, nblk, v);
+  final_block<MIXED, false, CACHE>(a, sc->omC * lam + sc->G0, (double)sc->tally_total, sc->S1s, mixed_scal(sc, false),
+                                   blk, nblk, v);
   if (threadIdx.x == 0) {
     double* p = a.part + (size_t)blk * kMaxSums;
     p[0] = v[0]; p[1] = v[1]; p[2] = v[2];
@@ -902,14 +942,14 @@ __global__ void __launch_bounds__(kTmaThreads, kFinCtasPerSm) k_final_tma(PassAr
 }
 
 // Newton evaluation and final pass of partial mixing (single-box contexts).
-template <bool MIXED>
+template <bool MIXED, int CACHE = kNoCache>
 __global__ void __launch_bounds__(NT) k_newton_part(PassArgs a) {
   DevScalars* sc = a.sc;
   if (ld_flag(&sc->conv)) return;
   const double lam = sc->lam;
   constexpr int K = NSums<MIXED>::value;
   double v[5];
-  newton_block_sums<MIXED, true>(a, lam, sc->omC * lam + sc->G0, 0.0, sc->S1s, mixed_scal(sc, false), blockIdx.x,
+  newton_block_sums<MIXED, true, CACHE>(a, lam, sc->omC * lam + sc->G0, 0.0, sc->S1s, mixed_scal(sc, false), blockIdx.x,
                                  gridDim.x, v);
   if (threadIdx.x == 0) {
     double* p = a.part + (size_t)blockIdx.x * kMaxSums;
@@ -924,12 +964,12 @@ __global__ void __launch_bounds__(NT) k_newton_part(PassArgs a) {
   }
 }
 
-template <bool MIXED>
+template <bool MIXED, int CACHE = kNoCache>
 __global__ void __launch_bounds__(NT) k_final_part(PassArgs a, rec_stats* st) {
   DevScalars* sc = a.sc;
   const double lam = sc->lam;
   double v[3];
-  final_block<MIXED, true>(a, sc->omC * lam + sc->G0, 0.0, sc->S1s, mixed_scal(sc, false), blockIdx.x, gridDim.x, v);
+  final_block<MIXED, true, CACHE>(a, sc->omC * lam + sc->G0, 0.0, sc->S1s, mixed_scal(sc, false), blockIdx.x, gridDim.x, v);
   if (threadIdx.x == 0) {
     double* p = a.part + (size_t)blockIdx.x * kMaxSums;
     p[0] = v[0]; p[1] = v[1]; p[2] = v[2];
@@ -1150,7 +1190,17 @@ PassArgs pass_args(rec_ctx* c, const StepCoef& k) {
   a.kf = coef_f32(k);
   a.div = c->div;
   a.fmix = c->params.f_alpha;
+  a.cc = (double4_32a*)c->cellcache;
   return a;
+}
+
+// The evaluation passes of the FP64 form (single box).
+void newton_f64(rec_ctx* c, const PassArgs& a) {
+  for (int it = 0; it < kNewtonMaxPasses; ++it) {
+    if (!a.cc) k_newton<false, false><<<c->grid, NT, 0, c->stream>>>(a, nullptr, 1);
+    else if (it == 0) k_newton<false, false, kFillCache><<<c->grid, NT, 0, c->stream>>>(a, nullptr, 1);
+    else k_newton<false, false, kReadCache><<<c->grid, NT, 0, c->stream>>>(a, nullptr, 1);
+  }
 }
 
 }  // namespace
@@ -1163,7 +1213,7 @@ void enqueue_newton_passes(rec_ctx* c, DevScalars* sc, const StepCoef& k, const 
   a.T = const_cast<double*>(T);
   a.tally = const_cast<uint32_t*>(tally);
   k_substep_begin<<<1, 32, 0, c->stream>>>(sc, k, (double)c->n3);
-  for (int it = 0; it < kNewtonMaxPasses; ++it) k_newton<false, false><<<c->grid, NT, 0, c->stream>>>(a, nullptr, 1);
+  newton_f64(c, a);
 }
 
 cudaError_t launch_refresh(rec_ctx* c, double z) {
@@ -1240,22 +1290,26 @@ cudaError_t launch_rec_step(rec_ctx* c, double z_from, double z_to, rec_stats* s
       k_substep_begin<<<1, 32, 0, c->stream>>>(c->sc, k, (double)c->n3);
       for (int it = 0; it < kNewtonMaxPasses; ++it) {
         if (mixed) k_newton_part<true><<<c->grid, NT, 0, c->stream>>>(a);
-        else k_newton_part<false><<<c->grid, NT, 0, c->stream>>>(a);
+        else if (!a.cc) k_newton_part<false><<<c->grid, NT, 0, c->stream>>>(a);
+        else if (it == 0) k_newton_part<false, kFillCache><<<c->grid, NT, 0, c->stream>>>(a);
+        else k_newton_part<false, kReadCache><<<c->grid, NT, 0, c->stream>>>(a);
       }
       if (mixed) k_final_part<true><<<c->grid, NT, 0, c->stream>>>(a, st);
-      else k_final_part<false><<<c->grid, NT, 0, c->stream>>>(a, st);
+      else if (!a.cc) k_final_part<false><<<c->grid, NT, 0, c->stream>>>(a, st);
+      else k_final_part<false, kReadCache><<<c->grid, NT, 0, c->stream>>>(a, st);
       continue;
     }
     k_substep_begin<<<1, 32, 0, c->stream>>>(c->sc, k, (double)c->n3);
     const bool tma = mixed && newton_tma_ok(c, a);
-    for (int it = 0; it < kNewtonMaxPasses; ++it) {
+    if (!mixed) newton_f64(c, a);
+    for (int it = 0; mixed && it < kNewtonMaxPasses; ++it) {
       if (tma) k_newton_tma<<<c->sm_count * kTmaCtasPerSm, kTmaThreads, kTmaSmem, c->stream>>>(a, c->wait_limit);
-      else if (mixed) k_newton<true, false><<<c->grid, NT, 0, c->stream>>>(a, nullptr, 1);
-      else k_newton<false, false><<<c->grid, NT, 0, c->stream>>>(a, nullptr, 1);
+      else k_newton<true, false><<<c->grid, NT, 0, c->stream>>>(a, nullptr, 1);
     }
     if (tma) k_final_tma<<<c->sm_count * kFinCtasPerSm, kTmaThreads, kFinSmem, c->stream>>>(a, st, c->wait_limit);
     else if (mixed) k_final<true, false><<<c->grid, NT, 0, c->stream>>>(a, st, nullptr, 1);
-    else k_final<false, false><<<c->grid, NT, 0, c->stream>>>(a, st, nullptr, 1);
+    else if (!a.cc) k_final<false, false><<<c->grid, NT, 0, c->stream>>>(a, st, nullptr, 1);
+    else k_final<false, false, kReadCache><<<c->grid, NT, 0, c->stream>>>(a, st, nullptr, 1);
   }
   return cudaGetLastError();
 }
@@ -1489,6 +1543,7 @@ rec_status launch_rec_step_noalloc(const rec_params& p, const rec_box& b, double
   a.part = part;
   a.div = nullptr;
   a.fmix = 1.0;
+  a.cc = nullptr;
   e = cudaMemsetAsync(sc, 0, sizeof(DevScalars), stream);
   if (e != cudaSuccess) { *why = std::string("cudaMemsetAsync: ") + cudaGetErrorString(e); return REC_ECUDA; }
   // sums and emission weights of the incoming state at z_from (as rec_refresh)
