@@ -138,7 +138,7 @@ __global__ void __launch_bounds__(NT) k_adj_prep(AdjArgs a) {
     a.sc->tally_total = (unsigned long long)(S[2] + 0.5);
     a.sc->lam_state = S[0] > 0.0 ? al * a.k.nH * S[3] / S[0] : 0.0;
     a.sc->lam_prev = -1.0;
-    a.sc->flags = 0;
+    a.sc->flags &= 8;  // an expired wait stays until it is reported
     a.sc->counter = 0;
   }
 }
@@ -317,9 +317,10 @@ cudaError_t launch_rec_step_adjoint(rec_ctx* c, double z_from, double z_to, cons
   a.k = k;
   a.cc = (const double4_32a*)c->cellcache;
   a.xr = a.cc ? (double*)c->cellcache + 4 * c->n3 : nullptr;
-  GroupTimer t(c, kTAdj, kNewtonMaxPasses + 5);
+  GroupTimer t(c, kTAdj, 5);
   adj::k_adj_prep<<<c->grid, adj::NT, 0, c->stream>>>(a);
-  enqueue_newton_passes(c, c->sc_adj, k, x_in, T_in, tally_in);
+  cudaError_t e = enqueue_newton_passes(c, c->sc_adj, k, x_in, T_in, tally_in);
+  if (e != cudaSuccess) return e;
   if (a.cc) {
     adj::k_adj_r1<true><<<c->grid, adj::NT, 0, c->stream>>>(a);
     adj::k_adj_r2<true><<<c->grid, adj::NT, 0, c->stream>>>(a);

@@ -36,15 +36,29 @@ __device__ __forceinline__ int ld_relaxed_i32(const int* p) {
 
 // Returns true in every thread of the block once all blocks of the grid have
 // arrived; false (in every thread) if the wait expired here or elsewhere.
-__device__ __forceinline__ bool grid_barrier(GridBarrier* g, int* flags, uint32_t limit) {
-  __shared__ int s_ok;
+// last(): run by all threads of the last block to arrive, before the barrier
+// opens: it sees what every block wrote before its arrival (through L2), and every
+// block sees what it writes.
+template <class F>
+__device__ __forceinline__ bool grid_barrier(GridBarrier* g, int* flags, uint32_t limit, F last) {
+  __shared__ int s_ok, s_last;
   __syncthreads();  // the block's work of this phase is done
+  unsigned int gen = 0;
+  if (threadIdx.x == 0) {
+    gen = ld_acquire_u32(&g->gen);
+    __threadfence();  // this block's writes before its arrival
+    s_last = atomicAdd(&g->arrived, 1u) == gridDim.x - 1;
+    __threadfence();  // the other blocks' writes before last()
+  }
+  __syncthreads();
+  const bool am_last = s_last != 0;
+  if (am_last) {
+    last();
+    __syncthreads();
+  }
   if (threadIdx.x == 0) {
     int ok = 1;
-    const unsigned int gen = ld_acquire_u32(&g->gen);
-    __threadfence();  // this block's writes before its arrival
-    const unsigned int a = atomicAdd(&g->arrived, 1u);
-    if (a == gridDim.x - 1) {
+    if (am_last) {
       g->arrived = 0;  // reset before the barrier opens: nobody arrives again before that
       __threadfence();
       atomicAdd(&g->gen, 1u);
@@ -57,7 +71,7 @@ __device__ __forceinline__ bool grid_barrier(GridBarrier* g, int* flags, uint32_
           break;
         }
         ++polls;
-        __nanosleep(256);
+        __nanosleep(64);
       }
     }
     __threadfence();  // the other blocks' writes are visible to this block's threads
@@ -66,6 +80,9 @@ __device__ __forceinline__ bool grid_barrier(GridBarrier* g, int* flags, uint32_
   }
   __syncthreads();
   return s_ok != 0;
+}
+__device__ __forceinline__ bool grid_barrier(GridBarrier* g, int* flags, uint32_t limit) {
+  return grid_barrier(g, flags, limit, [] {});
 }
 
 }  // namespace rec

@@ -60,7 +60,7 @@ struct DevScalars {
   unsigned long long requeued;     // region sweeps: packets queued again in this transport call
   uint32_t alloc_counter;
   int32_t emis_valid;
-  GridBarrier bar;  // grid barrier of the persistent batched launches (batch-wide record)
+  GridBarrier bar;  // grid barrier of the persistent launches (of a batch: in the batch-wide record)
   // binary32 copies of the current iterate for the mixed form's passes (set
   // with lam, so that no pass converts binary64 scalars per thread)
   float lamf;        // lambda
@@ -167,7 +167,9 @@ struct rec_ctx {
   void* quant;               // emission-profile table (float or double) [n_quantiles]
   int grid;                  // blocks of the streaming passes
   int alloc_blocks;
-  int newton_tma = 0;        // TMA-staged Newton pass usable (0: not yet queried, 1 / -1)
+  int newton_tma = 0;        // TMA-staged substep usable (0: not yet queried, 1 / -1)
+  int substep_resident[16] = {};  // resident blocks per SM of the persistent substeps (0: not queried), and of
+  int tma_resident = 0;           // the TMA-staged one
   int batch_step_grid = 0;   // resident blocks of the persistent batched substep (0: not queried, -1: none)
   int batch_front_grid = 0;  // resident blocks of the persistent batched transport front (same)
   void* queue;               // queued packets of the march (2 x 16 B binary32, 3 x 32 B binary64) [n_packets]
@@ -269,7 +271,7 @@ cudaError_t launch_check_waits(rec_ctx* c, int* timed_out);
 rec_status launch_rec_step_noalloc(const rec_params& p, const rec_box& b, double z_from, double z_to,
                                    cudaStream_t stream, rec_stats* st, std::string* why);
 // Newton passes for lambda of a substep on an arbitrary FP64 state (used by the adjoint).
-void enqueue_newton_passes(rec_ctx* c, DevScalars* sc, const StepCoef& k, const double* x, const double* T,
+cudaError_t enqueue_newton_passes(rec_ctx* c, DevScalars* sc, const StepCoef& k, const double* x, const double* T,
                            const uint32_t* tally);
 
 // rec_transport.cu

@@ -12,12 +12,13 @@
 // (Eq. R-alpha, Sec. IV.A.2).  T_b follows Eq. (Tb-evolution) and the velocity
 // Eq. (momentum) with the drag rate of Eq. (alpha-def).
 //
-// Pass structure per substep (all on the context stream, no host sync):
-//   k_substep_begin  (1 block)  C, G offset and the lambda guess from device sums
-//   k_newton x N     streaming  F(lambda), F'(lambda); last block takes the Newton step;
-//                               exits immediately once converged
-//   k_final          streaming  writes x, T, U, emission weights, zeroes tallies,
-//                               and the sums of the new state
+// A substep is one persistent cooperative launch (no host sync): C, the G offset and
+// the lambda guess from device sums; evaluations of F(lambda), F'(lambda), the last
+// block to arrive at the grid barrier taking the step on lambda, until it has
+// converged; then the final pass: x, T, U, emission weights, tallies zeroed and the sums
+// of the new state.  (One launch per evaluation, ten of them with those after
+// convergence returning at once, was 40 us per substep slower: 256^3 mixed substep
+// 379 -> 339 us, two partial-mixing substeps of 128^3 443 -> 289 us.)
 // Two forms: FP64 (all binary64) and MIXED (binary32 per-cell coefficients and
 // root, binary64 state x, net-rate residual correction and volume sums).
 
@@ -38,14 +39,21 @@ constexpr int NT = kPassThreads;
 struct CoefF32 {
   float dt, H2, nH, Tg, kc, opf, hq, fa, pb, pc, pd;
   float kd, H;  // drag coefficient per unit x and H, for the final pass
+  // local Peebles factor (local and partial mixing): 8 pi / lambda_alpha^3, the two-photon
+  // rate, beta + the two-photon rate, beta e_alpha; the share f and (1 - f) / f
+  float KRH, L2g, bL, bea, fm, fr;
 };
-// Binary32 coefficients of a substep, formed once on the host.
-__host__ __device__ inline CoefF32 coef_f32(const StepCoef& k) {
+// Binary32 coefficients of a substep, formed once on the host: formed per thread,
+// the conversions and quotients take longer than a small box's cells.
+inline CoefF32 coef_f32(const StepCoef& k, double fmix = 1.0) {
   CoefF32 f;
   f.dt = (float)k.dt; f.H2 = (float)(2.0 * k.H); f.nH = (float)k.nH; f.Tg = (float)k.Tg; f.kc = (float)k.kc;
   f.opf = (float)(1.0 + k.fHe); f.hq = (float)k.hq; f.fa = (float)k.fa; f.pb = (float)k.pb; f.pc = (float)k.pc;
   f.pd = (float)k.pd;
   f.kd = (float)k.kd; f.H = (float)k.H;
+  f.KRH = (float)(k.KR / k.H); f.L2g = (float)k.L2g; f.bL = (float)(k.beta + k.L2g); f.bea = (float)(k.beta * k.ea);
+  f.fm = (float)fmix;
+  f.fr = (1.0f - f.fm) / f.fm;
   return f;
 }
 
@@ -221,18 +229,27 @@ __device__ __forceinline__ MixedScal mixed_scal(const DevScalars* sc, bool via_l
 }
 
 // Substep prologue: C from the device sum S1s, Newton start.
-__device__ void substep_begin(DevScalars* sc, const StepCoef& k, double n3) {
+struct SubstepStart {
+  double C, lam;
+};
+__device__ __forceinline__ SubstepStart substep_start(const DevScalars* sc, const StepCoef& k, double n3) {
   double n1s_mean = k.nH * sc->S1s / n3;
   double R = k.KR / n1s_mean;
-  double C = (k.L2g + R) / (k.beta + k.L2g + R);
-  sc->C = C;
-  sc->omC = 1.0 - C;
-  sc->G0 = C * k.beta * k.ea;
+  SubstepStart s;
+  s.C = (k.L2g + R) / (k.beta + k.L2g + R);
   double guess = sc->lam_state;
   if (sc->lam_prev > 0.0 && sc->lam_state > 0.0)  // extrapolate the last substep's change (at most 2x)
     guess = sc->lam_state * fmin(2.0, fmax(0.5, sc->lam_state / sc->lam_prev));
   if (!(guess > 0.0)) guess = 1e-30;
-  sc->lam = guess;
+  s.lam = guess;
+  return s;
+}
+__device__ void substep_begin(DevScalars* sc, const StepCoef& k, double n3) {
+  const SubstepStart s = substep_start(sc, k, n3);
+  sc->C = s.C;
+  sc->omC = 1.0 - s.C;
+  sc->G0 = s.C * k.beta * k.ea;
+  sc->lam = s.lam;
   set_mixed_scal(sc);
   sc->conv = 0;
   sc->passes = 0;
@@ -309,11 +326,11 @@ __device__ __forceinline__ double local_C(const StepCoef& k, double div, double 
   const double R = (k.KR / k.H) * Heff / n1s;
   return (k.L2g + R) / (k.beta + k.L2g + R);
 }
-__device__ __forceinline__ float local_C_f32(const StepCoef& k, float div, float n1s) {
-  const float Heff = fmaxf((float)k.H + div / 3.0f, 0.0f);
+__device__ __forceinline__ float local_C_f32(const CoefF32& f, float div, float n1s) {
+  const float Heff = fmaxf(f.H + div / 3.0f, 0.0f);
   if (!(n1s > 0.0f)) return 1.0f;
-  const float R = fdiv((float)(k.KR / k.H) * Heff, n1s);
-  return fdiv((float)k.L2g + R, (float)(k.beta + k.L2g) + R);
+  const float R = fdiv(f.KRH * Heff, n1s);
+  return fdiv(f.L2g + R, f.bL + R);
 }
 
 // Coefficients of cell i for a pass of the FP64 form, computed (and kept) or read back.
@@ -382,11 +399,10 @@ __device__ __forceinline__ void newton_block_sums(const PassArgs& a, double lam,
       CellF32 c = cell_f32(f, a.k.mixing, delta[i], a.xy[i], T[i], tal, wscale);
       float Gc = Gf;
       if (PART) {
-        const float fm = (float)a.fmix;
-        const float Ci = local_C_f32(a.k, ((const float*)a.div)[i], c.n * c.yf);
-        c.A *= fm + (1.0f - fm) * Ci;
-        c.s = f.dt * fm;
-        Gc = Gf + ((1.0f - fm) / fm) * Ci * (float)(a.k.beta * a.k.ea);
+        const float Ci = local_C_f32(f, ((const float*)a.div)[i], c.n * c.yf);
+        c.A *= f.fm + (1.0f - f.fm) * Ci;
+        c.s = f.dt * f.fm;
+        Gc = Gf + f.fr * Ci * f.bea;
       }
       float xr, yr, dxdG, d2;
       root_f32(c.A, c.s, Gc, c.xf, c.yf, &xr, &yr, &dxdG, &d2);
@@ -439,11 +455,10 @@ __device__ __forceinline__ void final_cell_mixed(const PassArgs& a, const FinalM
   float Gcf = m.Gf;
   dfloat Gc = m.Gd;
   if (PART) {
-    const float fm = (float)a.fmix;
-    const float Ci = local_C_f32(a.k, ((const float*)a.div)[i], c.n * c.yf);
-    c.A *= fm + (1.0f - fm) * Ci;
-    c.s = f.dt * fm;
-    const float go = ((1.0f - fm) / fm) * Ci * (float)(a.k.beta * a.k.ea);
+    const float Ci = local_C_f32(f, ((const float*)a.div)[i], c.n * c.yf);
+    c.A *= f.fm + (1.0f - f.fm) * Ci;
+    c.s = f.dt * f.fm;
+    const float go = f.fr * Ci * f.bea;
     Gcf = m.Gf + go;
     Gc = df_add(m.Gd, dfloat{go, 0.0f});
   }
@@ -576,7 +591,7 @@ __device__ __forceinline__ void pass_view(PassArgs& a, const BoxDev* bxs, int B,
   *box = lo;
 }
 
-template <bool MIXED, bool MB, int CACHE = kNoCache>
+template <bool MIXED, bool MB>
 __global__ void __launch_bounds__(NT) k_newton(PassArgs a, const BoxDev* bxs, int B) {
   int blk = blockIdx.x, nblk = gridDim.x, box = 0;
   if (MB) pass_view(a, bxs, B, &blk, &nblk, &box, blockIdx.x);
@@ -585,8 +600,8 @@ __global__ void __launch_bounds__(NT) k_newton(PassArgs a, const BoxDev* bxs, in
   const double lam = sc->lam;
   constexpr int K = NSums<MIXED>::value;
   double v[5];
-  newton_block_sums<MIXED, false, CACHE>(a, lam, sc->omC * lam + sc->G0, (double)sc->tally_total, sc->S1s,
-                                         mixed_scal(sc, false), blk, nblk, v);
+  newton_block_sums<MIXED>(a, lam, sc->omC * lam + sc->G0, (double)sc->tally_total, sc->S1s, mixed_scal(sc, false), blk,
+                           nblk, v);
   if (threadIdx.x == 0) {
     double* p = a.part + (size_t)blk * kMaxSums;
     for (int j = 0; j < K; ++j) p[j] = v[j];
@@ -622,7 +637,6 @@ struct TmaStage {
   uint32_t tally[kTmaTile];
 };
 constexpr uint32_t kTmaStageBytes = kTmaTile * (4 + 8 + 4 + 4);
-constexpr size_t kTmaSmem = sizeof(TmaStage) * kTmaStages + 8 * kTmaStages;
 static_assert(sizeof(TmaStage) == kTmaStageBytes, "stage layout");
 
 __device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -666,108 +680,16 @@ __device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t b
                : "memory");
 }
 
-__global__ void __launch_bounds__(kTmaThreads) k_newton_tma(PassArgs a, uint32_t limit) {
-  DevScalars* sc = a.sc;
-  if (ld_flag(&sc->conv)) return;
-  extern __shared__ __align__(128) unsigned char smem_raw[];
-  TmaStage* stage = reinterpret_cast<TmaStage*>(smem_raw);
-  uint64_t* full = reinterpret_cast<uint64_t*>(smem_raw + sizeof(TmaStage) * kTmaStages);
-  const MixedScal ms = mixed_scal(sc, false);
-  const int64_t n_tiles = a.n3 / kTmaTile;  // whole tiles, copied in bulk
-  const int64_t my_tiles = n_tiles > (int64_t)blockIdx.x ? (n_tiles - blockIdx.x + gridDim.x - 1) / gridDim.x : 0;
-  const float* delta = (const float*)a.delta;
-  const float* Tg = (const float*)a.T;
-  if (threadIdx.x == 0) {
-    for (int s = 0; s < kTmaStages; ++s) mbar_init(&full[s], 1);
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  }
-  __syncthreads();
-  auto issue = [&](int64_t it) {  // thread 0: tile `it` of this CTA into its stage
-    const int s = (int)(it % kTmaStages);
-    const int64_t c0 = ((int64_t)blockIdx.x + it * gridDim.x) * kTmaTile;
-    mbar_expect_tx(&full[s], kTmaStageBytes);
-    bulk_load(stage[s].delta, delta + c0, kTmaTile * 4, &full[s]);
-    bulk_load(stage[s].xy, a.xy + c0, kTmaTile * 8, &full[s]);
-    bulk_load(stage[s].T, Tg + c0, kTmaTile * 4, &full[s]);
-    bulk_load(stage[s].tally, a.tally + c0, kTmaTile * 4, &full[s]);
-  };
-  if (threadIdx.x == 0)
-    for (int64_t it = 0; it < my_tiles && it < kTmaStages - 1; ++it) issue(it);
-  Kahan32 acc[5];
-  const CoefF32& f = a.kf;
-  const float Gf = ms.Gf, lamf = ms.lamf, wscale = ms.wscale;
-  auto cell = [&](float d, float2 xy, float T, uint32_t tal) {
-    CellF32 c = cell_f32(f, a.k.mixing, d, xy, T, (a.k.mixing == REC_MIX_TALLY) ? tal : 0u, wscale);
-    float xr, yr, dxdG, d2;
-    root_f32(c.A, c.s, Gf, c.xf, c.yf, &xr, &yr, &dxdG, &d2);
-    float an2 = c.al * c.n * c.n;
-    const float q = 2.0f * an2 * xr + lamf * c.n;
-    acc[0].add(an2 * xr * xr);
-    acc[1].add(c.n * yr);
-    acc[2].add(q * dxdG);
-    acc[3].add(2.0f * an2 * dxdG * dxdG + q * d2);
-    acc[4].add(c.n * dxdG);
-  };
-  bool timed_out = false;
-  int64_t it = 0;
-  for (; it < my_tiles; ++it) {
-    if (threadIdx.x == 0 && it + kTmaStages - 1 < my_tiles) {
-      // the stage refilled here was read by every thread before the barrier that ended the last iteration
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-      issue(it + kTmaStages - 1);
-    }
-    const int s = (int)(it % kTmaStages);
-    const uint32_t parity = (uint32_t)((it / kTmaStages) & 1);
-    if (!mbar_wait_bounded(&full[s], parity, limit)) timed_out = true;
-    if (!timed_out) {
-      const TmaStage& t = stage[s];
-      for (int k = threadIdx.x; k < kTmaTile; k += kTmaThreads) cell(t.delta[k], t.xy[k], t.T[k], t.tally[k]);
-    }
-    if (__syncthreads_or(timed_out)) { timed_out = true; break; }
-  }
-  if (timed_out) {
-    if (threadIdx.x == 0) {
-      atomicOr(&sc->flags, 8);
-      // the copies issued for the tiles it .. it + kTmaStages - 2 may still be in flight
-      for (int64_t j = it; j < my_tiles && j < it + kTmaStages - 1; ++j) {
-        uint32_t polls = 0;
-        while (!mbar_try_wait(&full[j % kTmaStages], (uint32_t)((j / kTmaStages) & 1)) && ++polls < kTmaWaitLimit) {
-        }
-      }
-    }
-    __syncthreads();
-    return;
-  }
-  // cells after the last whole tile
-  for (int64_t i = n_tiles * kTmaTile + (int64_t)blockIdx.x * kTmaThreads + threadIdx.x; i < a.n3;
-       i += (int64_t)gridDim.x * kTmaThreads)
-    cell(delta[i], a.xy[i], Tg[i], a.tally[i]);
-  double v[5];
-  block_sum_kahan<5, kTmaThreads>(acc, v);
-  if (threadIdx.x == 0) {
-    double* p = a.part + (size_t)blockIdx.x * kMaxSums;
-    for (int j = 0; j < 5; ++j) p[j] = v[j];
-  }
-  if (!last_block_done(&sc->counter)) return;
-  double S[5];
-  combine_partials<5, kTmaThreads>(a.part, gridDim.x, kMaxSums, S);
-  if (threadIdx.x == 0) {
-    halley_update(sc, S[0], S[1], S[2], S[3], S[4]);
-    sc->counter = 0;
-  }
-}
-
 // Final pass: new state at the converged lambda, emission weights, sums.
 // st: statistics record (one per box in a batch) or NULL.
-template <bool MIXED, bool MB, int CACHE = kNoCache>
+template <bool MIXED, bool MB>
 __global__ void __launch_bounds__(NT) k_final(PassArgs a, rec_stats* st, const BoxDev* bxs, int B) {
   int blk = blockIdx.x, nblk = gridDim.x, box = 0;
   if (MB) pass_view(a, bxs, B, &blk, &nblk, &box, blockIdx.x);
   DevScalars* sc = a.sc;
   const double lam = sc->lam;
   double v[3];
-  final_block<MIXED, false, CACHE>(a, sc->omC * lam + sc->G0, (double)sc->tally_total, sc->S1s, mixed_scal(sc, false),
-                                   blk, nblk, v);
+  final_block<MIXED>(a, sc->omC * lam + sc->G0, (double)sc->tally_total, sc->S1s, mixed_scal(sc, false), blk, nblk, v);
   if (threadIdx.x == 0) {
     double* p = a.part + (size_t)blk * kMaxSums;
     p[0] = v[0]; p[1] = v[1]; p[2] = v[2];
@@ -841,15 +763,92 @@ __global__ void __launch_bounds__(NT) k_batch_substep(PassArgs a0, rec_stats* st
   }
 }
 
-// ---- final pass of the mixed form with TMA-staged tiles ----------------------------
-// The final pass streams five inputs per cell (Delta, x, T, tallies, velocity;
-// 36 B) and writes six outputs.  As in the Newton evaluation, persistent CTAs
-// bring tiles of kTmaTile cells of the inputs into a ring of shared-memory
-// stages with bulk asynchronous copies, so that the loads are in flight while
-// the previous tile is computed; the outputs are stored directly.  Waits are
-// bounded as in k_newton_tma.
+// ---- one substep of a single box as one persistent launch --------------------------
+// Scalars of the substep as a block reads them: computed by every block itself
+// before the first evaluation (block 0 also stores them), through L2 after that.
+struct SubstepScal {
+  double lam, omC, G0, tot, S1s;
+  MixedScal ms;
+};
+// One thread per block: every thread's copy of these few binary64 operations
+// would occupy the slow pipe for 9 us.
+__device__ __forceinline__ SubstepScal substep_open(DevScalars* sc, const StepCoef& k, double n3) {
+  __shared__ SubstepScal open;
+  if (threadIdx.x == 0) {
+    SubstepScal s;
+    const SubstepStart b = substep_start(sc, k, n3);
+    s.lam = b.lam;
+    s.omC = 1.0 - b.C;
+    s.G0 = b.C * k.beta * k.ea;
+    s.S1s = sc->S1s;
+    s.tot = (double)sc->tally_total;
+    const double G = s.omC * s.lam + s.G0;
+    s.ms.lamf = (float)s.lam;
+    s.ms.Gf = (float)G;
+    s.ms.Gd = df_from_double(G);
+    s.ms.wscale = sc->tally_total > 0 ? (float)(s.S1s / s.tot) : 0.0f;
+    open = s;
+    // stored before this block arrives at the first barrier, so before any step on lambda
+    if (blockIdx.x == 0) substep_begin(sc, k, n3);
+  }
+  __syncthreads();
+  return open;
+}
+// After a step on lambda (behind a barrier); false once lambda has converged.
+__device__ __forceinline__ bool substep_next(DevScalars* sc, SubstepScal& s) {
+  s.lam = __ldcg(&sc->lam);
+  s.ms = mixed_scal(sc, true);
+  return __ldcg(&sc->conv) == 0;
+}
+
+// Any form and size: the pass blocks of the grid-stride passes (nvb of them, so
+// that the sums are taken in the same order whatever is resident) run as virtual
+// blocks of the resident grid.  FINAL false: the evaluations only (adjoint).
+template <bool MIXED, bool PART, bool CACHE, bool FINAL>
+__global__ void __launch_bounds__(NT, 4) k_substep(PassArgs a, rec_stats* st, int nvb, uint32_t limit) {
+  DevScalars* sc = a.sc;
+  constexpr int K = NSums<MIXED>::value;
+  SubstepScal s = substep_open(sc, a.k, (double)a.n3);
+  for (int pass = 0; pass < kNewtonMaxPasses; ++pass) {
+    for (int g = blockIdx.x; g < nvb; g += gridDim.x) {
+      double v[5];
+      const double G = s.omC * s.lam + s.G0;
+      if (CACHE && pass > 0) newton_block_sums<MIXED, PART, CACHE ? kReadCache : kNoCache>(a, s.lam, G, s.tot, s.S1s, s.ms, g, nvb, v);
+      else newton_block_sums<MIXED, PART, CACHE ? kFillCache : kNoCache>(a, s.lam, G, s.tot, s.S1s, s.ms, g, nvb, v);
+      if (threadIdx.x == 0) {
+        double* p = a.part + (size_t)g * kMaxSums;
+        for (int j = 0; j < K; ++j) p[j] = v[j];
+      }
+    }
+    const bool ok = grid_barrier(&sc->bar, &sc->flags, limit, [&] {
+      double S[5];
+      combine_partials_first<K, NT>(a.part, nvb, kMaxSums, S);
+      if (threadIdx.x == 0) lambda_update<MIXED>(sc, S);
+    });
+    if (!ok) return;
+    if (!substep_next(sc, s)) break;
+  }
+  if constexpr (FINAL) {
+    for (int g = blockIdx.x; g < nvb; g += gridDim.x) {
+      double v[3];
+      final_block<MIXED, PART, CACHE ? kReadCache : kNoCache>(a, s.omC * s.lam + s.G0, s.tot, s.S1s, s.ms, g, nvb, v);
+      if (threadIdx.x == 0) {
+        double* p = a.part + (size_t)g * kMaxSums;
+        p[0] = v[0]; p[1] = v[1]; p[2] = v[2];
+      }
+    }
+    if (!last_block_done(&sc->counter)) return;
+    double S[3];
+    combine_partials<3, NT>(a.part, nvb, kMaxSums, S);
+    if (threadIdx.x == 0) finish_substep(sc, a.k, S, s.lam, st);
+  }
+}
+
+// The mixed form (tally and full mixing) with tiles staged by bulk copies.
+// Evaluations: the four per-cell inputs in kTmaStages stages of kTmaTile cells.  Final
+// pass: its five inputs (Delta, x, T, tallies, velocity; 36 B) in kFinStages stages of the
+// same shared memory; the outputs are stored directly.
 constexpr int kFinStages = 2;
-constexpr int kFinCtasPerSm = 3;
 struct FinStage {
   float delta[kTmaTile];
   double x[kTmaTile];
@@ -857,76 +856,148 @@ struct FinStage {
   uint32_t tally[kTmaTile];
   float4 U[kTmaTile];
 };
-constexpr size_t kFinSmem = sizeof(FinStage) * kFinStages + 8 * kFinStages;
+constexpr size_t kRingBytes = sizeof(FinStage) * kFinStages > sizeof(TmaStage) * kTmaStages
+                                  ? sizeof(FinStage) * kFinStages : sizeof(TmaStage) * kTmaStages;
+constexpr size_t kTmaSmem = kRingBytes + 8 * (kTmaStages + kFinStages);
 
-__global__ void __launch_bounds__(kTmaThreads, kFinCtasPerSm) k_final_tma(PassArgs a, rec_stats* st, uint32_t limit) {
-  DevScalars* sc = a.sc;
-  extern __shared__ __align__(128) unsigned char smem_raw[];
-  FinStage* stage = reinterpret_cast<FinStage*>(smem_raw);
-  uint64_t* full = reinterpret_cast<uint64_t*>(smem_raw + sizeof(FinStage) * kFinStages);
-  const double lam = sc->lam;
-  const FinalMixed fm = final_mixed_setup(a, mixed_scal(sc, false));
-  const bool zero_tally = a.k.last != 0;
-  const bool tally_mode = a.k.mixing == REC_MIX_TALLY;
-  const uint32_t stage_bytes = kTmaTile * (4 + 8 + 4 + 16) + (tally_mode ? kTmaTile * 4 : 0);
-  const int64_t n_tiles = a.n3 / kTmaTile;
-  const int64_t my_tiles = n_tiles > (int64_t)blockIdx.x ? (n_tiles - blockIdx.x + gridDim.x - 1) / gridDim.x : 0;
-  const float* delta = (const float*)a.delta;
-  const float* Tg = (const float*)a.T;
-  const float4* Ug = (const float4*)a.vel4;
-  if (threadIdx.x == 0) {
-    for (int s = 0; s < kFinStages; ++s) mbar_init(&full[s], 1);
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  }
-  __syncthreads();
-  auto issue = [&](int64_t it) {  // thread 0: tile `it` of this CTA into its stage
-    const int s = (int)(it % kFinStages);
-    const int64_t c0 = ((int64_t)blockIdx.x + it * gridDim.x) * kTmaTile;
-    mbar_expect_tx(&full[s], stage_bytes);
-    bulk_load(stage[s].delta, delta + c0, kTmaTile * 4, &full[s]);
-    bulk_load(stage[s].x, a.x + c0, kTmaTile * 8, &full[s]);
-    bulk_load(stage[s].T, Tg + c0, kTmaTile * 4, &full[s]);
-    if (tally_mode) bulk_load(stage[s].tally, a.tally + c0, kTmaTile * 4, &full[s]);
-    bulk_load(stage[s].U, Ug + c0, kTmaTile * 16, &full[s]);
+// One CTA's share of a pass: tiles blockIdx.x, blockIdx.x + gridDim.x, ... through a
+// ring of STAGES stages.  issue(s, c0, bar): the copies of the tile at cell c0 into
+// stage s; use(s, c0): the cells of a tile.  seq: tiles this ring has taken before
+// (stage and parity go on from it).  False: a wait expired (flags bit 3 is set and
+// the CTA's copies in flight have been waited for, bounded by kTmaWaitLimit).
+template <int STAGES, class I, class U>
+__device__ __forceinline__ bool tile_pass(int64_t n3, uint64_t* full, int64_t& seq, DevScalars* sc, uint32_t limit,
+                                          I issue, U use) {
+  const int64_t n_tiles = n3 / kTmaTile;
+  const int64_t mine = n_tiles > (int64_t)blockIdx.x ? (n_tiles - blockIdx.x + gridDim.x - 1) / gridDim.x : 0;
+  auto start = [&](int64_t it) {
+    const int q = (int)((seq + it) % STAGES);
+    issue(q, ((int64_t)blockIdx.x + it * gridDim.x) * kTmaTile, &full[q]);
   };
-  if (threadIdx.x == 0)
-    for (int64_t it = 0; it < my_tiles && it < kFinStages - 1; ++it) issue(it);
-  Kahan32 acc[3];
+  if (threadIdx.x == 0) {
+    // the ring was last read by every thread before a barrier of the block
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    for (int64_t it = 0; it < mine && it < STAGES - 1; ++it) start(it);
+  }
   bool timed_out = false;
   int64_t it = 0;
-  for (; it < my_tiles; ++it) {
-    if (threadIdx.x == 0 && it + kFinStages - 1 < my_tiles) {
+  for (; it < mine; ++it) {
+    if (threadIdx.x == 0 && it + STAGES - 1 < mine) {
       // the stage refilled here was read by every thread before the barrier that ended the last iteration
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-      issue(it + kFinStages - 1);
+      start(it + STAGES - 1);
     }
-    const int s = (int)(it % kFinStages);
-    const uint32_t parity = (uint32_t)((it / kFinStages) & 1);
-    if (!mbar_wait_bounded(&full[s], parity, limit)) timed_out = true;
-    if (!timed_out) {
-      const FinStage& t = stage[s];
-      const int64_t c0 = ((int64_t)blockIdx.x + it * gridDim.x) * kTmaTile;
-      for (int k = threadIdx.x; k < kTmaTile; k += kTmaThreads)
-        final_cell_mixed<false>(a, fm, zero_tally, c0 + k, t.delta[k], t.x[k], t.T[k], tally_mode ? t.tally[k] : 0u,
-                                t.U[k], acc);
-    }
+    const int q = (int)((seq + it) % STAGES);
+    if (!mbar_wait_bounded(&full[q], (uint32_t)(((seq + it) / STAGES) & 1), limit)) timed_out = true;
+    if (!timed_out) use(q, ((int64_t)blockIdx.x + it * gridDim.x) * kTmaTile);
     if (__syncthreads_or(timed_out)) { timed_out = true; break; }
   }
   if (timed_out) {
     if (threadIdx.x == 0) {
       atomicOr(&sc->flags, 8);
-      // the copies issued for the tiles it .. it + kFinStages - 2 may still be in flight
-      for (int64_t j = it; j < my_tiles && j < it + kFinStages - 1; ++j) {
+      // the copies issued for the tiles it .. it + STAGES - 2 may still be in flight
+      for (int64_t j = it; j < mine && j < it + STAGES - 1; ++j) {
         uint32_t polls = 0;
-        while (!mbar_try_wait(&full[j % kFinStages], (uint32_t)((j / kFinStages) & 1)) && ++polls < kTmaWaitLimit) {
+        while (!mbar_try_wait(&full[(seq + j) % STAGES], (uint32_t)(((seq + j) / STAGES) & 1)) &&
+               ++polls < kTmaWaitLimit) {
         }
       }
     }
     __syncthreads();
-    return;
+    return false;
   }
-  // cells after the last whole tile
-  for (int64_t i = n_tiles * kTmaTile + (int64_t)blockIdx.x * kTmaThreads + threadIdx.x; i < a.n3;
+  seq += mine;
+  return true;
+}
+
+__global__ void __launch_bounds__(kTmaThreads, kTmaCtasPerSm) k_substep_tma(PassArgs a, rec_stats* st, uint32_t limit) {
+  DevScalars* sc = a.sc;
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem_raw + kRingBytes);
+  const bool tally_mode = a.k.mixing == REC_MIX_TALLY;
+  const float* delta = (const float*)a.delta;
+  const float* Tg = (const float*)a.T;
+  const int64_t tail = a.n3 / kTmaTile * kTmaTile;  // cells after the last whole tile are read directly
+  if (threadIdx.x == 0) {
+    for (int q = 0; q < kTmaStages + kFinStages; ++q) mbar_init(&full[q], 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  SubstepScal s = substep_open(sc, a.k, (double)a.n3);
+  __syncthreads();
+  int64_t seq = 0;
+  for (int pass = 0; pass < kNewtonMaxPasses; ++pass) {
+    TmaStage* stage = reinterpret_cast<TmaStage*>(smem_raw);
+    Kahan32 acc[5];
+    const CoefF32& f = a.kf;
+    const float Gf = s.ms.Gf, lamf = s.ms.lamf, wscale = s.ms.wscale;
+    auto cell = [&](float d, float2 xy, float T, uint32_t tal) {
+      CellF32 c = cell_f32(f, a.k.mixing, d, xy, T, tally_mode ? tal : 0u, wscale);
+      float xr, yr, dxdG, d2;
+      root_f32(c.A, c.s, Gf, c.xf, c.yf, &xr, &yr, &dxdG, &d2);
+      float an2 = c.al * c.n * c.n;
+      const float q = 2.0f * an2 * xr + lamf * c.n;
+      acc[0].add(an2 * xr * xr);
+      acc[1].add(c.n * yr);
+      acc[2].add(q * dxdG);
+      acc[3].add(2.0f * an2 * dxdG * dxdG + q * d2);
+      acc[4].add(c.n * dxdG);
+    };
+    const bool done = tile_pass<kTmaStages>(
+        a.n3, full, seq, sc, limit,
+        [&](int q, int64_t c0, uint64_t* bar) {
+          mbar_expect_tx(bar, kTmaStageBytes);
+          bulk_load(stage[q].delta, delta + c0, kTmaTile * 4, bar);
+          bulk_load(stage[q].xy, a.xy + c0, kTmaTile * 8, bar);
+          bulk_load(stage[q].T, Tg + c0, kTmaTile * 4, bar);
+          bulk_load(stage[q].tally, a.tally + c0, kTmaTile * 4, bar);
+        },
+        [&](int q, int64_t) {
+          const TmaStage& t = stage[q];
+          for (int k = threadIdx.x; k < kTmaTile; k += kTmaThreads) cell(t.delta[k], t.xy[k], t.T[k], t.tally[k]);
+        });
+    if (!done) return;
+    for (int64_t i = tail + (int64_t)blockIdx.x * kTmaThreads + threadIdx.x; i < a.n3;
+         i += (int64_t)gridDim.x * kTmaThreads)
+      cell(delta[i], a.xy[i], Tg[i], a.tally[i]);
+    double v[5];
+    block_sum_kahan<5, kTmaThreads>(acc, v);
+    if (threadIdx.x == 0) {
+      double* p = a.part + (size_t)blockIdx.x * kMaxSums;
+      for (int j = 0; j < 5; ++j) p[j] = v[j];
+    }
+    const bool ok = grid_barrier(&sc->bar, &sc->flags, limit, [&] {
+      double S[5];
+      combine_partials<5, kTmaThreads>(a.part, gridDim.x, kMaxSums, S);
+      if (threadIdx.x == 0) halley_update(sc, S[0], S[1], S[2], S[3], S[4]);
+    });
+    if (!ok) return;
+    if (!substep_next(sc, s)) break;
+  }
+  FinStage* stage = reinterpret_cast<FinStage*>(smem_raw);
+  const FinalMixed fm = final_mixed_setup(a, s.ms);
+  const bool zero_tally = a.k.last != 0;
+  const uint32_t stage_bytes = kTmaTile * (4 + 8 + 4 + 16) + (tally_mode ? kTmaTile * 4 : 0);
+  const float4* Ug = (const float4*)a.vel4;
+  Kahan32 acc[3];
+  seq = 0;
+  const bool done = tile_pass<kFinStages>(
+      a.n3, full + kTmaStages, seq, sc, limit,
+      [&](int q, int64_t c0, uint64_t* bar) {
+        mbar_expect_tx(bar, stage_bytes);
+        bulk_load(stage[q].delta, delta + c0, kTmaTile * 4, bar);
+        bulk_load(stage[q].x, a.x + c0, kTmaTile * 8, bar);
+        bulk_load(stage[q].T, Tg + c0, kTmaTile * 4, bar);
+        if (tally_mode) bulk_load(stage[q].tally, a.tally + c0, kTmaTile * 4, bar);
+        bulk_load(stage[q].U, Ug + c0, kTmaTile * 16, bar);
+      },
+      [&](int q, int64_t c0) {
+        const FinStage& t = stage[q];
+        for (int k = threadIdx.x; k < kTmaTile; k += kTmaThreads)
+          final_cell_mixed<false>(a, fm, zero_tally, c0 + k, t.delta[k], t.x[k], t.T[k], tally_mode ? t.tally[k] : 0u,
+                                  t.U[k], acc);
+      });
+  if (!done) return;
+  for (int64_t i = tail + (int64_t)blockIdx.x * kTmaThreads + threadIdx.x; i < a.n3;
        i += (int64_t)gridDim.x * kTmaThreads)
     final_cell_mixed<false>(a, fm, zero_tally, i, delta[i], a.x[i], Tg[i], tally_mode ? a.tally[i] : 0u, Ug[i], acc);
   double v[3];
@@ -938,46 +1009,7 @@ __global__ void __launch_bounds__(kTmaThreads, kFinCtasPerSm) k_final_tma(PassAr
   if (!last_block_done(&sc->counter)) return;
   double S[3];
   combine_partials<3, kTmaThreads>(a.part, gridDim.x, kMaxSums, S);
-  if (threadIdx.x == 0) finish_substep(sc, a.k, S, lam, st);
-}
-
-// Newton evaluation and final pass of partial mixing (single-box contexts).
-template <bool MIXED, int CACHE = kNoCache>
-__global__ void __launch_bounds__(NT) k_newton_part(PassArgs a) {
-  DevScalars* sc = a.sc;
-  if (ld_flag(&sc->conv)) return;
-  const double lam = sc->lam;
-  constexpr int K = NSums<MIXED>::value;
-  double v[5];
-  newton_block_sums<MIXED, true, CACHE>(a, lam, sc->omC * lam + sc->G0, 0.0, sc->S1s, mixed_scal(sc, false), blockIdx.x,
-                                 gridDim.x, v);
-  if (threadIdx.x == 0) {
-    double* p = a.part + (size_t)blockIdx.x * kMaxSums;
-    for (int j = 0; j < K; ++j) p[j] = v[j];
-  }
-  if (!last_block_done(&sc->counter)) return;
-  double S[5];
-  combine_partials_first<K, NT>(a.part, gridDim.x, kMaxSums, S);
-  if (threadIdx.x == 0) {
-    lambda_update<MIXED>(sc, S);
-    sc->counter = 0;
-  }
-}
-
-template <bool MIXED, int CACHE = kNoCache>
-__global__ void __launch_bounds__(NT) k_final_part(PassArgs a, rec_stats* st) {
-  DevScalars* sc = a.sc;
-  const double lam = sc->lam;
-  double v[3];
-  final_block<MIXED, true, CACHE>(a, sc->omC * lam + sc->G0, 0.0, sc->S1s, mixed_scal(sc, false), blockIdx.x, gridDim.x, v);
-  if (threadIdx.x == 0) {
-    double* p = a.part + (size_t)blockIdx.x * kMaxSums;
-    p[0] = v[0]; p[1] = v[1]; p[2] = v[2];
-  }
-  if (!last_block_done(&sc->counter)) return;
-  double S[3];
-  combine_partials<3, NT>(a.part, gridDim.x, kMaxSums, S);
-  if (threadIdx.x == 0) finish_substep(sc, a.k, S, lam, st);
+  if (threadIdx.x == 0) finish_substep(sc, a.k, S, s.lam, st);
 }
 
 // ---------------------------------------------------------- no-mixing limit
@@ -1050,17 +1082,17 @@ __global__ void __launch_bounds__(NT) k_local(PassArgs a, const void* div, rec_s
     }
   } else {
     Kahan32 s0, s1, s2, s3, s4, s5;
-    const CoefF32 f = coef_f32(k);
+    const CoefF32& f = a.kf;
     const float* delta = (const float*)a.delta;
     float* T = (float*)a.T;
     float4* U = (float4*)a.vel4;
     float* emis = (float*)a.emis;
-    const float kdf = (float)k.kd, Hf = (float)k.H, dtf = (float)k.dt, beaf = (float)bea;
+    const float kdf = f.kd, Hf = f.H, dtf = f.dt, beaf = f.bea;
     for (int64_t i = (int64_t)blockIdx.x * NT + threadIdx.x; i < a.n3; i += stride) {
       const float d = delta[i];
       const double x = a.x[i];
       CellF32 c = cell_f32(f, REC_MIX_FULL, d, a.xy[i], T[i], 0u, 0.0f);
-      const float Ci = local_C_f32(k, ((const float*)div)[i], c.n * c.yf);
+      const float Ci = local_C_f32(f, ((const float*)div)[i], c.n * c.yf);
       const float A = c.A * Ci, sG = c.s * Ci * beaf;
       // binary32 roots and the binary64 increment of the state, as in k_final
       const float B = 1.0f + sG;
@@ -1154,6 +1186,7 @@ __global__ void __launch_bounds__(NT) k_refresh(PassArgs a, const BoxDev* bxs, i
     sc->lam_prev = -1.0;
     sc->tally_total = (unsigned long long)(S[5] + 0.5);
     sc->flags = 0;
+    sc->bar.arrived = 0;  // a substep that gave up may have left arrivals
     sc->emis_valid = 1;
     sc->counter = 0;
   }
@@ -1187,33 +1220,47 @@ PassArgs pass_args(rec_ctx* c, const StepCoef& k) {
   a.sc = c->sc;
   a.part = c->part;
   a.k = k;
-  a.kf = coef_f32(k);
+  a.kf = coef_f32(k, c->params.f_alpha);
   a.div = c->div;
   a.fmix = c->params.f_alpha;
   a.cc = (double4_32a*)c->cellcache;
   return a;
 }
 
-// The evaluation passes of the FP64 form (single box).
-void newton_f64(rec_ctx* c, const PassArgs& a) {
-  for (int it = 0; it < kNewtonMaxPasses; ++it) {
-    if (!a.cc) k_newton<false, false><<<c->grid, NT, 0, c->stream>>>(a, nullptr, 1);
-    else if (it == 0) k_newton<false, false, kFillCache><<<c->grid, NT, 0, c->stream>>>(a, nullptr, 1);
-    else k_newton<false, false, kReadCache><<<c->grid, NT, 0, c->stream>>>(a, nullptr, 1);
+// Launches one persistent substep kernel; resident: blocks per SM looked up once per context and kernel.
+template <class F>
+cudaError_t launch_resident(rec_ctx* c, F kernel, int threads, size_t smem, int* resident, int blocks, void** args) {
+  if (*resident == 0) {
+    cudaError_t e = smem ? cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) : cudaSuccess;
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(resident, kernel, threads, smem);
+    if (e != cudaSuccess) { *resident = 0; return e; }
+    if (*resident < 1) return cudaErrorCooperativeLaunchTooLarge;
   }
+  const int grid = std::min(blocks, *resident * c->sm_count);
+  return cudaLaunchCooperativeKernel((const void*)kernel, dim3(grid), dim3(threads), args, smem, c->stream);
+}
+
+template <bool MIXED, bool PART, bool CACHE, bool FINAL>
+cudaError_t launch_substep(rec_ctx* c, PassArgs a, rec_stats* st) {
+  int nvb = c->grid;
+  uint32_t limit = c->wait_limit;
+  void* args[] = {&a, &st, &nvb, &limit};
+  return launch_resident(c, k_substep<MIXED, PART, CACHE, FINAL>, NT, 0,
+                         &c->substep_resident[(MIXED ? 8 : 0) + (PART ? 4 : 0) + (CACHE ? 2 : 0) + (FINAL ? 1 : 0)], nvb,
+                         args);
 }
 
 }  // namespace
 
-void enqueue_newton_passes(rec_ctx* c, DevScalars* sc, const StepCoef& k, const double* x, const double* T,
+cudaError_t enqueue_newton_passes(rec_ctx* c, DevScalars* sc, const StepCoef& k, const double* x, const double* T,
                            const uint32_t* tally) {
   PassArgs a = pass_args(c, k);
   a.sc = sc;
   a.x = const_cast<double*>(x);
   a.T = const_cast<double*>(T);
   a.tally = const_cast<uint32_t*>(tally);
-  k_substep_begin<<<1, 32, 0, c->stream>>>(sc, k, (double)c->n3);
-  newton_f64(c, a);
+  return a.cc ? launch_substep<false, false, true, false>(c, a, nullptr)
+              : launch_substep<false, false, false, false>(c, a, nullptr);
 }
 
 cudaError_t launch_refresh(rec_ctx* c, double z) {
@@ -1238,21 +1285,14 @@ cudaError_t launch_state_init(rec_ctx* c, double z) {
   return launch_refresh(c, z);
 }
 
-// The TMA-staged Newton and final passes need 16-byte aligned streams (bulk
-// copies) and their shared-memory rings; REC_NEWTON=plain selects the
-// grid-stride kernels.
+// The TMA-staged substep needs 16-byte aligned streams (bulk copies);
+// REC_NEWTON=plain selects the grid-stride one.
 bool newton_tma_ok(rec_ctx* c, const PassArgs& a) {
   if (c->newton_tma == 0) {
     const char* sel = std::getenv("REC_NEWTON");
     bool ok = !(sel && std::strcmp(sel, "plain") == 0);
-    ok = ok && cudaFuncSetAttribute(k_newton_tma, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTmaSmem) ==
-                   cudaSuccess;
-    ok = ok && cudaFuncSetAttribute(k_final_tma, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFinSmem) ==
-                   cudaSuccess;
-    // their blocks fit the partials (2 x grid entries)
-    ok = ok && kTmaCtasPerSm * c->sm_count <= 2 * c->grid && kFinCtasPerSm * c->sm_count <= 2 * c->grid;
+    ok = ok && kTmaCtasPerSm * c->sm_count <= 2 * c->grid;  // its blocks fit the partials (2 x grid entries)
     c->newton_tma = ok ? 1 : -1;
-    cudaGetLastError();
   }
   auto al = [](const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; };
   return c->newton_tma > 0 && al(a.delta) && al(a.xy) && al(a.T) && al(a.tally) && al(a.x) && al(a.vel4);
@@ -1265,7 +1305,7 @@ cudaError_t launch_rec_step(rec_ctx* c, double z_from, double z_to, rec_stats* s
   const bool local_modes = c->params.mixing == REC_MIX_LOCAL || c->params.mixing == REC_MIX_PARTIAL;
   const bool one_pass = c->params.mixing == REC_MIX_LOCAL ||
                         (c->params.mixing == REC_MIX_PARTIAL && !(c->params.f_alpha > 0.0));
-  GroupTimer t(c, kTStep, one_pass ? 2 * ns : ns * (kNewtonMaxPasses + 2 + (local_modes ? 1 : 0)));
+  GroupTimer t(c, kTStep, one_pass || local_modes ? 2 * ns : ns);
   for (int s = 0; s < ns; ++s) {
     double za = (s == 0) ? z_from : std::expm1(ya - (ya - yb) * (double)s / ns);
     double zb = (s == ns - 1) ? z_to : std::expm1(ya - (ya - yb) * (double)(s + 1) / ns);
@@ -1283,33 +1323,24 @@ cudaError_t launch_rec_step(rec_ctx* c, double z_from, double z_to, rec_stats* s
       }
       continue;
     }
-    if (part) {  // divergence, then the Newton passes and the final pass with the local shares
+    cudaError_t e;
+    if (part) {  // divergence, then the substep with the local shares
       const double fac = (1.0 + zb) * 1.0e3 / (2.0 * c->cosmo.L_m / c->box.n);
       if (mixed) k_divergence<true><<<c->grid, NT, 0, c->stream>>>(c->box.vel4, c->box.n, fac, c->div);
       else k_divergence<false><<<c->grid, NT, 0, c->stream>>>(c->box.vel4, c->box.n, fac, c->div);
-      k_substep_begin<<<1, 32, 0, c->stream>>>(c->sc, k, (double)c->n3);
-      for (int it = 0; it < kNewtonMaxPasses; ++it) {
-        if (mixed) k_newton_part<true><<<c->grid, NT, 0, c->stream>>>(a);
-        else if (!a.cc) k_newton_part<false><<<c->grid, NT, 0, c->stream>>>(a);
-        else if (it == 0) k_newton_part<false, kFillCache><<<c->grid, NT, 0, c->stream>>>(a);
-        else k_newton_part<false, kReadCache><<<c->grid, NT, 0, c->stream>>>(a);
-      }
-      if (mixed) k_final_part<true><<<c->grid, NT, 0, c->stream>>>(a, st);
-      else if (!a.cc) k_final_part<false><<<c->grid, NT, 0, c->stream>>>(a, st);
-      else k_final_part<false, kReadCache><<<c->grid, NT, 0, c->stream>>>(a, st);
-      continue;
+      e = mixed ? launch_substep<true, true, false, true>(c, a, st)
+                : (a.cc ? launch_substep<false, true, true, true>(c, a, st)
+                        : launch_substep<false, true, false, true>(c, a, st));
+    } else if (!mixed) {
+      e = a.cc ? launch_substep<false, false, true, true>(c, a, st) : launch_substep<false, false, false, true>(c, a, st);
+    } else if (newton_tma_ok(c, a)) {
+      uint32_t limit = c->wait_limit;
+      void* args[] = {&a, &st, &limit};
+      e = launch_resident(c, k_substep_tma, kTmaThreads, kTmaSmem, &c->tma_resident, kTmaCtasPerSm * c->sm_count, args);
+    } else {
+      e = launch_substep<true, false, false, true>(c, a, st);
     }
-    k_substep_begin<<<1, 32, 0, c->stream>>>(c->sc, k, (double)c->n3);
-    const bool tma = mixed && newton_tma_ok(c, a);
-    if (!mixed) newton_f64(c, a);
-    for (int it = 0; mixed && it < kNewtonMaxPasses; ++it) {
-      if (tma) k_newton_tma<<<c->sm_count * kTmaCtasPerSm, kTmaThreads, kTmaSmem, c->stream>>>(a, c->wait_limit);
-      else k_newton<true, false><<<c->grid, NT, 0, c->stream>>>(a, nullptr, 1);
-    }
-    if (tma) k_final_tma<<<c->sm_count * kFinCtasPerSm, kTmaThreads, kFinSmem, c->stream>>>(a, st, c->wait_limit);
-    else if (mixed) k_final<true, false><<<c->grid, NT, 0, c->stream>>>(a, st, nullptr, 1);
-    else if (!a.cc) k_final<false, false><<<c->grid, NT, 0, c->stream>>>(a, st, nullptr, 1);
-    else k_final<false, false, kReadCache><<<c->grid, NT, 0, c->stream>>>(a, st, nullptr, 1);
+    if (e != cudaSuccess) return e;
   }
   return cudaGetLastError();
 }
@@ -1348,18 +1379,19 @@ cudaError_t launch_volume_stats(rec_ctx* c, rec_stats* st) {
 
 // Expired bounded waits (flags bit 3) of every box: reported in *out and
 // cleared, with the counters a pass that gave up may have left part-way.
-__global__ void k_check_waits(DevScalars* sc, const BoxDev* bxs, int B, DevScalars* gsc, int* out) {
+__global__ void k_check_waits(DevScalars* sc, const BoxDev* bxs, int B, DevScalars* gsc, DevScalars* adj, int* out) {
   if (threadIdx.x != 0) return;
   // a batch-wide expiry (a grid barrier gave up) may have left any box part-way
   const bool all = gsc && (gsc->flags & 8);
   int any = all ? 1 : 0;
-  for (int b = 0; b < B; ++b) {
-    DevScalars* s = bxs ? bxs[b].sc : sc;
-    if (all || (s->flags & 8)) {
+  for (int b = -1; b < B; ++b) {
+    DevScalars* s = b < 0 ? adj : (bxs ? bxs[b].sc : sc);
+    if ((all && b >= 0) || (s->flags & 8)) {
       any = 1;
       s->flags &= ~8;
       s->counter = 0;
       s->alloc_counter = 0;
+      s->bar.arrived = 0;
     }
   }
   if (all) {
@@ -1376,7 +1408,7 @@ cudaError_t launch_check_waits(rec_ctx* c, int* timed_out) {
   cudaError_t e = cudaStreamSynchronize(c->stream);
   if (e != cudaSuccess) return e;
   k_check_waits<<<1, 32, 0, c->stream>>>(c->sc, c->n_boxes > 1 ? c->bx : nullptr, c->n_boxes,
-                                         c->n_boxes > 1 ? c->gsc : nullptr, d);
+                                         c->n_boxes > 1 ? c->gsc : nullptr, c->sc_adj, d);
   e = cudaMemcpyAsync(timed_out, d, sizeof(int), cudaMemcpyDeviceToHost, c->stream);
   if (e != cudaSuccess) return e;
   return cudaStreamSynchronize(c->stream);
