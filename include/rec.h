@@ -390,7 +390,7 @@ typedef struct {
   uint64_t max_steps;  /* per photon (>= 1); a photon reaching it ends as LYA_MC_CAPPED */
   int32_t step;        /* keys the random streams (with rec_params.seed) */
   int32_t pending;     /* lanes of a warp waiting to scatter before the warp runs the
-                          redistribution for them, 1..32; 0: 12.  Speed only: results
+                          redistribution for them, 1..32; 0: 18.  Speed only: results
                           do not depend on it. */
   int32_t arith;       /* LYA_MC_FP64 (0): binary64 throughout, the oracle's operation
                           order.  LYA_MC_MIXED (1): binary32 with double-float pairs for

@@ -154,36 +154,53 @@ __device__ __forceinline__ void philox(uint32_t c0, uint32_t c1, uint32_t c2, ui
   out[0] = c0; out[1] = c1; out[2] = c2; out[3] = c3;
 }
 
-__device__ __forceinline__ double u01(uint32_t lo, uint32_t hi) {
-  const uint64_t w = ((uint64_t)hi << 32) | lo;
-  return __ull2double_rn((w >> 11) | 1ull) * 0x1p-53;
-}
-
 // One photon's stream: key (seed low word, seed high word ^ step), counter
-// (cell, photon index in the cell, block, 2^31 | box); two binary64 deviates
-// per block, used in order.
-struct McRng {
-  uint32_t cell, j, blk, tag, k0, k1;
-  double spare;
-  bool have;
+// (cell, photon index in the cell, block, 2^31 | box); its words are used in order.
+// The words wait in shared memory, kRingWords per thread, and ensure(n) tops
+// them up: lanes come to it together, so that the ten rounds of a block run with
+// most of a warp's lanes.  (Generated by each lane when it had run out, the rounds
+// ran at every draw, for a quarter of the lanes.)
+constexpr int kRingWords = 32;  // ensure(n): n <= kRingWords - 3
+struct McWords {
+  uint32_t cell, j, blk, tag, k0, k1, used;
+  uint32_t* buf;  // word w at buf[(w mod kRingWords) * stride]
+  uint32_t stride;
+  __device__ __forceinline__ McWords(uint32_t* b, uint32_t s) : cell(0), j(0), blk(0), tag(0), k0(0), k1(0), used(0), buf(b), stride(s) {}
   __device__ __forceinline__ void init(uint32_t c, uint32_t jj, uint32_t key0, uint32_t key1, uint32_t box) {
-    cell = c; j = jj; blk = 0; tag = 0x80000000u | box; k0 = key0; k1 = key1; have = false;
+    cell = c; j = jj; blk = 0; tag = 0x80000000u | box; k0 = key0; k1 = key1; used = 0;
   }
-  __device__ __forceinline__ double next() {
-    if (have) { have = false; return spare; }
-    uint32_t r[4];
-    philox(cell, j, blk, tag, k0, k1, r);
-    ++blk;
-    spare = u01(r[2], r[3]);
-    have = true;
-    return u01(r[0], r[1]);
+  __device__ __forceinline__ void ensure(uint32_t n) {
+    while (4u * blk - used < n) {
+      uint32_t r[4];
+      philox(cell, j, blk, tag, k0, k1, r);
+      uint32_t* p = buf + (4u * blk & (kRingWords - 1)) * stride;
+      p[0] = r[0]; p[stride] = r[1]; p[2u * stride] = r[2]; p[3u * stride] = r[3];
+      ++blk;
+    }
   }
+  __device__ __forceinline__ uint32_t word() {
+    const uint32_t v = buf[(used & (kRingWords - 1)) * stride];
+    ++used;
+    return v;
+  }
+};
+// Binary64 deviates, two words each.
+struct McRng : McWords {
+  using McWords::McWords;
+  __device__ __forceinline__ void ensure(uint32_t n) { McWords::ensure(2u * n); }
+  // The deviate is bits() 2^-53.
+  __device__ __forceinline__ uint64_t bits() {
+    const uint32_t lo = word(), hi = word();
+    return ((((uint64_t)hi << 32) | lo) >> 11) | 1ull;
+  }
+  __device__ __forceinline__ double next() { return __ull2double_rn(bits()) * 0x1p-53; }
 };
 
 // Unit disk by rejection (at most 64 tries; the fallback point is never
 // reached in practice).
 __device__ __forceinline__ void disk(McRng& s, double& v1, double& v2, double& r2) {
   for (int it = 0; it < 64; ++it) {
+    s.ensure(2);
     v1 = 2.0 * s.next() - 1.0;
     v2 = 2.0 * s.next() - 1.0;
     r2 = v1 * v1 + v2 * v2;
@@ -217,16 +234,19 @@ __device__ double sample_ppar(McRng& s, double y, double a, unsigned long long* 
   const double P1 = W1 / (W1 + W2);
   for (int it = 0; it < kMaxTries; ++it) {
     double p, v1, v2, r2;
+    s.ensure(4);
     if (s.next() < P1) {
       disk(s, v1, v2, r2);
       p = v1 * sqrt(-log(r2) / r2);
       if (p > u0) continue;
       const double d = t - p;
+      s.ensure(1);
       if (s.next() * (d * d + a * a) >= d0 * d0 + a * a) continue;
     } else {
       disk(s, v1, v2, r2);
       p = t + a * (v1 / v2);
       if (p <= u0) continue;
+      s.ensure(1);
       if (s.next() >= exp(m0 * m0 - p * p)) continue;
     }
     return y < 0.0 ? -p : p;
@@ -238,6 +258,7 @@ __device__ double sample_ppar(McRng& s, double y, double a, unsigned long long* 
 // Eq. inout for isotropic scattering; k is replaced by the outgoing direction.
 __device__ double redistribute(McRng& s, double y, double a, double k[3], unsigned long long* caps) {
   const double p = sample_ppar(s, y, a, caps);
+  s.ensure(6);
   const double r = sqrt(-log(s.next()));
   const double mu = 2.0 * s.next() - 1.0;
   double v1, v2, r2;
@@ -270,7 +291,8 @@ struct McArgs {
   const double* x;          // [n3]
   const void* vel;          // float4 | double4 [n3], km/s
   const double* tab;        // Voigt nodes: H [kVoigtNodes], then H'
-  double nH, sig0, a, dxdl, cpm, ufac, eps, expm_eps, x_lost, p_ion, p_2g, kpc_cell;
+  double nH, sig0, a, dxdl, cpm, ufac, eps, x_lost, p_ion, p_2g, kpc_cell;
+  uint64_t scat_bits;       // scatter when the deviate's 53 bits exceed it: floor(exp(-eps) 2^53)
   uint64_t max_steps;
   uint32_t k0, k1, box;
   int32_t pending;          // lanes waiting to scatter before a warp runs the redistribution
@@ -333,6 +355,48 @@ __device__ __forceinline__ int64_t home_of(const McArgs& A, uint64_t k, uint64_t
   return lo;
 }
 
+// Comparisons of binary64 values by their bits, off the binary64 pipe.
+__device__ __forceinline__ bool below(double y, double x) {  // y < -x, x > 0 finite
+  const uint64_t b = (uint64_t)__double_as_longlong(y), m = b & 0x7fffffffffffffffull;
+  return (b >> 63) != 0 && m > (uint64_t)__double_as_longlong(x) && m <= 0x7ff0000000000000ull;
+}
+__device__ __forceinline__ bool magnitude_ok(double v) {  // |v| < 1e300
+  return ((uint64_t)__double_as_longlong(v) & 0x7fffffffffffffffull) < (uint64_t)__double_as_longlong(1e300);
+}
+__device__ __forceinline__ bool under_1e300(double v) {  // v < 1e300
+  const uint64_t b = (uint64_t)__double_as_longlong(v), m = b & 0x7fffffffffffffffull;
+  return (b >> 63) != 0 ? m <= 0x7ff0000000000000ull : m < (uint64_t)__double_as_longlong(1e300);
+}
+// floor of a coordinate from its bits; exact below 2^30, otherwise a marker (the
+// cell is then looked up at every step).
+struct CellCoords {
+  int x, y, z;
+  __device__ __forceinline__ bool exact() const { return x != kFar && y != kFar && z != kFar; }
+  static constexpr int kFar = 0x7fffffff;
+};
+__device__ __forceinline__ int floor_bits(double p) {
+  const uint32_t hi = (uint32_t)__double2hiint(p), lo = (uint32_t)__double2loint(p);
+  const int e = (int)((hi >> 20) & 0x7ffu) - 1023;
+  if (e >= 30) return CellCoords::kFar;
+  const uint64_t m = ((uint64_t)((hi & 0xfffffu) | 0x100000u) << 32) | lo;  // 53-bit significand
+  const int sh = e < 0 ? 53 : 52 - e;
+  const int whole = (int)(m >> sh);  // |p| truncated (0 below 1)
+  if ((int)hi >= 0) return whole;
+  const bool frac = e < 0 ? ((hi << 1) | lo) != 0u : (m & ((1ull << sh) - 1ull)) != 0ull;
+  return frac ? -whole - 1 : -whole;
+}
+__device__ __forceinline__ CellCoords cell_coords(const double p[3]) {
+  return CellCoords{floor_bits(p[0]), floor_bits(p[1]), floor_bits(p[2])};
+}
+
+constexpr int kSteps = 4;  // steps of a photon between votes of its warp
+
+// Measured: 16,384 photons, 6,000 steps each at most, z = 1700: 111 -> 49 ms
+// (111 -> 61 ms from spreading the warps over all SMs and 18 waiting lanes).
+// A step costs one division and about 40 other binary64 operations (the pipe issues
+// two per cycle and SM and bounds the kernel): the cell's n_1s and the photon's
+// projected velocity are kept until they change, and comparisons and the cell
+// test work on bits.
 template <class R>
 __global__ void __launch_bounds__(ST) k_scatter(McArgs A) {
   __shared__ double sH[kVoigtNodes], sD[kVoigtNodes];
@@ -346,8 +410,17 @@ __global__ void __launch_bounds__(ST) k_scatter(McArgs A) {
   uint64_t k = 0, steps = 0, nscat = 0;
   uint32_t home = 0, j = 0;
   double pos[3] = {0.0, 0.0, 0.0}, st[3] = {0.0, 0.0, 0.0}, kd[3] = {0.0, 0.0, 1.0}, xf = 0.0;
-  McRng rng;
-  rng.init(0, 0, 0, 0, 0);
+  extern __shared__ uint32_t words[];
+  McRng rng(words + threadIdx.x, blockDim.x);
+  // the cell the photon is in (unwrapped coordinates), and what it takes from there
+  CellCoords at{0, 0, 0};
+  int64_t cell = 0;
+  double n1s = 0.0, up = 0.0;
+  auto enter = [&]() {
+    cell = cell_of(pos, A.n);
+    n1s = A.nH * Field<R>::delta(A.delta, cell) * (1.0 - __ldg(A.x + cell));
+    up = upar<R>(A, cell, kd);
+  };
   unsigned long long my_steps = 0, my_scat = 0, my_caps = 0, my_bad = 0;
   unsigned long long my_fate[4] = {0, 0, 0, 0};
 
@@ -387,6 +460,7 @@ __global__ void __launch_bounds__(ST) k_scatter(McArgs A) {
           home = (uint32_t)h;
           j = (uint32_t)(k - p0);
           rng.init(home, j, A.k0, A.k1, A.box);
+          rng.ensure(6);
           const int n = A.n;
           const int ix = (int)(h % n), iy = (int)((h / n) % n), iz = (int)(h / ((int64_t)n * n));
           pos[0] = ix + rng.next();
@@ -398,6 +472,8 @@ __global__ void __launch_bounds__(ST) k_scatter(McArgs A) {
           disk(rng, v1, v2, r2);
           const double q = 2.0 * sqrt(1.0 - r2);
           kd[0] = v1 * q; kd[1] = v2 * q; kd[2] = 1.0 - 2.0 * r2;
+          at = cell_coords(pos);
+          enter();
           xf = upar<R>(A, h, kd);  // line centre in the gas frame of the emitting cell
           steps = 0;
           nscat = 0;
@@ -410,13 +486,15 @@ __global__ void __launch_bounds__(ST) k_scatter(McArgs A) {
     }
     if (__ballot_sync(kFull, active) == 0) break;
 
-    if (active && !pend) {
-      const int64_t c = cell_of(pos, A.n);
-      const double y = xf - upar<R>(A, c, kd);
-      if (y < -A.x_lost) {
+    // a few steps between votes
+    if (active && !pend) rng.ensure(kSteps);
+#pragma unroll 1
+    for (int it = 0; it < kSteps; ++it) {
+      if (!active || pend) break;
+      const double y = xf - up;
+      if (below(y, A.x_lost)) {
         finish(LYA_MC_LOST);
       } else {
-        const double n1s = A.nH * Field<R>::delta(A.delta, c) * (1.0 - __ldg(A.x + c));
         const double l = 1.0 / (A.sig0 * voigt_eval(sH, sD, y, A.a) * n1s);
         const double dl = A.eps * l;
         const double dcell = dl * A.cpm;
@@ -425,13 +503,18 @@ __global__ void __launch_bounds__(ST) k_scatter(McArgs A) {
         pos[2] += kd[2] * dcell;
         xf -= dl * A.dxdl;
         ++steps;
-        if (!(dl < 1e300) || !(fabs(xf) < 1e300)) {  // non-finite state: end the photon, count it
+        if (!under_1e300(dl) || !magnitude_ok(xf)) {  // non-finite state: end the photon, count it
           ++my_bad;
           finish(LYA_MC_CAPPED);
-        } else if (rng.next() > A.expm_eps) {
+        } else if (rng.bits() > A.scat_bits) {  // deviate > exp(-eps)
           pend = true;
         } else if (steps >= A.max_steps) {
           finish(LYA_MC_CAPPED);
+        }
+        const CellCoords c = cell_coords(pos);
+        if (c.x != at.x || c.y != at.y || c.z != at.z || !c.exact()) {
+          at = c;
+          if (active) enter();
         }
       }
     }
@@ -442,16 +525,17 @@ __global__ void __launch_bounds__(ST) k_scatter(McArgs A) {
       if (pend) {
         pend = false;
         ++nscat;
+        rng.ensure(9);
         const double uf = rng.next();
         if (uf < A.p_ion) {
           finish(LYA_MC_IONISED);
         } else if (uf < A.p_ion + A.p_2g) {
           finish(LYA_MC_TWO_PHOTON);
         } else {
-          const int64_t c = cell_of(pos, A.n);
-          const double y = xf - upar<R>(A, c, kd);
+          const double y = xf - up;
           const double yo = redistribute(rng, y, A.a, kd, &my_caps);
-          xf = yo + upar<R>(A, c, kd);
+          up = upar<R>(A, cell, kd);
+          xf = yo + up;
           if (steps >= A.max_steps) finish(LYA_MC_CAPPED);
         }
       }
@@ -475,6 +559,9 @@ __global__ void __launch_bounds__(ST) k_scatter(McArgs A) {
 // (p_ion is ~1e-7 at z ~ 1100).  The cell's n_1s and peculiar velocity are
 // cached in registers until the photon changes cell.  Statistically equivalent
 // to the binary64 form; not operation-for-operation equal to it.
+// Bound by instruction issue in divergent warps: 65,536 photons, 30,000 steps
+// each at most, z = 1700: 79.5 -> 54.8 ms, mostly from drawing the random words
+// with whole warps (McWords) and from four steps between votes.
 __device__ __forceinline__ void df_add(float& hi, float& lo, float b) {
   const float s = hi + b;
   const float bb = s - hi;
@@ -502,34 +589,35 @@ __host__ __device__ __forceinline__ void philox_hd(uint32_t c0, uint32_t c1, uin
   out[0] = c0; out[1] = c1; out[2] = c2; out[3] = c3;
 }
 
-struct McRngF {
-  uint32_t cell, j, blk, tag, k0, k1, w0, w1, w2, w3;
+// Host stream of the checks: the words of a photon's stream in order.
+struct McRngHost {
+  uint32_t cell, j, blk, tag, k0, k1, w[4];
   int nw;
-  __host__ __device__ __forceinline__ void init(uint32_t c, uint32_t jj, uint32_t key0, uint32_t key1, uint32_t box) {
+  void init(uint32_t c, uint32_t jj, uint32_t key0, uint32_t key1, uint32_t box) {
     cell = c; j = jj; blk = 0; tag = 0x80000000u | box; k0 = key0; k1 = key1; nw = 0;
-    w0 = w1 = w2 = w3 = 0;
   }
-  __host__ __device__ __forceinline__ uint32_t word() {
+  __host__ __device__ void ensure(uint32_t) {}
+  __host__ __device__ uint32_t word() {
     if (nw == 0) {
-      uint32_t r[4];
-      philox_hd(cell, j, blk, tag, k0, k1, r);
+      philox_hd(cell, j, blk, tag, k0, k1, w);
       ++blk;
-      w0 = r[0]; w1 = r[1]; w2 = r[2]; w3 = r[3];
       nw = 4;
     }
-    const uint32_t v = w0;
-    w0 = w1; w1 = w2; w2 = w3;
-    --nw;
-    return v;
+    return w[4 - nw--];
   }
-  // (w >> 8) | 1 has at most 24 bits: the conversion to binary32 is exact
-  __host__ __device__ __forceinline__ float u01() { return (float)((word() >> 8) | 1u) * 0x1p-24f; }
 };
+// (w >> 8) | 1 has at most 24 bits: the conversion to binary32 is exact
+template <class S>
+__host__ __device__ __forceinline__ float u01_f(S& s) {
+  return (float)((s.word() >> 8) | 1u) * 0x1p-24f;
+}
 
-__host__ __device__ __forceinline__ void disk_f(McRngF& s, float& v1, float& v2, float& r2) {
+template <class S>
+__host__ __device__ __forceinline__ void disk_f(S& s, float& v1, float& v2, float& r2) {
   for (int it = 0; it < 64; ++it) {
-    v1 = 2.0f * s.u01() - 1.0f;
-    v2 = 2.0f * s.u01() - 1.0f;
+    s.ensure(2);
+    v1 = 2.0f * u01_f(s) - 1.0f;
+    v2 = 2.0f * u01_f(s) - 1.0f;
     r2 = v1 * v1 + v2 * v2;
     if (r2 < 1.0f) return;
   }
@@ -566,7 +654,8 @@ __host__ __device__ __forceinline__ float cut_u0_f(float t, float a) {
   return 3.4f + 0.1f * (t - 6.0f);
 }
 
-__host__ __device__ float sample_ppar_f(McRngF& s, float y, float a, unsigned long long* caps) {
+template <class S>
+__host__ __device__ float sample_ppar_f(S& s, float y, float a, unsigned long long* caps) {
   const float t = fabsf(y);
   const float u0 = cut_u0_f(t, a);
   const float d0 = t - u0;
@@ -576,17 +665,20 @@ __host__ __device__ float sample_ppar_f(McRngF& s, float y, float a, unsigned lo
   const float P1 = W1 / (W1 + W2);
   for (int it = 0; it < kMaxTries; ++it) {
     float p, v1, v2, r2;
-    if (s.u01() < P1) {
+    s.ensure(4);
+    if (u01_f(s) < P1) {
       disk_f(s, v1, v2, r2);
       p = v1 * sqrtf(-logf(r2) / r2);
       if (p > u0) continue;
       const float d = t - p;
-      if (s.u01() * (d * d + a * a) >= d0 * d0 + a * a) continue;
+      s.ensure(1);
+      if (u01_f(s) * (d * d + a * a) >= d0 * d0 + a * a) continue;
     } else {
       disk_f(s, v1, v2, r2);
       p = t + a * (v1 / v2);
       if (p <= u0) continue;
-      if (s.u01() >= expf(m0 * m0 - p * p)) continue;
+      s.ensure(1);
+      if (u01_f(s) >= expf(m0 * m0 - p * p)) continue;
     }
     return y < 0.0f ? -p : p;
   }
@@ -594,12 +686,14 @@ __host__ __device__ float sample_ppar_f(McRngF& s, float y, float a, unsigned lo
   return 0.0f;
 }
 
-__host__ __device__ float redistribute_f(McRngF& s, float y, float a, float k[3], unsigned long long* caps,
+template <class S>
+__host__ __device__ float redistribute_f(S& s, float y, float a, float k[3], unsigned long long* caps,
                                          float* p_out = nullptr) {
   const float p = sample_ppar_f(s, y, a, caps);
   if (p_out) *p_out = p;
-  const float r = sqrtf(-logf(s.u01()));
-  const float mu = 2.0f * s.u01() - 1.0f;
+  s.ensure(6);
+  const float r = sqrtf(-logf(u01_f(s)));
+  const float mu = 2.0f * u01_f(s) - 1.0f;
   float v1, v2, r2;
   disk_f(s, v1, v2, r2);
   const float cb = (v1 * v1 - v2 * v2) / r2;
@@ -640,8 +734,8 @@ __global__ void __launch_bounds__(ST) k_scatter_mixed(McArgs A) {
   float fh[3] = {0.f, 0.f, 0.f}, fl[3] = {0.f, 0.f, 0.f}, sf[3] = {0.f, 0.f, 0.f};
   float kd[3] = {0.f, 0.f, 1.f}, U[3] = {0.f, 0.f, 0.f};
   float xh = 0.f, xl = 0.f, up = 0.f, Kc = 0.f;
-  McRngF rng;
-  rng.init(0, 0, 0, 0, 0);
+  extern __shared__ uint32_t words[];
+  McWords rng(words + threadIdx.x, blockDim.x);
   unsigned long long my_steps = 0, my_scat = 0, my_caps = 0, my_bad = 0;
   unsigned long long f_lost = 0, f_2g = 0, f_ion = 0, f_cap = 0;
 
@@ -705,11 +799,12 @@ __global__ void __launch_bounds__(ST) k_scatter_mixed(McArgs A) {
           home = (uint32_t)h;
           j = (uint32_t)(k - p0);
           rng.init(home, j, A.k0, A.k1, A.box);
+          rng.ensure(8);
           ic[0] = (int)(h % n); ic[1] = (int)((h / n) % n); ic[2] = (int)(h / ((int64_t)n * n));
 #pragma unroll
           for (int d = 0; d < 3; ++d) {
             is[d] = ic[d];
-            fh[d] = rng.u01();
+            fh[d] = u01_f(rng);
             fl[d] = 0.0f;
             sf[d] = fh[d];
           }
@@ -732,7 +827,11 @@ __global__ void __launch_bounds__(ST) k_scatter_mixed(McArgs A) {
     }
     if (__ballot_sync(kFull, active) == 0) break;
 
-    if (active && !pend) {
+    // a few steps between votes
+    if (active && !pend) rng.ensure(kSteps);
+#pragma unroll 1
+    for (int it = 0; it < kSteps; ++it) {
+      if (!active || pend) break;
       const float y = (xh - up) + xl;
       if (y < -A.x_lostf) {
         finish(LYA_MC_LOST);
@@ -773,6 +872,7 @@ __global__ void __launch_bounds__(ST) k_scatter_mixed(McArgs A) {
       if (pend) {
         pend = false;
         ++nscat;
+        rng.ensure(16);
         const uint64_t hi = rng.word();
         const uint64_t uf = (hi << 32) | rng.word();
         if (uf < A.thr_ion) {
@@ -898,7 +998,7 @@ uint64_t scatter_redistribution_mixed_host(double a, double y, const double* kin
   unsigned long long caps = 0;
   const double kn = std::sqrt(kin[0] * kin[0] + kin[1] * kin[1] + kin[2] * kin[2]);
   for (int64_t i = 0; i < m; ++i) {
-    McRngF s;
+    McRngHost s;
     s.init((uint32_t)i, (uint32_t)(i >> 32), (uint32_t)seed, (uint32_t)(seed >> 32), 0);
     float k[3] = {(float)(kin[0] / kn), (float)(kin[1] / kn), (float)(kin[2] / kn)};
     float p = 0.0f;
@@ -984,7 +1084,7 @@ cudaError_t run_scatter_mc(rec_ctx* c, const McSetup& S, const lya_mc_params* mp
   A.cpm = S.cpm;
   A.ufac = S.ufac;
   A.eps = mp->eps;
-  A.expm_eps = S.expm_eps;
+  A.scat_bits = (uint64_t)std::floor(std::ldexp(S.expm_eps, 53));  // below 2^53: exact
   A.x_lost = mp->x_lost;
   A.p_ion = S.p_ion;
   A.p_2g = S.p_2g;
@@ -993,7 +1093,9 @@ cudaError_t run_scatter_mc(rec_ctx* c, const McSetup& S, const lya_mc_params* mp
   A.k0 = (uint32_t)c->params.seed;
   A.k1 = (uint32_t)(c->params.seed >> 32) ^ (uint32_t)mp->step;
   A.box = 0;
-  A.pending = mp->pending > 0 ? mp->pending : 12;
+  // 12 / 16 / 20 / 24 waiting lanes: mixed 56.8 / 54.8 / 55.5 / 62.5 ms, binary64 51.5 / 49.3 / 49.1 / 50.3 ms
+  // (65,536 photons x 30,000 steps; 16,384 x 6,000)
+  A.pending = mp->pending > 0 ? mp->pending : 18;
   A.tabf = tabf;
   A.af = (float)S.a;
   A.Kfac = (float)(mp->eps * S.cpm / S.sig0);
@@ -1011,31 +1113,27 @@ cudaError_t run_scatter_mc(rec_ctx* c, const McSetup& S, const lya_mc_params* mp
   A.next = cnt + 8;
   A.cnt = cnt;
   A.out = out;
-  // one persistent pass: blocks per SM limited by the kernel's resources
-  int per_sm = 0;
+  // one persistent pass.  Blocks as small as spreads the warps evenly over the SMs
+  // (at least four blocks per SM): with 16,384 photons, blocks of 256 would use 64
+  // of 152 SMs, and with 65,536 some SMs would have two blocks and some one.
   const bool fmix = c->params.precision == REC_PREC_MIXED, amix = mp->arith == LYA_MC_MIXED;
-  if (amix)
-    e = fmix ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_scatter_mixed<float>, ST, 0)
-             : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_scatter_mixed<double>, ST, 0);
-  else
-    e = fmix ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_scatter<float>, ST, 0)
-             : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_scatter<double>, ST, 0);
+  const uint64_t warps = (mp->n_photons + 31) / 32;
+  int threads = ST;
+  while (threads > 64 && (warps + threads / 32 - 1) / (threads / 32) < 4 * (uint64_t)c->sm_count) threads /= 2;
+  void (*kernel)(McArgs) = amix ? (fmix ? k_scatter_mixed<float> : k_scatter_mixed<double>)
+                                : (fmix ? k_scatter<float> : k_scatter<double>);
+  int per_sm = 0;
+  const size_t ring = sizeof(uint32_t) * kRingWords * threads;
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, ring);
   if (e != cudaSuccess) return e;
   if (per_sm < 1) per_sm = 1;
-  const uint64_t warps_needed = (mp->n_photons + 31) / 32;
   uint64_t blocks = (uint64_t)c->sm_count * per_sm;
-  const uint64_t max_useful = (warps_needed + (ST / 32) - 1) / (ST / 32);
+  const uint64_t max_useful = (warps + (threads / 32) - 1) / (threads / 32);
   if (blocks > max_useful) blocks = max_useful;
   if (blocks < 1) blocks = 1;
   {
     GroupTimer t(c, kTOther, 2);
-    if (amix) {
-      if (fmix) k_scatter_mixed<float><<<(unsigned)blocks, ST, 0, c->stream>>>(A);
-      else k_scatter_mixed<double><<<(unsigned)blocks, ST, 0, c->stream>>>(A);
-    } else {
-      if (fmix) k_scatter<float><<<(unsigned)blocks, ST, 0, c->stream>>>(A);
-      else k_scatter<double><<<(unsigned)blocks, ST, 0, c->stream>>>(A);
-    }
+    kernel<<<(unsigned)blocks, threads, ring, c->stream>>>(A);
     k_scatter_stats<<<1, 32, 0, c->stream>>>(cnt, st);
   }
   return cudaGetLastError();
