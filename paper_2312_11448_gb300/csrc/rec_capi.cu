@@ -71,6 +71,16 @@ rec_status check_box(const rec_box& b, std::string* why) {
   return REC_OK;
 }
 
+// Leading intervals of the emission-profile table from which the interpolated
+// frequency is <= 0 whatever the rounding, in the working precision of the transport.
+int early_nodes(const rec_params& p) {
+  const bool mixed = p.precision == REC_PREC_MIXED;
+  auto q = [&](int i) { return mixed ? (double)(float)p.emission_quantiles[i] : p.emission_quantiles[i]; };
+  int k = 0;
+  while (k + 1 < p.n_quantiles && (q(k + 1) == 0.0 || q(k + 1) <= -0x1p-20 * std::fabs(q(k)))) ++k;
+  return k;
+}
+
 size_t round_up(size_t v, size_t m) { return (v + m - 1) / m * m; }
 
 rec_tuning default_tuning(bool mixed, bool batch, uint64_t packets, int sm_count) {
@@ -133,6 +143,7 @@ rec_status init_batch(const rec_params* params, const rec_box* boxes, int32_t n_
   rec_ctx* c = new (std::nothrow) rec_ctx();
   if (!c) return fail(nullptr, REC_ENOMEM, "host allocation failed");
   c->params = *params;
+  c->early_nodes = early_nodes(*params);
   c->params.emission_quantiles = nullptr;
   c->box = boxes[0];
   c->boxes.assign(boxes, boxes + n_boxes);
@@ -280,6 +291,7 @@ rec_status rec_init(const rec_params* params, const rec_box* boxes, int32_t n_bo
   rec_ctx* c = new (std::nothrow) rec_ctx();
   if (!c) return fail(nullptr, REC_ENOMEM, "host allocation failed");
   c->params = *params;
+  c->early_nodes = early_nodes(*params);
   c->params.emission_quantiles = nullptr;  // copied to the device below
   c->box = b;
   c->stream = (cudaStream_t)cuda_stream;

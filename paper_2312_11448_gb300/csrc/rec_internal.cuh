@@ -164,6 +164,7 @@ struct rec_ctx {
   unsigned long long* cpre;  // first march chunk of each bucket [super-tiles + 1]
   uint32_t* velq = nullptr;  // compact velocity copy of the march (rec_velq.cuh); NULL: no memory for it
   unsigned long long* partQ; // allocation block sums / offsets [alloc blocks]
+  int early_nodes = 0;       // leading nodes of the emission-profile table with xi <= 0 (see early_word)
   void* quant;               // emission-profile table (float or double) [n_quantiles]
   int grid;                  // blocks of the streaming passes
   int alloc_blocks;

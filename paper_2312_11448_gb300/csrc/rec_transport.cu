@@ -29,6 +29,7 @@
 // intrinsics (never contracted into FMA), in binary32 for the mixed form and
 // binary64 for the FP64 form, so its integer results are reproducible.
 
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 
@@ -118,9 +119,11 @@ constexpr uint32_t kAllocBlock = 0x000A110Cu;  // counter block of the allocatio
 __device__ __forceinline__ float u01f(uint32_t r) {
   return __fsub_rn(__uint_as_float(0x3f800000u | (r >> 9)), 0x1.fffffep-1f);
 }
+// Binary64: the same with the top 52 bits of the word pair, 1 + m 2^-52 minus 1 - 2^-53:
+// one operation on the binary64 pipe (a conversion and a product before).
 __device__ __forceinline__ double u01d(uint32_t lo, uint32_t hi) {
-  uint64_t w = ((uint64_t)hi << 32) | lo;
-  return __ull2double_rn((w >> 11) | 1ull) * 0x1p-53;
+  const uint64_t w = ((uint64_t)hi << 32) | lo;
+  return __dsub_rn(__longlong_as_double((long long)(0x3ff0000000000000ull | (w >> 12))), 0x1.fffffffffffffp-1);
 }
 
 // ---- explicitly rounded arithmetic -----------------------------------------------
@@ -156,6 +159,7 @@ template <> struct Draws<float> {
   // block 0: three cell offsets and the frequency quantile; blocks 1..16: two
   // direction pairs each
   static constexpr int kPairs = 2;
+  static constexpr uint32_t kQuantBlock = 0;  // its last word leads the quantile's bits
   template <class S>
   static __device__ __forceinline__ void position(const S& s, uint32_t c, uint32_t j, float f[3], float* uq) {
     U4 r = draw(s, c, j, 0u);
@@ -176,6 +180,7 @@ template <> struct Draws<double> {
   // blocks 0, 1: three cell offsets and the quantile (two words per deviate);
   // blocks 2..33: one direction pair each
   static constexpr int kPairs = 1;
+  static constexpr uint32_t kQuantBlock = 1;
   template <class S>
   static __device__ __forceinline__ void position(const S& s, uint32_t c, uint32_t j, double f[3], double* uq) {
     U4 r = draw(s, c, j, 0u), q = draw(s, c, j, 1u);
@@ -672,6 +677,7 @@ struct TransportArgs {
   R kappa, cth;
   Stream strm;
   Keys ks;  // round keys of strm (emission)
+  uint32_t early;  // packets whose quantile word is below it have xi <= 0 (early_word)
   uint32_t* tally;
   DevScalars* sc;
   typename Vec4<R>::T* queue;  // 3 entries per queued packet
@@ -748,6 +754,12 @@ struct Ray {
   int sx, sy, sz;
 };
 
+__device__ __forceinline__ int step_sign(float v) { return (v > 0.0f) - (v < 0.0f); }
+__device__ __forceinline__ int step_sign(double v) {  // by the bits
+  const uint32_t hi = (uint32_t)__double2hiint(v), lo = (uint32_t)__double2loint(v);
+  return ((hi & 0x7fffffffu) | lo) == 0u ? 0 : ((int)hi < 0 ? -1 : 1);
+}
+
 // tDelta and step of one axis from the direction cosine (Amanatides-Woo).
 template <class R>
 // Written without branches: 1/|n_d| correctly rounded (the same value as the
@@ -755,7 +767,7 @@ template <class R>
 // crossed.
 __device__ __forceinline__ void axis_setup(R nd, R* tD, int* st) {
   using A = Ar<R>;
-  *st = (nd > (R)0) - (nd < (R)0);
+  *st = step_sign(nd);
   *tD = A::rcp(fabs(nd));
 }
 
@@ -771,12 +783,16 @@ __device__ __forceinline__ uint32_t wrap_step(uint32_t i, int s, uint32_t n) {
   return s > 0 ? (i + 1 == n ? 0 : i + 1) : (i == 0 ? n - 1 : i - 1);
 }
 
+// Order of two positive numbers or +inf; binary64 by the bits, off the binary64 pipe.
+__device__ __forceinline__ bool le_pos(float a, float b) { return a <= b; }
+__device__ __forceinline__ bool le_pos(double a, double b) { return __double_as_longlong(a) <= __double_as_longlong(b); }
+
 // Path length along the ray at which the packet leaves its current cell: the
 // nearest face, ties broken x < y < z.
 template <class R>
 __device__ __forceinline__ R dda_exit(const Ray<R>& r, bool* ax0, bool* ax1, bool* ax2) {
-  *ax0 = r.tMx <= r.tMy && r.tMx <= r.tMz;
-  *ax1 = !*ax0 && r.tMy <= r.tMz;
+  *ax0 = le_pos(r.tMx, r.tMy) && le_pos(r.tMx, r.tMz);
+  *ax1 = !*ax0 && le_pos(r.tMy, r.tMz);
   *ax2 = !*ax0 && !*ax1;
   return *ax0 ? r.tMx : (*ax1 ? r.tMy : r.tMz);
 }
@@ -786,22 +802,6 @@ template <class R, class V>
 __device__ __forceinline__ R doppler(const Ray<R>& r, const V& U) {
   using A = Ar<R>;
   return A::add(A::add(A::mul(r.knx, U.x), A::mul(r.kny, U.y)), A::mul(r.knz, U.z));
-}
-
-template <class R, bool P2>
-__device__ __forceinline__ void dda_advance(Ray<R>& r, bool ax0, bool ax1, bool ax2, R s_exit, uint32_t n);
-
-template <class R, bool P2 = false, class V>
-__device__ __forceinline__ int march_cell(Ray<R>& r, const V& Uc, uint32_t n) {
-  using A = Ar<R>;
-  R dc = doppler(r, Uc);
-  bool ax0, ax1, ax2;
-  const R s_exit = dda_exit(r, &ax0, &ax1, &ax2);
-  // resonance in this cell at path length u0 - kappa n.U_c: absorb unless beyond the exit
-  if (A::sub(r.u0, dc) <= s_exit) return 1;
-  if (r.kc >= kMaxCrossings) return 2;
-  dda_advance<R, P2>(r, ax0, ax1, ax2, s_exit, n);
-  return 0;
 }
 
 // The step across the exit face: periodic neighbour along the exit axis and
@@ -896,6 +896,7 @@ struct EmitBox {
   uint32_t box;  // fourth Philox counter word
   Tiles tl;
   uint32_t bk0;
+  uint32_t early;  // TransportArgs::early, or 0 where the box's velocities are not all finite
 };
 
 // Emission of one packet, in three parts: the cell of each of a warp's 32
@@ -904,11 +905,14 @@ struct EmitBox {
 // resonance test in the home cell, the home tally or the queue entry.
 
 // Cell and index within the cell of packet base + lane (< N): the coarse index
-// gives the cell of the warp's first packet, then a 32-cell window of the
-// packet prefix resolves the rest with shuffles.
+// gives the cell c0 of the warp's first packet, and the prefix values of the 32 cells
+// after it, those below base + 32, mark where in the warp a new cell begins (bit s of
+// *starts for a cell that begins at packet base + s; at[s], shared memory of the
+// warp, names it).  The packets of a cell are neighbouring lanes: *starts also
+// groups the warp by cells, if *whole (no packet lies beyond those 32 cells).
 template <class R, bool FRESH>
-__device__ __forceinline__ bool emit_locate(const EmitBox<R>& e, uint32_t base, uint32_t N, uint32_t* cell_out,
-                                            uint32_t* j_out) {
+__device__ __forceinline__ bool emit_locate(const EmitBox<R>& e, uint32_t base, uint32_t N, uint32_t* at,
+                                            uint32_t* cell_out, uint32_t* j_out, uint32_t* starts, bool* whole) {
   const int lane = threadIdx.x & 31;
   const uint32_t n3 = e.n3;
   const uint32_t p = base + lane;
@@ -917,42 +921,64 @@ __device__ __forceinline__ bool emit_locate(const EmitBox<R>& e, uint32_t base, 
   const uint32_t Pc0 = ld_index<FRESH>(e.P + c0);
   const uint32_t widx = c0 + 1u + lane;
   const uint32_t wv = (widx <= n3) ? ld_index<FRESH>(e.P + widx) : 0xffffffffu;
-  // off = number of window entries <= p (the window is sorted): binary search
-  // over the 32 lane values with shuffles
-  uint32_t off = 0;
-#pragma unroll
-  for (uint32_t step = 16; step > 0; step >>= 1) {
-    const uint32_t probe = __shfl_sync(0xffffffffu, wv, (off + step - 1u) & 31u);
-    if (probe <= p) off += step;
-  }
-  const uint32_t w31 = __shfl_sync(0xffffffffu, wv, 31);  // every lane takes part
-  if (off == 31u && w31 <= p) off = 32u;
-  const uint32_t prev = __shfl_sync(0xffffffffu, wv, (off > 0 ? off - 1u : 0u) & 31u);
-  uint32_t cell = c0 + off, Pc = (off == 0) ? Pc0 : prev;
-  if (act && off >= 32) {
+  const uint32_t next = __shfl_down_sync(0xffffffffu, wv, 1);
+  const uint32_t s = wv - base;  // >= 1: the warp's first packet lies in c0
+  const uint32_t m = __reduce_or_sync(0xffffffffu, s < 32u ? 1u << s : 0u);
+  __syncwarp();  // at is read no more
+  if (s < 32u && (lane == 31 || next != wv)) at[s] = (uint32_t)lane + 1u;  // the last of the cells that begin there
+  __syncwarp();
+  const uint32_t mine = m & (0xffffffffu >> (31 - lane));
+  const uint32_t b = 31u - (uint32_t)__clz((int)mine);  // where the packet's cell begins
+  const uint32_t off = mine ? at[b & 31u] : 0u;
+  uint32_t cell = c0 + off, j = mine ? (uint32_t)lane - b : p - Pc0;
+  *whole = !__any_sync(0xffffffffu, act && off == 32u);
+  if (act && off == 32u) {
     cell = upper_bound<FRESH>(e.P, c0 + 32u, n3, p) - 1u;
-    Pc = ld_index<FRESH>(e.P + cell);
+    j = p - ld_index<FRESH>(e.P + cell);
   }
   *cell_out = cell;
-  *j_out = p - Pc;
+  *j_out = j;
+  *starts = m;
   return act;
 }
 
-// (1) injection point uniform in the cell (Philox block 0, which also holds the
-// frequency quantile), the emission frequency from the tabulated inverse CDF
-// and the thermal speed in cells.
+// Lanes of the group of neighbouring lanes that a lane belongs to, from the
+// lanes where groups start (lane 0 always starts one).
+__device__ __forceinline__ unsigned lane_group(uint32_t starts) {
+  const int lane = threadIdx.x & 31;
+  const uint32_t upto = 0xffffffffu >> (31 - lane);
+  const uint32_t low = (starts | 1u) & upto, high = starts & ~upto;
+  const uint32_t from = 0xffffffffu << (31 - __clz((int)low));
+  return from & (high ? (high & (0u - high)) - 1u : 0xffffffffu);
+}
+// The same from keys: neighbouring lanes with equal keys.
+__device__ __forceinline__ unsigned key_group(uint32_t key) {
+  const uint32_t before = __shfl_up_sync(0xffffffffu, key, 1);
+  return lane_group(__ballot_sync(0xffffffffu, key != before));
+}
+
+// (1) the emission frequency from the tabulated inverse CDF at the packet's
+// quantile, and the thermal speed in cells.
 template <class R>
-__device__ __forceinline__ void emit_draw0(const TransportArgs<R>& a, const EmitBox<R>& e, uint32_t cell, uint32_t j,
-                                           R f[3], R* xi, R* vt) {
+__device__ __forceinline__ void emit_draw0(const TransportArgs<R>& a, const EmitBox<R>& e, uint32_t cell, R uq, R* xi,
+                                           R* vt) {
   using A = Ar<R>;
-  R uq;
-  Draws<R>::position(KStream{a.ks, e.box}, cell, j, f, &uq);
   R tq = A::mul(uq, (R)(a.M - 1));
   int k;
   const R fr = A::sub(tq, quant_node<R>(tq, a.M, &k));
   R q0 = __ldg(a.quant + k), q1 = __ldg(a.quant + k + 1);
   *xi = A::add(q0, A::mul(fr, A::sub(q1, q0)));
   *vt = A::sqr(A::mul(__ldg(e.T + cell), e.cth));
+}
+
+// 2 u - 1 (2 u is exact, so one rounding as in the separate operations), and
+// 0 < s < 1 for a sum of squares (binary64 by the bits).
+__device__ __forceinline__ float centred(float u) { return __fmaf_rn(2.0f, u, -1.0f); }
+__device__ __forceinline__ double centred(double u) { return __fma_rn(2.0, u, -1.0); }
+__device__ __forceinline__ bool in_disk(float s) { return s < 1.0f && s > 0.0f; }
+__device__ __forceinline__ bool in_disk(double s) {
+  const uint64_t b = (uint64_t)__double_as_longlong(s);
+  return b - 1u < 0x3ff0000000000000ull - 1u;
 }
 
 // The rest of a packet's emission (all lanes of the warp call it; lanes with
@@ -982,24 +1008,24 @@ __device__ __forceinline__ void emit_rest(const TransportArgs<R>& a, const EmitB
       typename Draws<R>::Block blk = Draws<R>::block(ks, cell, j, 0);
       R ua, ub;
       Draws<R>::pair_from(blk, 0, &ua, &ub);
-      R v1 = A::sub(A::mul(two, ua), one), v2 = A::sub(A::mul(two, ub), one);
+      R v1 = centred(ua), v2 = centred(ub);
       R s = A::add(A::mul(v1, v1), A::mul(v2, v2));
-      bool ok = s < one && s > zero;
+      bool ok = in_disk(s);
       int t = 1;
       if (Draws<R>::kPairs == 2) {  // the block's second pair
         Draws<R>::pair_from(blk, 1, &ua, &ub);
-        const R w1 = A::sub(A::mul(two, ua), one), w2 = A::sub(A::mul(two, ub), one);
+        const R w1 = centred(ua), w2 = centred(ub);
         const R sw = A::add(A::mul(w1, w1), A::mul(w2, w2));
-        if (!ok && sw < one && sw > zero) { v1 = w1; v2 = w2; s = sw; ok = true; }
+        if (!ok && in_disk(sw)) { v1 = w1; v2 = w2; s = sw; ok = true; }
         t = 2;
       }
       for (; !ok && t < 32; ++t) {
         if (Draws<R>::first_of_block(t)) blk = Draws<R>::block(ks, cell, j, t);
         Draws<R>::pair_from(blk, t, &ua, &ub);
-        v1 = A::sub(A::mul(two, ua), one);
-        v2 = A::sub(A::mul(two, ub), one);
+        v1 = centred(ua);
+        v2 = centred(ub);
         s = A::add(A::mul(v1, v1), A::mul(v2, v2));
-        ok = s < one && s > zero;
+        ok = in_disk(s);
       }
       if (ok) {
         R fac = A::mul(two, A::sqr(A::sub(one, s)));
@@ -1008,7 +1034,7 @@ __device__ __forceinline__ void emit_rest(const TransportArgs<R>& a, const EmitB
     }
     r.knx = A::mul(e.kappa, nx); r.kny = A::mul(e.kappa, ny); r.knz = A::mul(e.kappa, nz);
     V Uh = e.vel[cell];
-    R dh = A::add(A::add(A::mul(r.knx, Uh.x), A::mul(r.kny, Uh.y)), A::mul(r.knz, Uh.z));
+    const R dh = doppler(r, Uh);
     r.u0 = A::add(A::mul(xi, vt), dh);
     e.tl.template coords<P2>(cell, &r.ix, &r.iy, &r.iz);
     axis_setup<R>(nx, &r.tDx, &r.sx);
@@ -1020,21 +1046,25 @@ __device__ __forceinline__ void emit_rest(const TransportArgs<R>& a, const EmitB
     r.tMy = A::mul(r.sy < 0 ? f[1] : A::sub(one, f[1]), r.tDy);
     r.tMz = A::mul(r.sz < 0 ? f[2] : A::sub(one, f[2]), r.tDz);
     r.kc = 0;
-    int res = march_cell<R, P2>(r, Uh, n);  // home cell (res == 2 impossible with kc = 0)
-    home = res == 1;
-    queued = res == 0;
-    my_cross += r.kc;
+    // home cell: resonance at path length u0 - kappa n.U_home, absorb unless beyond the exit
+    bool ax0, ax1, ax2;
+    const R s_exit = dda_exit(r, &ax0, &ax1, &ax2);
+    home = A::sub(r.u0, dh) <= s_exit;
+    queued = !home;
     if (home) ++my_abs;
+    else {
+      dda_advance<R, P2>(r, ax0, ax1, ax2, s_exit, n);
+      ++my_cross;
+    }
   }
   // warp-aggregated tally of the packets resonant at home (mostly one cell per warp)
-  const uint32_t key = home ? cell : 0xffffffffu;
-  const unsigned m = __match_any_sync(0xffffffffu, key);
+  const unsigned m = key_group(cell) & __ballot_sync(0xffffffffu, home);
   if (home && lane == __ffs(m) - 1) atomicAdd(e.tally + cell, (uint32_t)__popc(m));
   // queue the others after their first step, in their home super-tile's bucket
   const unsigned qm = __ballot_sync(0xffffffffu, queued);
   if (qm) {
-    const uint32_t bk = queued ? e.bk0 + e.tl.template at<P2>(cell) : 0xffffffffu;
-    const unsigned gm = __match_any_sync(0xffffffffu, bk) & qm;
+    const uint32_t bk = e.bk0 + e.tl.template at<P2>(cell);
+    const unsigned gm = key_group(bk) & qm;
     unsigned long long qb = 0;
     const int leader = __ffs(gm) - 1;
     if (queued && lane == leader) qb = atomicAdd(&a.bfill[bk], (unsigned long long)__popc(gm));
@@ -1060,28 +1090,17 @@ __device__ __forceinline__ void emit_rest(const TransportArgs<R>& a, const EmitB
   }
 }
 
-// One warp emits the packets base .. base + 31 of one box (N packets).
-template <class R, bool P2, bool FRESH = false>
-__device__ __forceinline__ void emit_warp(const TransportArgs<R>& a, const EmitBox<R>& e, uint32_t base, uint32_t N,
-                                          uint64_t& my_abs, uint64_t& my_cross) {
-  uint32_t cell, j;
-  const bool act = emit_locate<R, FRESH>(e, base, N, &cell, &j);
-  R f[3] = {(R)0, (R)0, (R)0}, xi = (R)0, vt = (R)0;
-  if (act) emit_draw0<R>(a, e, cell, j, f, &xi, &vt);
-  emit_rest<R, P2>(a, e, act, cell, j, f, xi, vt, my_abs, my_cross);
-}
-
 // A packet emitted at or below the line centre (xi <= 0) is resonant in its
 // home cell whatever its direction: u0 - kappa n.U_home = (xi v_t + d) - d
 // with d = kappa n.U_home is <= 0 by the monotonicity of rounding, and the
 // exit distance is >= 0.  This holds exactly when xi v_t is not NaN (v_t
-// finite) and d is finite (|U| components <= 1e30 keep kappa n.U far from
-// overflow); such packets need no direction and are tallied at once.
-template <class R>
-__device__ __forceinline__ bool home_without_direction(R xi, R vt, const typename Vec4<R>::T& U) {
-  const R big = (R)1e30, vmax = sizeof(R) == 4 ? (R)3.4028234e38f : (R)1.7976931348623157e308;
-  return xi <= (R)0 && vt <= vmax && fabs(U.x) <= big && fabs(U.y) <= big && fabs(U.z) <= big;
-}
+// finite) and d is finite; such packets need no direction and are tallied at once.
+// - xi: the packet's quantile deviate u lies below a bound known to the host
+//   (early_word), so the word that leads u's bits decides, without the table.
+// - v_t = sqrt(T cth): T in [0, 1e15] by its bits, with cth <= 1e15 (early_word is 0 otherwise).
+// - d: the box's velocities are finite (EmitBox::early is 0 otherwise).
+__device__ __forceinline__ bool temperature_plain(float T) { return __float_as_uint(T) <= 0x58635fa9u; }
+__device__ __forceinline__ bool temperature_plain(double T) { return (uint32_t)__double2hiint(T) < 0x430c6bf5u; }
 
 // Emission in 64-packet windows.  The first Philox block of every packet
 // gives its frequency; the packets with xi <= 0 (about half) are absorbed at
@@ -1089,11 +1108,29 @@ __device__ __forceinline__ bool home_without_direction(R xi, R vt, const typenam
 // memory and are finished 32 at a time, so the warp's lanes stay busy in the
 // costly part (direction, ray set-up, home test); leftovers carry over to the
 // next window and are flushed at the end (and, in batches, at a change of box).
+// A waiting binary32 packet keeps its first block's words; the binary64 form is
+// bound by its arithmetic and draws its two blocks again.
 constexpr uint32_t kStash = 96;  // < 32 left over + 64 new
-template <class R>
-struct EmitStash {
+template <class R> struct EmitStash;
+template <> struct EmitStash<float> {
+  uint32_t at[32];
+  uint32_t cell[kStash], j[kStash], w0[kStash], w1[kStash], w2[kStash], w3[kStash];
+  __device__ __forceinline__ void put(uint32_t k, uint32_t c, uint32_t jj, const U4& r) {
+    cell[k] = c; j[k] = jj; w0[k] = r.a; w1[k] = r.b; w2[k] = r.c; w3[k] = r.d;
+  }
+  template <class S>
+  __device__ __forceinline__ void position(uint32_t k, const S&, uint32_t, uint32_t, float f[3], float* uq) const {
+    f[0] = u01f(w0[k]); f[1] = u01f(w1[k]); f[2] = u01f(w2[k]); *uq = u01f(w3[k]);
+  }
+};
+template <> struct EmitStash<double> {
+  uint32_t at[32];
   uint32_t cell[kStash], j[kStash];
-  R f0[kStash], f1[kStash], f2[kStash], xi[kStash], vt[kStash];
+  __device__ __forceinline__ void put(uint32_t k, uint32_t c, uint32_t jj, const U4&) { cell[k] = c; j[k] = jj; }
+  template <class S>
+  __device__ __forceinline__ void position(uint32_t, const S& s, uint32_t c, uint32_t jj, double f[3], double* uq) const {
+    Draws<double>::position(s, c, jj, f, uq);
+  }
 };
 
 // Finish up to 32 packets from the head of the ring (head, count: warp-uniform).
@@ -1109,9 +1146,11 @@ __device__ __forceinline__ void emit_finish32(const TransportArgs<R>& a, const E
   uint32_t cell = 0, j = 0;
   R f[3] = {(R)0, (R)0, (R)0}, xi = (R)0, vt = (R)0;
   if (act) {
-    cell = st.cell[k]; j = st.j[k];
-    f[0] = st.f0[k]; f[1] = st.f1[k]; f[2] = st.f2[k];
-    xi = st.xi[k]; vt = st.vt[k];
+    R uq;
+    cell = st.cell[k];
+    j = st.j[k];
+    st.position(k, KStream{a.ks, e.box}, cell, j, f, &uq);
+    emit_draw0<R>(a, e, cell, uq, &xi, &vt);
   }
   __syncwarp();  // read before the slots are reused
   head += take;
@@ -1130,24 +1169,24 @@ template <class R, bool P2, bool FRESH = false>
 __device__ __forceinline__ void emit_window64(const TransportArgs<R>& a, const EmitBox<R>& e, EmitStash<R>& st,
                                               uint32_t base, uint32_t N, uint32_t& head, uint32_t& count,
                                               uint64_t& my_abs, uint64_t& my_cross) {
-  using V = typename Vec4<R>::T;
   const int lane = threadIdx.x & 31;
   const unsigned lt = (1u << lane) - 1u;
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
-    uint32_t cell, j;
-    const bool act = emit_locate<R, FRESH>(e, base + 32u * h, N, &cell, &j);
-    R f[3] = {(R)0, (R)0, (R)0}, xi = (R)0, vt = (R)0;
+    if (base + 32u * h >= N) break;  // the coarse index ends at the last packet
+    uint32_t cell, j, starts;
+    bool whole;
+    const bool act = emit_locate<R, FRESH>(e, base + 32u * h, N, st.at, &cell, &j, &starts, &whole);
+    U4 r{0, 0, 0, 0};
     bool early = false;
     if (act) {
-      emit_draw0<R>(a, e, cell, j, f, &xi, &vt);
-      const V Uh = e.vel[cell];
-      early = home_without_direction<R>(xi, vt, Uh);
+      r = draw(KStream{a.ks, e.box}, cell, j, Draws<R>::kQuantBlock);
+      early = r.d < e.early && temperature_plain(__ldg(e.T + cell));
     }
     // home tally of the early packets (warp-aggregated)
-    const uint32_t key = early ? cell : 0xffffffffu;
-    const unsigned m = __match_any_sync(0xffffffffu, key);
-    if (early && lane == __ffs(m) - 1) atomicAdd(e.tally + cell, (uint32_t)__popc(m));
+    const unsigned em = __ballot_sync(0xffffffffu, early);
+    const unsigned m = em & (whole ? lane_group(starts) : key_group(cell));
+    if (early && (m & lt) == 0u) atomicAdd(e.tally + cell, (uint32_t)__popc(m));
     if (early) ++my_abs;
     // the others to the ring, in lane order after the waiting ones
     const bool pend = act && !early;
@@ -1155,67 +1194,12 @@ __device__ __forceinline__ void emit_window64(const TransportArgs<R>& a, const E
     if (pend) {
       uint32_t k = head + count + __popc(pm & lt);
       if (k >= kStash) k -= kStash;
-      st.cell[k] = cell; st.j[k] = j;
-      st.f0[k] = f[0]; st.f1[k] = f[1]; st.f2[k] = f[2];
-      st.xi[k] = xi; st.vt[k] = vt;
+      st.put(k, cell, j, r);
     }
     count += __popc(pm);
   }
   __syncwarp();
   while (count >= 32u) emit_finish32<R, P2>(a, e, st, head, count, my_abs, my_cross);
-}
-
-// The same window for batches, whose consecutive windows may belong to
-// different boxes: every waiting packet is finished before it returns (one
-// call site of the costly part keeps the batch kernels' register budget).
-template <class R, bool P2, bool FRESH = false>
-__device__ __forceinline__ void emit_window64_drain(const TransportArgs<R>& a, const EmitBox<R>& e, EmitStash<R>& st,
-                                              uint32_t base, uint32_t N, uint64_t& my_abs, uint64_t& my_cross) {
-  using V = typename Vec4<R>::T;
-  const int lane = threadIdx.x & 31;
-  const unsigned lt = (1u << lane) - 1u;
-  uint32_t npend = 0;
-#pragma unroll
-  for (int h = 0; h < 2; ++h) {
-    uint32_t cell, j;
-    const bool act = emit_locate<R, FRESH>(e, base + 32u * h, N, &cell, &j);
-    R f[3] = {(R)0, (R)0, (R)0}, xi = (R)0, vt = (R)0;
-    bool early = false;
-    if (act) {
-      emit_draw0<R>(a, e, cell, j, f, &xi, &vt);
-      const V Uh = e.vel[cell];
-      early = home_without_direction<R>(xi, vt, Uh);
-    }
-    // home tally of the early packets (warp-aggregated)
-    const uint32_t key = early ? cell : 0xffffffffu;
-    const unsigned m = __match_any_sync(0xffffffffu, key);
-    if (early && lane == __ffs(m) - 1) atomicAdd(e.tally + cell, (uint32_t)__popc(m));
-    if (early) ++my_abs;
-    // the others to the stash, in lane order after the pending ones
-    const bool pend = act && !early;
-    const unsigned pm = __ballot_sync(0xffffffffu, pend);
-    if (pend) {
-      const uint32_t k = npend + __popc(pm & lt);
-      st.cell[k] = cell; st.j[k] = j;
-      st.f0[k] = f[0]; st.f1[k] = f[1]; st.f2[k] = f[2];
-      st.xi[k] = xi; st.vt[k] = vt;
-    }
-    npend += __popc(pm);
-  }
-  __syncwarp();
-  for (uint32_t r0 = 0; r0 < npend; r0 += 32) {
-    const uint32_t k = r0 + lane;
-    const bool act = k < npend;
-    uint32_t cell = 0, j = 0;
-    R f[3] = {(R)0, (R)0, (R)0}, xi = (R)0, vt = (R)0;
-    if (act) {
-      cell = st.cell[k]; j = st.j[k];
-      f[0] = st.f0[k]; f[1] = st.f1[k]; f[2] = st.f2[k];
-      xi = st.xi[k]; vt = st.vt[k];
-    }
-    emit_rest<R, P2>(a, e, act, cell, j, f, xi, vt, my_abs, my_cross);
-  }
-  __syncwarp();  // the stash is reused by the next window
 }
 
 // Resident blocks per SM of the emission (registers and the shared-memory ring:
@@ -1224,7 +1208,8 @@ template <class R> constexpr int emit_occupancy() { return sizeof(R) == 4 ? 5 : 
 
 template <class R, bool P2>
 __global__ void __launch_bounds__(TT, emit_occupancy<R>()) k_emit(TransportArgs<R> a) {
-  const EmitBox<R> e{a.P, a.first, (uint32_t)a.n3, (uint32_t)a.n, a.vel, a.T, a.tally, a.kappa, a.cth, 0u, a.tl, 0u};
+  const EmitBox<R> e{a.P, a.first, (uint32_t)a.n3, (uint32_t)a.n, a.vel, a.T, a.tally, a.kappa, a.cth, 0u, a.tl, 0u,
+                     a.sc->vq_u > 0.0f ? a.early : 0u};
   const uint32_t N = __ldg(a.P + a.n3);  // packets actually allocated
   __shared__ EmitStash<R> stash[TT / 32];
   EmitStash<R>& st = stash[threadIdx.x >> 5];
@@ -1737,6 +1722,17 @@ void alloc_launch(rec_ctx* c, int blocks, const typename Vec4<R>::T* vel, const 
   k_alloc_prefix<R, IT><<<blocks, AT, 0, c->stream>>>(emis, c->n3, npk, c->sc, c->partQ, c->P, c->first, tl, c->bcap);
 }
 
+// Bound of the quantile's leading word w below which xi <= 0 (0: none).  The deviate
+// u < (w + 257) 2^-32 (binary32 keeps the top 23 bits and adds half a unit), the table node k = trunc(u (M - 1)) after
+// one rounding (2^-23 relative covers both precisions), and a node is safe if
+// interpolation from it cannot pass zero by rounding: its upper end q1 = 0 (then q1 - q0 is
+// exact), or q1 <= -2^-20 |q0|.
+uint32_t early_word(const rec_ctx* c, double cth) {
+  if (!(cth <= 1e15)) return 0u;
+  const double w = std::floor((double)c->early_nodes / (double)(c->params.n_quantiles - 1) * (1.0 - 0x1p-22) * 0x1p32) - 258.0;
+  return w > 0.0 ? (uint32_t)std::min(w, 4294967295.0) : 0u;
+}
+
 template <class R>
 cudaError_t run_transport(rec_ctx* c, int step, double z, rec_stats* st) {
   const rec_box& b = c->box;
@@ -1770,6 +1766,7 @@ cudaError_t run_transport(rec_ctx* c, int step, double z, rec_stats* st) {
   a.cth = (R)cth;
   a.strm = s;
   a.ks = key_schedule(s.k0, s.k1);
+  a.early = early_word(c, cth);
   a.tally = b.tally;
   a.sc = c->sc;
   a.queue = (typename Vec4<R>::T*)c->queue;
@@ -1963,53 +1960,12 @@ __global__ void __launch_bounds__(AT) k_alloc_prefix_batch(const BoxDev* bxs, in
 }
 
 // Emission over the batch packet space (each box padded to a multiple of 64,
-// so a warp's 64-packet window belongs to one box).  FRESH: the packet prefixes and
-// box scalars were written earlier in the same launch (read through L2).
+// so a warp's 64-packet window belongs to one box): the ring is flushed at each change of
+// box; one cell-coordinate path (exact multiply-high divisions) for every side keeps
+// the kernel within its registers.  FRESH: the packet prefixes and box scalars were
+// written earlier in the same launch (read through L2).
 template <class R, bool FRESH>
-__device__ __forceinline__ void emit_batch_body_drain(const TransportArgs<R>& a, const BoxDev* bxs, const BoxStep* bst, int B,
-                                                uint64_t tot_pk) {
-  using V = typename Vec4<R>::T;
-  __shared__ BoxCounters cnt;
-  __shared__ EmitStash<R> stash[TT / 32];
-  EmitStash<R>& st = stash[threadIdx.x >> 5];
-  box_counters_clear(cnt, B);
-  uint64_t my_abs = 0, my_cross = 0;
-  int cur = -1;
-  uint64_t lo_pk = 1, hi_pk = 0;  // packet range of box cur (empty before the first lookup)
-  uint32_t N = 0;
-  const uint64_t warps_total = (uint64_t)gridDim.x * (TT / 32);
-  // 64-packet windows: every box's packet space is padded to a multiple of 64
-  for (uint64_t gbase = ((uint64_t)blockIdx.x * (TT / 32) + (threadIdx.x >> 5)) * 64; gbase < tot_pk;
-       gbase += warps_total * 64) {
-    if (gbase < lo_pk || gbase >= hi_pk) {  // next box (uniform over the warp)
-      const int b = last_le(B, gbase, [&](int i) { return bxs[i].pk0; });
-      if (cur >= 0) box_counters_add(cnt, cur, my_abs, 0, my_cross);
-      my_abs = my_cross = 0;
-      cur = b;
-      lo_pk = bxs[b].pk0;
-      hi_pk = (b + 1 < B) ? bxs[b + 1].pk0 : tot_pk;
-      N = ld_index<FRESH>(bxs[b].P + bxs[b].n3);  // packets actually allocated to this box
-    }
-    const uint64_t base = gbase - lo_pk;
-    if (base >= N) continue;  // padding of the packet space
-    const BoxDev& d = bxs[cur];
-    const EmitBox<R> e{d.P, d.first, (uint32_t)d.n3, d.n, (const V*)d.vel4, (const R*)d.T, d.tally,
-                       (R)__ldcg(&bst[cur].kappa), (R)__ldcg(&bst[cur].cth),
-                       (uint32_t)cur, Tiles{d.n, d.nt, d.lg, d.mn, d.mn2, d.tlg}, d.bk0};
-    // power-of-two sides take cell coordinates by shifts and the periodic wrap
-    // by masks; other sides by exact multiply-high divisions (the binary64 form
-    // keeps one path: both would not fit its register budget)
-    if (sizeof(R) == 4 && d.p2) emit_window64_drain<R, true, FRESH>(a, e, st, (uint32_t)base, N, my_abs, my_cross);
-    else emit_window64_drain<R, false, FRESH>(a, e, st, (uint32_t)base, N, my_abs, my_cross);
-  }
-  if (cur >= 0) box_counters_add(cnt, cur, my_abs, 0, my_cross);
-  box_counters_flush(cnt, bxs, B);
-}
-// Binary32 batches: the ring carried over between windows (as the single-box
-// emission), flushed at each change of box; one cell-coordinate path (exact
-// multiply-high divisions) for every side keeps the kernel within its registers.
-template <class R, bool FRESH>
-__device__ __forceinline__ void emit_batch_body_ring(const TransportArgs<R>& a, const BoxDev* bxs, const BoxStep* bst,
+__device__ __forceinline__ void emit_batch_body(const TransportArgs<R>& a, const BoxDev* bxs, const BoxStep* bst,
                                                      int B, uint64_t tot_pk) {
   using V = typename Vec4<R>::T;
   __shared__ BoxCounters cnt;
@@ -2025,7 +1981,8 @@ __device__ __forceinline__ void emit_batch_body_ring(const TransportArgs<R>& a, 
     const BoxDev& d = bxs[b];
     return EmitBox<R>{d.P, d.first, (uint32_t)d.n3, d.n, (const V*)d.vel4, (const R*)d.T, d.tally,
                       (R)__ldcg(&bst[b].kappa), (R)__ldcg(&bst[b].cth),
-                      (uint32_t)b, Tiles{d.n, d.nt, d.lg, d.mn, d.mn2, d.tlg}, d.bk0};
+                      (uint32_t)b, Tiles{d.n, d.nt, d.lg, d.mn, d.mn2, d.tlg}, d.bk0,
+                      __ldcg(&d.sc->vq_u) > 0.0f ? a.early : 0u};
   };
   const uint64_t warps_total = (uint64_t)gridDim.x * (TT / 32);
   for (uint64_t gbase = ((uint64_t)blockIdx.x * (TT / 32) + (threadIdx.x >> 5)) * 64; gbase < tot_pk;
@@ -2049,15 +2006,8 @@ __device__ __forceinline__ void emit_batch_body_ring(const TransportArgs<R>& a, 
   box_counters_flush(cnt, bxs, B);
 }
 
-template <class R, bool FRESH>
-__device__ __forceinline__ void emit_batch_body(const TransportArgs<R>& a, const BoxDev* bxs, const BoxStep* bst, int B,
-                                                uint64_t tot_pk) {
-  if (sizeof(R) == 4) emit_batch_body_ring<R, FRESH>(a, bxs, bst, B, tot_pk);
-  else emit_batch_body_drain<R, FRESH>(a, bxs, bst, B, tot_pk);
-}
-
 template <class R>
-__global__ void __launch_bounds__(TT, 4) k_emit_batch(TransportArgs<R> a, const BoxDev* bxs, const BoxStep* bst,
+__global__ void __launch_bounds__(TT, sizeof(R) == 4 ? 4 : 3) k_emit_batch(TransportArgs<R> a, const BoxDev* bxs, const BoxStep* bst,
                                                       int B, uint64_t tot_pk) {
   emit_batch_body<R, false>(a, bxs, bst, B, tot_pk);
 }
@@ -2090,9 +2040,6 @@ __device__ __forceinline__ void transport_end_batch(const BoxDev* bxs, int B, co
     }
   }
 }
-__global__ void k_transport_end_batch(const BoxDev* bxs, int B, const unsigned long long* bfill, rec_stats* st) {
-  transport_end_batch(bxs, B, bfill, st);
-}
 
 // The allocation and the emission of a batched transport call as phases of
 // one persistent cooperative launch, separated by bounded grid barriers: box
@@ -2102,7 +2049,7 @@ __global__ void k_transport_end_batch(const BoxDev* bxs, int B, const unsigned l
 // per-phase kernels as virtual blocks.  A barrier that gives up ends the launch
 // (flags bit 3 of the batch record) and the march that follows finds no work.
 template <class R>
-__global__ void __launch_bounds__(AT, 4) k_batch_front(TransportArgs<R> a, const BoxDev* bxs, BoxStep* bst,
+__global__ void __launch_bounds__(AT, sizeof(R) == 4 ? 4 : 3) k_batch_front(TransportArgs<R> a, const BoxDev* bxs, BoxStep* bst,
                                                        BoxStepArgs bs, int B, uint32_t k0, uint32_t k1,
                                                        DevScalars* gsc, unsigned long long* partQ, unsigned long long* cpre,
                                                        uint32_t n_ablk, uint64_t tot_pk,
@@ -2137,6 +2084,9 @@ cudaError_t run_transport_batch(rec_ctx* c, int step, double z, rec_stats* st) {
   a.M = c->params.n_quantiles;
   a.strm = Stream{k0, k1, 0u};
   a.ks = key_schedule(k0, k1);
+  double cth_max = 0.0;
+  for (int b = 0; b < B; ++b) cth_max = std::max(cth_max, bs.s[b].cth);
+  a.early = early_word(c, cth_max);
   a.sc = c->gsc;
   a.queue = (typename Vec4<R>::T*)c->queue;
   a.nb = nb;
