@@ -704,7 +704,7 @@ def measured_peaks():
 PROFILED_SOURCE = {
     "march": ("k_march_256.md", "rec_transport.cu",
               (("// Traversal state of one packet.", "__device__ __forceinline__ void add_counters("),
-               ("// March of the queued packets.", "__global__ void k_transport_end("))),
+               ("// March of the queued packets.", "// Region sweeps, between two march launches (one block)"))),
     "emit": ("k_emit_256.md", "rec_transport.cu", None),
     "rec_step": ("rec_step_passes_256.md", "rec_step.cu", None),
 }

@@ -351,9 +351,9 @@ rec_status rec_transport_params(const rec_params* params, int32_t n, double z, d
  * launched since the last clear (arrays of REC_T_COUNT).  Groups:
  *   0  packet allocation (3 kernels per lya_transport)
  *   1  packet emission and home-cell test (1 kernel)
- *   2  march of the queued packets (1 kernel)
- *   3  transport bookkeeping (1 kernel)
- *   4  rec_step passes (begin, Newton, final per substep)
+ *   2  march of the queued packets (1 kernel), which also closes the call
+ *   3  unused (0)
+ *   4  rec_step passes (1 kernel per substep; local and partial mixing: 2)
  *   5  rec_step_adjoint passes
  *   6  rec_state_init / rec_refresh / rec_xe_adjoint */
 #define REC_T_COUNT 7

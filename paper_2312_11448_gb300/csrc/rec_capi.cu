@@ -87,16 +87,16 @@ rec_tuning default_tuning(bool mixed, bool batch, uint64_t packets, int sm_count
   rec_tuning t;
   rec::transport_limits(mixed, batch, &t.emit_blocks_per_sm, &t.march_blocks_per_sm);
   // Parked or idle lanes before a warp tests and refills: a refill costs the warp
-  // about as much as two rounds of its walk, so it waits for nearly half of
-  // its lanes (256^3, 1e8 packets: 4.53 / 4.00 / 4.04 ms per march at 8 / 14 / 18).
-  t.march_refill = 14;
-  // Chunks as large as leaves eight to a resident warp of the march (about half
-  // of the packets are queued): fewer look-ups of the next chunk (256^3, 1e8
-  // packets: 4.00 / 3.80 ms at 64 / 256), down to 32 so that small boxes use
-  // every warp.
+  // about as much as two rounds of its walk, so it waits for half of its lanes
+  // (256^3, 1e8 packets: 3.77 / 3.69 / 3.66 / 3.67 ms per march at 12 / 14 / 16 / 18).
+  t.march_refill = 16;
+  // Chunks as large as leaves three to a resident warp of the march (about half
+  // of the packets are queued), since looking the next chunk up takes microseconds
+  // (128^3, 1e7 packets: 524 / 398 / 314 / 299 us at 32 / 64 / 128 / 256; 100^3, 4e6:
+  // 204 / 162 / 151 / 159 us), down to 32 so that small boxes use every warp.
   t.march_chunk = 256;
   const uint64_t warps = (uint64_t)sm_count * (uint64_t)t.march_blocks_per_sm * 8;
-  while (t.march_chunk > 32 && packets / 2 < 8 * warps * (uint64_t)t.march_chunk) t.march_chunk /= 2;
+  while (t.march_chunk > 32 && packets / 2 < 3 * warps * (uint64_t)t.march_chunk) t.march_chunk /= 2;
   t.tile = 32;
   t.march_halo = 0;
   return t;
@@ -108,16 +108,43 @@ uint32_t log2u(uint32_t v) {
   return l;
 }
 
-// Device scratch that only saves time: NULL where it would take more than an
-// eighth of the memory that is free, or cannot be had.
-void* optional_scratch(size_t bytes) {
-  size_t free_bytes = 0, total = 0;
-  void* p = nullptr;
-  if (cudaMemGetInfo(&free_bytes, &total) != cudaSuccess || bytes > free_bytes / 8 || cudaMalloc(&p, bytes) != cudaSuccess) {
-    cudaGetLastError();
-    return nullptr;
+// The device scratch of a context is one allocation, carved up (a dozen
+// allocations took most of rec_init's time).
+struct Carver {
+  char* base = nullptr;
+  size_t used = 0;
+  template <class T>
+  void take(T** p, size_t bytes) {
+    *p = base ? (T*)(base + used) : nullptr;
+    used += round_up(std::max<size_t>(bytes, 1), 256);
   }
-  return p;
+};
+// lay(carver, optional): sets the pointers; optional: with the scratch that only saves
+// time.  That is left out where it would take more than an eighth of the memory
+// that is free, or cannot be had.
+template <class F>
+cudaError_t carve_scratch(rec_ctx* c, F lay) {
+  Carver need, with;
+  lay(need, false);
+  lay(with, true);
+  const size_t extra = with.used - need.used;
+  bool optional = extra > 0;
+  if (extra > ((size_t)256 << 20)) {
+    size_t free_bytes = 0, total = 0;
+    optional = cudaMemGetInfo(&free_bytes, &total) == cudaSuccess && extra <= free_bytes / 8;
+  }
+  cudaError_t e = cudaErrorMemoryAllocation;
+  if (optional) e = cudaMalloc(&c->slab, with.used);
+  if (e == cudaErrorMemoryAllocation) {
+    cudaGetLastError();
+    optional = false;
+    e = cudaMalloc(&c->slab, need.used);
+  }
+  if (e != cudaSuccess) { c->slab = nullptr; return e; }
+  Carver at;
+  at.base = (char*)c->slab;
+  lay(at, optional);
+  return cudaSuccess;
 }
 
 // Super-tile layout of every box of a batch for the tile side in use.
@@ -206,29 +233,31 @@ rec_status init_batch(const rec_params* params, const rec_box* boxes, int32_t n_
   const size_t qbytes = (size_t)params->n_quantiles * (mixed ? 4 : 8);
   const size_t part_n = std::max<size_t>(2 * (size_t)rec::kMaxSums * c->tot_pblk, (size_t)rec::kMaxSums * c->tot_ablk);
   const size_t qentry = mixed ? 32 : 96;  // two float4 | three double4 per queued packet
-  e = cudaMalloc(&c->sc, sizeof(rec::DevScalars) * n_boxes);
-  if (e == cudaSuccess) e = cudaMalloc(&c->gsc, sizeof(rec::DevScalars));
-  if (e == cudaSuccess) e = cudaMalloc(&c->sc_adj, sizeof(rec::DevScalars));
-  if (e == cudaSuccess) e = cudaMalloc(&c->part, sizeof(double) * part_n);
-  if (e == cudaSuccess) e = cudaMalloc(&c->P, sizeof(uint32_t) * nP);
-  if (e == cudaSuccess) e = cudaMalloc(&c->partQ, sizeof(unsigned long long) * (size_t)c->tot_ablk);
-  if (e == cudaSuccess) e = cudaMalloc(&c->first, sizeof(uint32_t) * nfirst);
-  if (e == cudaSuccess && mixed) e = cudaMalloc(&c->xy, sizeof(float) * 2 * nxy);
-  if (e == cudaSuccess) e = cudaMalloc(&c->bcap, sizeof(unsigned long long) * nb_alloc);
-  if (e == cudaSuccess) e = cudaMalloc(&c->bfill, sizeof(unsigned long long) * nb_alloc);
-  if (e == cudaSuccess) e = cudaMalloc(&c->cpre, sizeof(unsigned long long) * (nb_alloc + 1));
-  if (e == cudaSuccess) e = cudaMalloc(&c->quant, qbytes);
-  if (e == cudaSuccess) e = cudaMalloc(&c->queue, qentry * std::max<size_t>(npk_all, 1));
-  if (e == cudaSuccess) e = cudaMalloc(&c->bx, sizeof(rec::BoxDev) * n_boxes);
-  if (e == cudaSuccess) e = cudaMalloc(&c->bstep, sizeof(rec::BoxStep) * n_boxes);
+  e = carve_scratch(c, [&](Carver& m, bool optional) {
+    m.take(&c->sc, sizeof(rec::DevScalars) * n_boxes);
+    m.take(&c->gsc, sizeof(rec::DevScalars));
+    m.take(&c->sc_adj, sizeof(rec::DevScalars));
+    m.take(&c->part, sizeof(double) * part_n);
+    m.take(&c->P, sizeof(uint32_t) * nP);
+    m.take(&c->partQ, sizeof(unsigned long long) * (size_t)c->tot_ablk);
+    m.take(&c->first, sizeof(uint32_t) * nfirst);
+    if (mixed) m.take(&c->xy, sizeof(float) * 2 * nxy);
+    m.take(&c->bcap, sizeof(unsigned long long) * nb_alloc);
+    m.take(&c->bfill, sizeof(unsigned long long) * nb_alloc);
+    m.take(&c->cpre, sizeof(unsigned long long) * (nb_alloc + 1));
+    m.take(&c->quant, qbytes);
+    m.take(&c->queue, qentry * std::max<size_t>(npk_all, 1));
+    m.take(&c->bx, sizeof(rec::BoxDev) * n_boxes);
+    m.take(&c->bstep, sizeof(rec::BoxStep) * n_boxes);
+    c->velq = nullptr;
+    if (optional) m.take(&c->velq, sizeof(uint32_t) * nvelq);
+  });
   if (e != cudaSuccess) {
     rec_status r = (e == cudaErrorMemoryAllocation) ? fail(nullptr, REC_ENOMEM, "device allocation failed")
                                                     : cuda_fail(nullptr, e, "cudaMalloc");
     rec_free(c);
     return r;
   }
-  // scratch that only saves time is left out where memory is short
-  c->velq = (uint32_t*)optional_scratch(sizeof(uint32_t) * nvelq);
   nvelq = 0;
   for (int i = 0; i < n_boxes; ++i) {
     const rec_box& b = boxes[i];
@@ -317,38 +346,40 @@ rec_status rec_init(const rec_params* params, const rec_box* boxes, int32_t n_bo
   c->tune = default_tuning(params->precision == REC_PREC_MIXED, false, b.n_packets, c->sm_count);
 
   size_t qbytes = (size_t)params->n_quantiles * (params->precision == REC_PREC_MIXED ? 4 : 8);
-  e = cudaMalloc(&c->sc, sizeof(rec::DevScalars));
-  if (e == cudaSuccess) e = cudaMalloc(&c->sc_adj, sizeof(rec::DevScalars));
-  // block partials (two per block: the TMA-staged passes run more blocks than the grid)
-  if (e == cudaSuccess) e = cudaMalloc(&c->part, 2 * sizeof(double) * rec::kMaxSums * (size_t)c->grid);
-  if (e == cudaSuccess) e = cudaMalloc(&c->P, sizeof(uint32_t) * (size_t)(c->n3 + 1));
-  if (e == cudaSuccess) e = cudaMalloc(&c->partQ, sizeof(unsigned long long) * (size_t)c->alloc_blocks);
-  if (e == cudaSuccess) e = cudaMalloc(&c->first, sizeof(uint32_t) * (size_t)(b.n_packets / 32 + 2));
-  if (e == cudaSuccess && params->precision == REC_PREC_MIXED) e = cudaMalloc(&c->xy, sizeof(float) * 2 * (size_t)c->n3);
-  // local mixing: velocity divergence per cell (working precision)
-  if (e == cudaSuccess && (params->mixing == REC_MIX_LOCAL || params->mixing == REC_MIX_PARTIAL))
-    e = cudaMalloc(&c->div, (params->precision == REC_PREC_MIXED ? 4 : 8) * (size_t)c->n3);
-  {
-    // super-tiles of the march queue, sized for the smallest tile side
-    size_t nt = (size_t)((b.n + rec::kMinTile - 1) / rec::kMinTile), nb = nt * nt * nt;
-    if (e == cudaSuccess) e = cudaMalloc(&c->bcap, sizeof(unsigned long long) * nb);
-    if (e == cudaSuccess) e = cudaMalloc(&c->bfill, sizeof(unsigned long long) * nb);
-    if (e == cudaSuccess) e = cudaMalloc(&c->cpre, sizeof(unsigned long long) * (nb + 1));
-  }
-  if (e == cudaSuccess) e = cudaMalloc(&c->quant, qbytes);
-  // march queue: two float4 (mixed) or three double4_32a (FP64) per packet, worst case all packets
-  size_t qentry = params->precision == REC_PREC_MIXED ? 32 : 96;
-  if (e == cudaSuccess) e = cudaMalloc(&c->queue, qentry * (size_t)std::max<uint64_t>(b.n_packets, 1));
+  const bool mixed = params->precision == REC_PREC_MIXED;
+  const size_t n3 = (size_t)c->n3;
+  // super-tiles of the march queue, sized for the smallest tile side
+  const size_t nt = (size_t)((b.n + rec::kMinTile - 1) / rec::kMinTile), nb = nt * nt * nt;
+  e = carve_scratch(c, [&](Carver& m, bool optional) {
+    m.take(&c->sc, sizeof(rec::DevScalars));
+    m.take(&c->sc_adj, sizeof(rec::DevScalars));
+    // block partials (two per block: the TMA-staged passes run more blocks than the grid)
+    m.take(&c->part, 2 * sizeof(double) * rec::kMaxSums * (size_t)c->grid);
+    m.take(&c->P, sizeof(uint32_t) * (n3 + 1));
+    m.take(&c->partQ, sizeof(unsigned long long) * (size_t)c->alloc_blocks);
+    m.take(&c->first, sizeof(uint32_t) * (size_t)(b.n_packets / 32 + 2));
+    if (mixed) m.take(&c->xy, sizeof(float) * 2 * n3);
+    // local mixing: velocity divergence per cell (working precision)
+    if (params->mixing == REC_MIX_LOCAL || params->mixing == REC_MIX_PARTIAL) m.take(&c->div, (mixed ? 4 : 8) * n3);
+    m.take(&c->bcap, sizeof(unsigned long long) * nb);
+    m.take(&c->bfill, sizeof(unsigned long long) * nb);
+    m.take(&c->cpre, sizeof(unsigned long long) * (nb + 1));
+    m.take(&c->quant, qbytes);
+    // march queue: two float4 (mixed) or three double4_32a (FP64) per packet, worst case all packets
+    m.take(&c->queue, (mixed ? 32 : 96) * (size_t)std::max<uint64_t>(b.n_packets, 1));
+    c->velq = nullptr;
+    c->cellcache = nullptr;
+    if (optional) {
+      m.take(&c->velq, sizeof(uint32_t) * rec::velq_words((uint32_t)b.n));
+      if (!mixed && params->mixing != REC_MIX_LOCAL) m.take(&c->cellcache, 5 * sizeof(double) * n3);
+    }
+  });
   if (e != cudaSuccess) {
     rec_status r = (e == cudaErrorMemoryAllocation) ? fail(nullptr, REC_ENOMEM, "device allocation failed")
                                                     : cuda_fail(nullptr, e, "cudaMalloc");
     rec_free(c);
     return r;
   }
-  // scratch that only saves time is left out where memory is short
-  c->velq = (uint32_t*)optional_scratch(sizeof(uint32_t) * rec::velq_words((uint32_t)b.n));
-  if (params->precision == REC_PREC_FP64 && params->mixing != REC_MIX_LOCAL)
-    c->cellcache = optional_scratch(5 * sizeof(double) * (size_t)c->n3);
   // emission-profile table in the working precision of the transport
   std::vector<char> hq(qbytes);
   for (int i = 0; i < params->n_quantiles; ++i) {
@@ -648,32 +679,15 @@ void rec_free(rec_ctx* c) {
   for (int g = 0; g < REC_T_COUNT; ++g)
     for (auto& pr : c->ev[g]) { cudaEventDestroy(pr.first); cudaEventDestroy(pr.second); }
   for (cudaEvent_t e : c->pool) cudaEventDestroy(e);
-  cudaFree(c->sc);
-  cudaFree(c->sc_adj);
-  cudaFree(c->part);
-  cudaFree(c->P);
-  cudaFree(c->partQ);
-  cudaFree(c->quant);
-  cudaFree(c->queue);
-  cudaFree(c->velq);
-  cudaFree(c->cellcache);
-  cudaFree(c->first);
-  cudaFree(c->xy);
-  cudaFree(c->bcap);
-  cudaFree(c->bfill);
-  cudaFree(c->cpre);
+  cudaFree(c->slab);
   cudaFree(c->rqueue);
   cudaFree(c->rcount);
   cudaFree(c->scnt);
   cudaFree(c->rqn);
-  cudaFree(c->div);
   cudaFree(c->mc_scratch);
   cudaFree(c->trb_scratch);
   cudaFree(c->mf_cnt);
   if (c->gexec) cudaGraphExecDestroy(c->gexec);
-  cudaFree(c->bx);
-  cudaFree(c->bstep);
-  cudaFree(c->gsc);
   delete c;
 }
 

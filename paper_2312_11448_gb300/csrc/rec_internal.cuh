@@ -149,7 +149,9 @@ struct rec_ctx {
   cudaStream_t stream;
   int64_t n3;
   rec::Cosmo cosmo;
-  // device scratch owned by the context
+  // device scratch owned by the context: one allocation, which the pointers below
+  // lie in where nothing else is said
+  void* slab = nullptr;
   rec::DevScalars* sc;       // device scalars of the forward sweep
   rec::DevScalars* sc_adj;   // device scalars of the reverse sweep
   double* part;              // block partials [grid * kMaxSums]

@@ -16,15 +16,12 @@
 //   k_alloc_prefix  packet prefix P_i = floor((N prefixQ_i + u) / sum Q), exact
 //                   integer arithmetic; cell of every 32nd packet; packets per
 //                   32^3 super-tile
-//   k_bucket_offsets  queue bucket offsets (capacities) per super-tile
 //   k_emit          one packet per thread: warp-cooperative cell lookup in P,
 //                   Philox draws, emission, resonance test in the home cell
 //                   (warp-aggregated tally); the others step once and are queued
 //                   in their home super-tile's bucket
-//   k_bucket_scan   prefix of the queued counts (bucket order of the march)
 //   k_march         persistent warps march the queued packets (Amanatides-Woo),
 //                   refilling idle lanes from the queue; tally atomics
-//   k_transport_end counters to the statistics record
 // The march is written operation by operation with round-to-nearest
 // intrinsics (never contracted into FMA), in binary32 for the mixed form and
 // binary64 for the FP64 form, so its integer results are reproducible.
@@ -285,13 +282,15 @@ __device__ __forceinline__ void take_maxima(DevScalars* sc, float kappa) {
 }
 
 // Reads the emission weights once (their maximum, exact in the working precision)
-// and the velocities once (the scale of their compact copy).
+// and the velocities once (the scale of their compact copy); clears the bucket capacities.
 template <class R>
 __global__ void __launch_bounds__(kPassThreads) k_alloc_max(const R* emis, const typename Vec4<R>::T* vel, int64_t n3,
-                                                            float kappa, DevScalars* sc) {
+                                                            float kappa, DevScalars* sc, unsigned long long* bcap,
+                                                            int nb) {
   R m = (R)0;
   bool bad = false;
   VelMax vm;
+  for (int i = blockIdx.x * kPassThreads + threadIdx.x; i < nb; i += gridDim.x * kPassThreads) bcap[i] = 0ull;
   for (int64_t i = (int64_t)blockIdx.x * kPassThreads + threadIdx.x; i < n3; i += (int64_t)gridDim.x * kPassThreads) {
     const R r = emis[i];
     if (!(r >= (R)0) || isinf(r)) bad = true;
@@ -582,39 +581,44 @@ __device__ __forceinline__ void alloc_prefix_block(const R* emis, int64_t n3, ui
   }
 }
 
-template <class R, int IT>
-__global__ void __launch_bounds__(AT) k_alloc_prefix(const R* emis, int64_t n3, uint64_t n_packets, DevScalars* sc,
-                                                     const unsigned long long* partQ, uint32_t* P, uint32_t* first,
-                                                     Tiles tl, unsigned long long* bcap) {
-  const int64_t c0 = (int64_t)blockIdx.x * (AT * IT) + (int64_t)threadIdx.x * IT;
-  alloc_prefix_block<R, IT>(emis, n3, n_packets, sc->sumQ, sc->alloc_u, (R)sc->rmax, partQ[blockIdx.x], c0, P, first, tl,
-                        0u, bcap);
+// Exclusive prefix of one value per thread over the block (thread order); the total in *total.
+template <int NTH>
+__device__ __forceinline__ unsigned long long block_prefix(unsigned long long v, unsigned long long* total) {
+  __shared__ unsigned long long warp_sum[NTH / 32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  unsigned long long incl = v;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const unsigned long long t = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += t;
+  }
+  __syncthreads();  // warp_sum may still be read by a previous call
+  if (lane == 31) warp_sum[warp] = incl;
+  __syncthreads();
+  unsigned long long before = 0, all = 0;
+#pragma unroll
+  for (int w = 0; w < NTH / 32; ++w) {
+    const unsigned long long t = warp_sum[w];
+    if (w < warp) before += t;
+    all += t;
+  }
+  *total = all;
+  return before + incl - v;
 }
 
 // One block: bucket capacities -> offsets (in place); fill counters cleared.
 template <int NTH>
 __device__ __forceinline__ void bucket_offsets_block(unsigned long long* bcap, unsigned long long* bfill, int nb) {
-  __shared__ unsigned long long part[NTH];
   const int per = (nb + NTH - 1) / NTH;
-  unsigned long long s = 0;
-  for (int b = threadIdx.x * per; b < min(nb, (threadIdx.x + 1) * per); ++b) s += __ldcg(&bcap[b]);
-  part[threadIdx.x] = s;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    unsigned long long run = 0;
-    for (int t = 0; t < NTH; ++t) { unsigned long long v = part[t]; part[t] = run; run += v; }
-  }
-  __syncthreads();
-  unsigned long long run = part[threadIdx.x];
-  for (int b = threadIdx.x * per; b < min(nb, (threadIdx.x + 1) * per); ++b) {
+  unsigned long long s = 0, total;
+  for (int b = threadIdx.x * per; b < min(nb, (int)(threadIdx.x + 1) * per); ++b) s += __ldcg(&bcap[b]);
+  unsigned long long run = block_prefix<NTH>(s, &total);
+  for (int b = threadIdx.x * per; b < min(nb, (int)(threadIdx.x + 1) * per); ++b) {
     unsigned long long v = __ldcg(&bcap[b]);
     bcap[b] = run;
     run += v;
     bfill[b] = 0;
   }
-}
-__global__ void __launch_bounds__(1024) k_bucket_offsets(unsigned long long* bcap, unsigned long long* bfill, int nb) {
-  bucket_offsets_block<1024>(bcap, bfill, nb);
 }
 
 // One block: the march works through the queue in chunks of `chunk` packets
@@ -623,31 +627,43 @@ __global__ void __launch_bounds__(1024) k_bucket_offsets(unsigned long long* bca
 template <int NTH>
 __device__ __forceinline__ void bucket_scan_block(const unsigned long long* bfill, unsigned long long* cpre, int nb,
                                                   DevScalars* sc, uint32_t chunk) {
-  __shared__ unsigned long long part[NTH], qpart[NTH];
   const int per = (nb + NTH - 1) / NTH;
-  unsigned long long s = 0, q = 0;
-  for (int b = threadIdx.x * per; b < min(nb, (threadIdx.x + 1) * per); ++b) {
+  unsigned long long s = 0, q = 0, chunks, queued;
+  for (int b = threadIdx.x * per; b < min(nb, (int)(threadIdx.x + 1) * per); ++b) {
     const unsigned long long f = __ldcg(&bfill[b]);
     s += (f + chunk - 1) / chunk;
     q += f;
   }
-  part[threadIdx.x] = s;
-  qpart[threadIdx.x] = q;
-  __syncthreads();
+  unsigned long long run = block_prefix<NTH>(s, &chunks);
+  block_prefix<NTH>(q, &queued);
   if (threadIdx.x == 0) {
-    unsigned long long run = 0, qt = 0;
-    for (int t = 0; t < NTH; ++t) { unsigned long long v = part[t]; part[t] = run; run += v; qt += qpart[t]; }
-    cpre[nb] = run;
-    sc->qtail = qt;
+    cpre[nb] = chunks;
+    sc->qtail = queued;
     sc->march_next = 0;
     sc->requeued = 0;
   }
-  __syncthreads();
-  unsigned long long run = part[threadIdx.x];
-  for (int b = threadIdx.x * per; b < min(nb, (threadIdx.x + 1) * per); ++b) {
+  for (int b = threadIdx.x * per; b < min(nb, (int)(threadIdx.x + 1) * per); ++b) {
     cpre[b] = run;
     run += (__ldcg(&bfill[b]) + chunk - 1) / chunk;
   }
+}
+// The last block to finish turns the bucket capacities into offsets.
+template <class R, int IT>
+__global__ void __launch_bounds__(AT) k_alloc_prefix(const R* emis, int64_t n3, uint64_t n_packets, DevScalars* sc,
+                                                     const unsigned long long* partQ, uint32_t* P, uint32_t* first,
+                                                     Tiles tl, unsigned long long* bcap, unsigned long long* bfill,
+                                                     int nb) {
+  const int64_t c0 = (int64_t)blockIdx.x * (AT * IT) + (int64_t)threadIdx.x * IT;
+  alloc_prefix_block<R, IT>(emis, n3, n_packets, sc->sumQ, sc->alloc_u, (R)sc->rmax, partQ[blockIdx.x], c0, P, first,
+                            tl, 0u, bcap);
+  if (!last_block_done(&sc->alloc_counter)) return;
+  bucket_offsets_block<AT>(bcap, bfill, nb);
+  if (threadIdx.x == 0) sc->alloc_counter = 0;
+}
+
+// The launches of their own of a batch without the persistent front.
+__global__ void __launch_bounds__(1024) k_bucket_offsets(unsigned long long* bcap, unsigned long long* bfill, int nb) {
+  bucket_offsets_block<1024>(bcap, bfill, nb);
 }
 __global__ void __launch_bounds__(1024) k_bucket_scan(const unsigned long long* bfill, unsigned long long* cpre, int nb,
                                                       DevScalars* sc, uint32_t chunk) {
@@ -685,7 +701,7 @@ struct TransportArgs {
   int nb;                          // buckets (super-tiles)
   unsigned long long* boff;        // bucket start in the queue (capacity prefix)
   unsigned long long* bfill;       // packets queued per bucket
-  const unsigned long long* cpre;  // first march chunk of each bucket [nb + 1]
+  unsigned long long* cpre;        // first march chunk of each bucket [nb + 1]
   uint32_t chunk;                  // queued packets per march chunk
   int refill;                      // idle lanes of a warp that trigger a refill
   // region sweeps (single box, power-of-two side)
@@ -694,6 +710,7 @@ struct TransportArgs {
   unsigned long long* rqn;         // entries appended per part of the second queue [kRqParts]
   uint64_t rq_part;                // entries one part holds
   uint32_t halo;                   // region of a bucket: its super-tile and halo cells around it; 0: no limit
+  int closes;                      // this march is the call's last
   int resumed;                     // the queue holds full states of an earlier sweep (3 vectors per entry)
   // compact velocity copy (rec_velq.cuh) and its index masks
   const uint32_t* velq;
@@ -1221,6 +1238,10 @@ __global__ void __launch_bounds__(TT, emit_occupancy<R>()) k_emit(TransportArgs<
     emit_window64<R, P2>(a, e, st, (uint32_t)base, N, head, count, my_abs, my_cross);
   emit_flush<R, P2>(a, e, st, head, count, my_abs, my_cross);
   add_counters(a.sc, my_abs, 0, my_cross);
+  // the last block to finish prepares the march's chunks
+  if (!last_block_done(&a.sc->counter)) return;
+  bucket_scan_block<TT>(a.bfill, a.cpre, a.nb, a.sc, a.chunk);
+  if (threadIdx.x == 0) a.sc->counter = 0;
 }
 
 // March of the queued packets.  Persistent warps take chunks of a.chunk queued
@@ -1229,7 +1250,7 @@ __global__ void __launch_bounds__(TT, emit_occupancy<R>()) k_emit(TransportArgs<
 // they touch stay close in memory; each warp refills its idle lanes from its
 // current chunk, so that lanes stay busy whatever the spread of path lengths.
 //
-// A lane walks kMarchAhead cells per round.  For every cell it asks the bound of
+// A lane walks a few cells per round.  For every cell it asks the bound of
 // rec_velq.cuh, one 32-bit word of the compact velocity copy and one integer dot
 // product, whether the packet can be absorbed there at all; a cell whose
 // threshold exceeds any possible dot product is not even loaded.  A lane with
@@ -1237,7 +1258,10 @@ __global__ void __launch_bounds__(TT, emit_occupancy<R>()) k_emit(TransportArgs<
 // parked ones read the exact velocity of their candidate and take the exact
 // resonance test (tally and done, or on to the rest of the round), and the idle
 // ones take new packets, so that both run with many lanes at once.
-constexpr int kMarchAhead = 4;
+// Cells a lane walks per round, with their words in flight together (256^3 mixed: 3 / 4 /
+// 5 / 6 cells 4.07 / 3.57 / 3.60 / 3.43 ms, 8 cells 3.69 at three blocks per SM; FP64: 4 / 6
+// cells 7.97 / 8.28 ms).
+template <class R> struct MarchAhead { static constexpr int value = sizeof(R) == 4 ? 6 : 4; };
 
 // Resident blocks per SM of the march (register budget per thread; a batch
 // keeps the box of each lane's packet in registers).
@@ -1264,6 +1288,15 @@ __device__ __forceinline__ void load_word(uint32_t& w, const uint32_t* q, uint32
       : "+r"(w)
       : "l"(q), "r"(cell), "r"(thr), "r"(top));
 }
+
+// Loads that are not used again: past L1, which the words then have to themselves
+// (256^3: 3.43 -> 3.38 ms; a batch, short of registers, keeps plain loads).
+__device__ __forceinline__ float4 ld_stream(const float4* p) {
+  float4 v;
+  asm("ld.global.nc.L1::no_allocate.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ double4_32a ld_stream(const double4_32a* p) { return *p; }
 
 // One cell of the walk: returns the exit distance (the nearest face, ties
 // broken x < y < z) and steps across that face: its next distance, and its part
@@ -1323,6 +1356,23 @@ __device__ __forceinline__ R walk_step_any(R& tMx, R& tMy, R& tMz, R tDx, R tDy,
   return s;
 }
 
+// End of a transport call of a single box (one thread; the counters were added by
+// other blocks' atomics: read through L2).
+__device__ __forceinline__ void transport_end(DevScalars* sc, rec_stats* st) {
+  const unsigned long long absorbed = __ldcg(&sc->absorbed), capped = __ldcg(&sc->capped);
+  sc->tally_total = __ldcg(&sc->tally_total) + absorbed;
+  if (capped) atomicOr(&sc->flags, 2);
+  if (st) {
+    st->emitted = __ldcg(&sc->emitted);
+    st->absorbed = absorbed;
+    st->capped = capped;
+    st->crossings = __ldcg(&sc->crossings);
+    st->queued = __ldcg(&sc->qtail);
+    st->requeued = __ldcg(&sc->requeued);
+    st->flags = __ldcg(&sc->flags);
+  }
+}
+
 __device__ __forceinline__ void transport_end_batch(const BoxDev* bxs, int B, const unsigned long long* bfill,
                                                     rec_stats* st);
 
@@ -1335,7 +1385,7 @@ __global__ void __launch_bounds__(TT, (march_occupancy<R, MB, RS>())) k_march(Tr
   static_assert(!RS || (P2 && !MB), "region sweeps: single box of power-of-two side");
   static_assert(!MB || !P2, "a batch mixes sides");
   using V = typename Vec4<R>::T;
-  constexpr int kA = kMarchAhead;
+  constexpr int kA = MarchAhead<R>::value;
   const int lane = threadIdx.x & 31;
   const uint32_t n = (uint32_t)a.n;
   // region sweeps: bucket of the open chunk (its super-tile); path length at
@@ -1351,14 +1401,12 @@ __global__ void __launch_bounds__(TT, (march_occupancy<R, MB, RS>())) k_march(Tr
   uint32_t bx = a.vbx, ln = n;
   uint32_t lastx = 0, lasty = 0, lastz = 0;
   R lkappa = a.kappa;
-  VelqBox vb;
   if (!MB) {
-    vb = velq_box(a.velq ? a.sc->vq_u : 0.0f, a.sc->vq_v, (float)a.kappa);
     lastx = velq_x(n - 1u); lasty = velq_y(n - 1u, bx); lastz = velq_z(n - 1u, bx);
   }
-  const uint64_t n_chunks = a.cpre[a.nb];
-  uint64_t pos = 0, end = 0;  // queue slots [pos, end) left in the open chunk
-  bool more = n_chunks > 0;
+  uint64_t pos = 0;   // next queue slot of the open chunk
+  uint32_t left = 0;  // slots left in it
+  bool more = true;
   bool active = false, parked = false;
   // the packet: cell (three parts of the word index), face distances, steps, resonance
   uint32_t X = 0, Y = 0, Z = 0, Sx = 0, Sy = 0, Sz = 0, Ex = 0, Ey = 0, Ez = 0, kc = 0;
@@ -1368,7 +1416,8 @@ __global__ void __launch_bounds__(TT, (march_occupancy<R, MB, RS>())) k_march(Tr
   // the last round: cells, exit distances, words, first cell not yet cleared
   uint32_t cl[kA] = {}, qw[kA] = {}, kfrom = 0;
   R se[kA] = {};
-  uint64_t my_abs = 0, my_cap = 0, my_cross = 0;
+  // counters of the lane; crossings are flushed before 32 bits could overflow
+  uint32_t my_abs = 0, my_cap = 0, my_cross = 0;
   for (;;) {
     const unsigned stop = __ballot_sync(0xffffffffu, !active || parked);
     bool fresh = false;  // region sweeps: a round was completed, check the region
@@ -1396,7 +1445,7 @@ __global__ void __launch_bounds__(TT, (march_occupancy<R, MB, RS>())) k_march(Tr
           velq_coords(c, bx, &ix, &iy, &iz);
           const uint32_t lin = (iz * ln + iy) * ln + ix;
           const V* vel = MB ? (const V*)bxs[lbox].vel4 : a.vel;
-          const V U = vel[lin];
+          const V U = MB ? vel[lin] : ld_stream(vel + lin);
           Ray<R> r;
           r.knx = knx; r.kny = kny; r.knz = knz;
           // resonance in the cell at path length u0 - kappa n.U: absorb unless beyond its exit
@@ -1405,6 +1454,11 @@ __global__ void __launch_bounds__(TT, (march_occupancy<R, MB, RS>())) k_march(Tr
           if (hit || kcell >= kMaxCrossings) {
             active = parked = false;
             my_cross += kcell - 1;  // crossings up to this cell; the first was counted at emission
+            if (my_cross >= 0x80000000u) {
+              if (MB) box_counters_add(cnt, lbox, 0, 0, my_cross);
+              else atomicAdd(&a.sc->crossings, (unsigned long long)my_cross);
+              my_cross = 0;
+            }
             if (hit) { atomicAdd((MB ? bxs[lbox].tally : a.tally) + lin, 1u); ++my_abs; }
             else ++my_cap;
           } else {
@@ -1417,14 +1471,15 @@ __global__ void __launch_bounds__(TT, (march_occupancy<R, MB, RS>())) k_march(Tr
       // refill idle lanes in lane order from the warp's chunks
       unsigned idle = __ballot_sync(0xffffffffu, !active);
       while (idle && more) {
-        if (pos >= end) {
+        if (left == 0) {
           // next chunk in queue order, shared by all warps: the warps in flight
           // stay on neighbouring chunks, so their rays start close together
           unsigned long long nc = 0;
           if (lane == 0) nc = atomicAdd(&a.sc->march_next, 1ull);
           const uint64_t chunk = __shfl_sync(0xffffffffu, nc, 0);
-          if (chunk >= n_chunks) { more = false; break; }
-          // bucket of this chunk: last b with cpre[b] <= chunk (uniform over the warp)
+          if (chunk >= __ldg(a.cpre + a.nb)) { more = false; break; }
+          // bucket of this chunk: last b with cpre[b] <= chunk (cpre[0] = 0), the lanes
+          // probing 32 places at once, so two rounds of loads for up to 1024 buckets
           uint32_t lo = 0, hi = (uint32_t)a.nb;
           while (hi - lo > 1) {
             uint32_t mid = (lo + hi) >> 1;
@@ -1433,11 +1488,11 @@ __global__ void __launch_bounds__(TT, (march_occupancy<R, MB, RS>())) k_march(Tr
           }
           const uint64_t k0 = (chunk - __ldg(a.cpre + lo)) * a.chunk;
           pos = a.boff[lo] + k0;
-          end = pos + min((uint64_t)a.chunk, (uint64_t)(a.bfill[lo] - k0));
+          left = (uint32_t)min((uint64_t)a.chunk, (uint64_t)(a.bfill[lo] - k0));
           if (RS) cbk = lo;
           if (MB) cbox = last_le(B, lo, [&](int i) { return bxs[i].bk0; });  // last b with bk0 <= lo
         }
-        const uint32_t take = (uint32_t)min((uint64_t)__popc(idle), end - pos);
+        const uint32_t take = min((uint32_t)__popc(idle), left);
         const uint32_t rank = __popc(idle & ((1u << lane) - 1u));
         if (((idle >> lane) & 1u) && rank < take) {
           const uint64_t slot = pos + rank;
@@ -1454,7 +1509,6 @@ __global__ void __launch_bounds__(TT, (march_occupancy<R, MB, RS>())) k_march(Tr
               q = d.velq;
               lkappa = (R)bst[lbox].kappa;
               lastx = velq_x(ln - 1u); lasty = velq_y(ln - 1u, bx); lastz = velq_z(ln - 1u, bx);
-              vb = velq_box(q ? d.sc->vq_u : 0.0f, d.sc->vq_v, (float)lkappa);
             }
           }
           uint32_t cell;
@@ -1471,7 +1525,8 @@ __global__ void __launch_bounds__(TT, (march_occupancy<R, MB, RS>())) k_march(Tr
             knx = q2v.x; kny = q2v.y; knz = q2v.z;
             kc = to_bits<R>(q2v.w);
           } else {
-            const V q0v = a.queue[QV * slot], q1v = a.queue[QV * slot + 1];
+            const V* entry = a.queue + QV * slot;
+            const V q0v = MB ? entry[0] : ld_stream(entry), q1v = MB ? entry[1] : ld_stream(entry + 1);
             cell = to_bits<R>(q0v.x);
             tMx = q0v.y; tMy = q0v.z; tMz = q0v.w;
             u0 = q1v.w;
@@ -1517,10 +1572,15 @@ __global__ void __launch_bounds__(TT, (march_occupancy<R, MB, RS>())) k_march(Tr
           Sy = sy > 0 ? 0u - lm.y : 0u - 2u;
           Sz = sz > 0 ? 0u - lm.z : 0u - 4u;
           if (!P2) { Ex = sx > 0 ? lastx : 0u; Ey = sy > 0 ? lasty : 0u; Ez = sz > 0 ? lastz : 0u; }
-          vp = velq_packet(vb, (float)knx, (float)kny, (float)knz, (float)u0);
+          {
+            const DevScalars* bsc = MB ? bxs[lbox].sc : a.sc;
+            const VelqBox vb = velq_box(q ? bsc->vq_u : 0.0f, bsc->vq_v, (float)lkappa);
+            vp = velq_packet(vb, (float)knx, (float)kny, (float)knz, (float)u0);
+          }
           active = true;
         }
         pos += take;
+        left -= take;
         idle = __ballot_sync(0xffffffffu, !active);
       }
     }
@@ -1597,6 +1657,12 @@ __global__ void __launch_bounds__(TT, (march_occupancy<R, MB, RS>())) k_march(Tr
     }
   } else {
     add_counters(a.sc, my_abs, my_cap, my_cross);
+    // the last block of the last march closes the call: tally total, statistics
+    if (!a.closes || !last_block_done(&a.sc->counter)) return;
+    if (threadIdx.x == 0) {
+      transport_end(a.sc, st);
+      a.sc->counter = 0;
+    }
   }
 }
 
@@ -1610,7 +1676,6 @@ __global__ void __launch_bounds__(1024) k_requeue_scan(unsigned long long* rcoun
                                                        DevScalars* sc, uint32_t chunk, uint64_t part_cap) {
   constexpr int NTH = 1024;
   static_assert(kRqParts <= NTH, "one thread per part");
-  __shared__ unsigned long long pe[NTH], pc[NTH];
   __shared__ unsigned long long stored;
   if (threadIdx.x == 0) stored = 0;
   __syncthreads();
@@ -1622,28 +1687,19 @@ __global__ void __launch_bounds__(1024) k_requeue_scan(unsigned long long* rcoun
   }
   const int per = (nb + NTH - 1) / NTH;
   const int b0 = threadIdx.x * per, b1 = min(nb, (int)(threadIdx.x + 1) * per);
-  unsigned long long se = 0, sc_ = 0;
+  unsigned long long se = 0, sc_ = 0, all, chunks;
   for (int b = b0; b < b1; ++b) {
     const unsigned long long f = __ldcg(&rcount[b]);
     se += f;
     sc_ += (f + chunk - 1) / chunk;
   }
-  pe[threadIdx.x] = se;
-  pc[threadIdx.x] = sc_;
-  __syncthreads();
+  unsigned long long re = block_prefix<NTH>(se, &all);
+  unsigned long long rc = block_prefix<NTH>(sc_, &chunks);
   if (threadIdx.x == 0) {
-    unsigned long long re = 0, rc = 0;
-    for (int t = 0; t < NTH; ++t) {
-      const unsigned long long ve = pe[t], vc = pc[t];
-      pe[t] = re; pc[t] = rc;
-      re += ve; rc += vc;
-    }
-    cpre[nb] = rc;
+    cpre[nb] = chunks;
     sc->requeued += stored;
     sc->march_next = 0;
   }
-  __syncthreads();
-  unsigned long long re = pe[threadIdx.x], rc = pc[threadIdx.x];
   for (int b = b0; b < b1; ++b) {
     const unsigned long long f = __ldcg(&rcount[b]);
     boff[b] = re;
@@ -1690,21 +1746,6 @@ __global__ void __launch_bounds__(TT) k_requeue_place(TransportArgs<R> a, unsign
   }
 }
 
-__global__ void k_transport_end(DevScalars* sc, rec_stats* st) {
-  if (threadIdx.x != 0) return;
-  sc->tally_total += sc->absorbed;
-  if (sc->capped) sc->flags |= 2;
-  if (st) {
-    st->emitted = sc->emitted;
-    st->absorbed = sc->absorbed;
-    st->capped = sc->capped;
-    st->crossings = sc->crossings;
-    st->queued = sc->qtail;
-    st->requeued = sc->requeued;
-    st->flags = sc->flags;
-  }
-}
-
 // Consecutive cells per thread of the single-box allocation: few for small
 // boxes, whose time is one thread's serial chain (quotients, remainders) on a
 // part of the chip, many for large ones, where the passes stream and the
@@ -1718,8 +1759,8 @@ void alloc_launch(rec_ctx* c, int blocks, const typename Vec4<R>::T* vel, const 
   const uint64_t npk = c->box.n_packets;
   k_alloc_sum<R, IT><<<blocks, AT, 0, c->stream>>>(emis, vel, c->n3, npk, s, c->sc, c->partQ, c->P, c->velq,
                                                    velq_bits((uint32_t)c->box.n), tl);
-  cudaMemsetAsync(c->bcap, 0, sizeof(unsigned long long) * nb, c->stream);
-  k_alloc_prefix<R, IT><<<blocks, AT, 0, c->stream>>>(emis, c->n3, npk, c->sc, c->partQ, c->P, c->first, tl, c->bcap);
+  k_alloc_prefix<R, IT><<<blocks, AT, 0, c->stream>>>(emis, c->n3, npk, c->sc, c->partQ, c->P, c->first, tl, c->bcap,
+                                                      c->bfill, nb);
 }
 
 // Bound of the quantile's leading word w below which xi <= 0 (0: none).  The deviate
@@ -1744,14 +1785,13 @@ cudaError_t run_transport(rec_ctx* c, int step, double z, rec_stats* st) {
   double kappa, cth;
   transport_scalars(c->cosmo, b.n, z, &kappa, &cth);
   {
-    GroupTimer t(c, kTAlloc, 4);
+    GroupTimer t(c, kTAlloc, 3);
     const typename Vec4<R>::T* vel = (const typename Vec4<R>::T*)b.vel4;
-    k_alloc_max<R><<<c->grid, kPassThreads, 0, c->stream>>>((const R*)b.emis, vel, c->n3, (float)kappa, c->sc);
+    k_alloc_max<R><<<c->grid, kPassThreads, 0, c->stream>>>((const R*)b.emis, vel, c->n3, (float)kappa, c->sc, c->bcap, nb);
     const int it = alloc_items(c->n3), ab = c->alloc_blocks;
     if (it == 1) alloc_launch<R, 1>(c, ab, vel, s, tl, nb);
     else if (it == 4) alloc_launch<R, 4>(c, ab, vel, s, tl, nb);
     else alloc_launch<R, kAllocItems>(c, ab, vel, s, tl, nb);
-    k_bucket_offsets<<<1, 1024, 0, c->stream>>>(c->bcap, c->bfill, nb);
   }
   TransportArgs<R> a;
   a.P = c->P;
@@ -1783,23 +1823,23 @@ cudaError_t run_transport(rec_ctx* c, int step, double z, rec_stats* st) {
   a.rq_part = 0;
   a.halo = 0;
   a.resumed = 0;
+  a.closes = 1;
   a.velq = c->velq;
   a.vbx = velq_bits((uint32_t)b.n);
   a.vm = velq_masks((uint32_t)b.n, a.vbx, p2);
   {
-    GroupTimer t(c, kTEmit, 2);
+    GroupTimer t(c, kTEmit, 1);
     const int eb = c->sm_count * tu.emit_blocks_per_sm;
     if (p2) k_emit<R, true><<<eb, TT, 0, c->stream>>>(a);
     else k_emit<R, false><<<eb, TT, 0, c->stream>>>(a);
-    k_bucket_scan<<<1, 1024, 0, c->stream>>>(c->bfill, c->cpre, nb, c->sc, a.chunk);
   }
   const uint32_t halo = (uint32_t)tu.march_halo;
   const bool sweeps = p2 && halo > 0 && c->rqueue && ((uint32_t)tu.tile + 2u * halo) < (uint32_t)b.n;
   if (!sweeps) {
     GroupTimer t(c, kTMarch, 1);
     const int mb = c->sm_count * tu.march_blocks_per_sm;
-    if (p2) k_march<R, true, false><<<mb, TT, 0, c->stream>>>(a, nullptr, 1, nullptr, nullptr);
-    else k_march<R, false, false><<<mb, TT, 0, c->stream>>>(a, nullptr, 1, nullptr, nullptr);
+    if (p2) k_march<R, true, false><<<mb, TT, 0, c->stream>>>(a, nullptr, 1, nullptr, st);
+    else k_march<R, false, false><<<mb, TT, 0, c->stream>>>(a, nullptr, 1, nullptr, st);
   } else {
     // region sweeps: each march leaves the packets that stray beyond the halo of
     // their bucket's super-tile in the second queue; those are placed by the
@@ -1819,13 +1859,10 @@ cudaError_t run_transport(rec_ctx* c, int step, double z, rec_stats* st) {
         k_requeue_place<R><<<kRqParts, TT, 0, c->stream>>>(a, c->scnt);
       }
       a.resumed = k > 0;
-      a.halo = (k + 1 < kMaxSweeps) ? halo : 0u;
-      k_march<R, true, false, true><<<mb, TT, 0, c->stream>>>(a, nullptr, 1, nullptr, nullptr);
+      a.closes = k + 1 == kMaxSweeps;
+      a.halo = a.closes ? 0u : halo;
+      k_march<R, true, false, true><<<mb, TT, 0, c->stream>>>(a, nullptr, 1, nullptr, st);
     }
-  }
-  {
-    GroupTimer t(c, kTEnd, 1);
-    k_transport_end<<<1, 32, 0, c->stream>>>(c->sc, st);
   }
   return cudaGetLastError();
 }
