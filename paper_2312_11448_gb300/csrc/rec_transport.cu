@@ -362,6 +362,9 @@ struct Tiles {
   __device__ __forceinline__ uint32_t at(uint32_t cell) const {
     uint32_t ix, iy, iz;
     coords<P2>(cell, &ix, &iy, &iz);
+    return tile_of(ix, iy, iz);
+  }
+  __device__ __forceinline__ uint32_t tile_of(uint32_t ix, uint32_t iy, uint32_t iz) const {
     return ((iz >> tlg) * nt + (iy >> tlg)) * nt + (ix >> tlg);
   }
   __device__ __forceinline__ uint32_t of(uint32_t cell) const { return at<false>(cell); }
@@ -1015,6 +1018,8 @@ __device__ __forceinline__ void emit_rest(const TransportArgs<R>& a, const EmitB
   bool home = false, queued = false;
   Ray<R> r;
   R nx = zero, ny = zero, nz = one;
+  e.tl.template coords<P2>(cell, &r.ix, &r.iy, &r.iz);
+  const uint32_t bk = e.bk0 + e.tl.tile_of(r.ix, r.iy, r.iz);  // bucket of the home cell
   if (act) {
     const KStream ks{a.ks, e.box};
     // isotropic direction (Marsaglia 1972): the first accepted of the candidate
@@ -1053,7 +1058,6 @@ __device__ __forceinline__ void emit_rest(const TransportArgs<R>& a, const EmitB
     V Uh = e.vel[cell];
     const R dh = doppler(r, Uh);
     r.u0 = A::add(A::mul(xi, vt), dh);
-    e.tl.template coords<P2>(cell, &r.ix, &r.iy, &r.iz);
     axis_setup<R>(nx, &r.tDx, &r.sx);
     axis_setup<R>(ny, &r.tDy, &r.sy);
     axis_setup<R>(nz, &r.tDz, &r.sz);
@@ -1080,7 +1084,6 @@ __device__ __forceinline__ void emit_rest(const TransportArgs<R>& a, const EmitB
   // queue the others after their first step, in their home super-tile's bucket
   const unsigned qm = __ballot_sync(0xffffffffu, queued);
   if (qm) {
-    const uint32_t bk = e.bk0 + e.tl.template at<P2>(cell);
     const unsigned gm = key_group(bk) & qm;
     unsigned long long qb = 0;
     const int leader = __ffs(gm) - 1;
@@ -1339,17 +1342,45 @@ __device__ __forceinline__ double walk_step(double& tMx, double& tMy, double& tM
   if (pz) { tMz = t; Z = (Z + Sz) & mz; }
   return s;
 }
-// Sides that are no power of two: the last cell in the direction of travel
-// (end) steps to the first one (last ^ end, since one of the two is offset 0),
-// set up beforehand as an addition, since the mask would not wrap there.
-template <class R>
-__device__ __forceinline__ R walk_step_any(R& tMx, R& tMy, R& tMz, R tDx, R tDy, R tDz, uint32_t& X, uint32_t& Y,
-                                           uint32_t& Z, uint32_t Sx, uint32_t Sy, uint32_t Sz, uint32_t mx,
-                                           uint32_t my, uint32_t mz, uint32_t Ex, uint32_t Ey, uint32_t Ez,
-                                           uint32_t lx, uint32_t ly, uint32_t lz) {
+// Sides that are no power of two: from the last cell in the direction of travel
+// (end, offset E) the step goes to the first one (last ^ E, since one of the two is
+// offset 0), where the mask would not wrap.
+__device__ __forceinline__ float walk_step_any(float& tMx, float& tMy, float& tMz, float tDx, float tDy, float tDz,
+                                               uint32_t& X, uint32_t& Y, uint32_t& Z, uint32_t Sx, uint32_t Sy,
+                                               uint32_t Sz, uint32_t mx, uint32_t my, uint32_t mz, uint32_t Ex,
+                                               uint32_t Ey, uint32_t Ez, uint32_t lx, uint32_t ly, uint32_t lz) {
+  float s;
+  asm("{\n\t.reg .pred px, py, pz, ex, ey, ez;\n\t"
+      "min.f32 %0, %1, %2, %3;\n\t"
+      "setp.eq.f32 px, %1, %0;\n\t"
+      "setp.eq.and.f32 py|pz, %2, %0, !px;\n\t"
+      "@px add.rn.f32 %1, %1, %7;\n\t"
+      "@py add.rn.f32 %2, %2, %8;\n\t"
+      "@pz add.rn.f32 %3, %3, %9;\n\t"
+      "setp.eq.and.u32 ex, %4, %16, px;\n\t"
+      "setp.eq.and.u32 ey, %5, %17, py;\n\t"
+      "setp.eq.and.u32 ez, %6, %18, pz;\n\t"
+      "@px add.u32 %4, %4, %10;\n\t"
+      "@py add.u32 %5, %5, %11;\n\t"
+      "@pz add.u32 %6, %6, %12;\n\t"
+      "@px and.b32 %4, %4, %13;\n\t"
+      "@py and.b32 %5, %5, %14;\n\t"
+      "@pz and.b32 %6, %6, %15;\n\t"
+      "@ex xor.b32 %4, %16, %19;\n\t"
+      "@ey xor.b32 %5, %17, %20;\n\t"
+      "@ez xor.b32 %6, %18, %21;\n\t}"
+      : "=&f"(s), "+f"(tMx), "+f"(tMy), "+f"(tMz), "+r"(X), "+r"(Y), "+r"(Z)
+      : "f"(tDx), "f"(tDy), "f"(tDz), "r"(Sx), "r"(Sy), "r"(Sz), "r"(mx), "r"(my), "r"(mz), "r"(Ex), "r"(Ey), "r"(Ez),
+        "r"(lx), "r"(ly), "r"(lz));
+  return s;
+}
+__device__ __forceinline__ double walk_step_any(double& tMx, double& tMy, double& tMz, double tDx, double tDy,
+                                                double tDz, uint32_t& X, uint32_t& Y, uint32_t& Z, uint32_t Sx,
+                                                uint32_t Sy, uint32_t Sz, uint32_t mx, uint32_t my, uint32_t mz,
+                                                uint32_t Ex, uint32_t Ey, uint32_t Ez, uint32_t lx, uint32_t ly,
+                                                uint32_t lz) {
   const uint32_t x0 = X, y0 = Y, z0 = Z;
-  const R s = walk_step(tMx, tMy, tMz, tDx, tDy, tDz, X, Y, Z, Sx, Sy, Sz, mx, my, mz);
-  // one axis moved; from its end the masked step left a wrong offset
+  const double s = walk_step(tMx, tMy, tMz, tDx, tDy, tDz, X, Y, Z, Sx, Sy, Sz, mx, my, mz);
   if (X != x0 && x0 == Ex) X = lx ^ Ex;
   if (Y != y0 && y0 == Ey) Y = ly ^ Ey;
   if (Z != z0 && z0 == Ez) Z = lz ^ Ez;
