@@ -54,6 +54,8 @@ struct DevScalars {
   unsigned long long emitted, absorbed, capped, crossings;
   unsigned long long tally_total;  // packets absorbed in the current tallies
   unsigned long long sumQ;         // sum of quantised emission weights
+  unsigned long long div_v, div_m; // sumQ as a divisor: reciprocal words and normalising shift
+  int32_t div_shift;
   unsigned long long alloc_u;      // systematic-sampling offset in [0, sumQ)
   unsigned long long qtail;        // packets queued for the march
   unsigned long long march_next;   // next queue chunk handed to a march warp

@@ -291,6 +291,7 @@ __global__ void __launch_bounds__(kPassThreads) k_alloc_max(const R* emis, const
   bool bad = false;
   VelMax vm;
   for (int i = blockIdx.x * kPassThreads + threadIdx.x; i < nb; i += gridDim.x * kPassThreads) bcap[i] = 0ull;
+#pragma unroll 4
   for (int64_t i = (int64_t)blockIdx.x * kPassThreads + threadIdx.x; i < n3; i += (int64_t)gridDim.x * kPassThreads) {
     const R r = emis[i];
     if (!(r >= (R)0) || isinf(r)) bad = true;
@@ -312,6 +313,10 @@ __device__ __forceinline__ uint64_t quantised(R r, R rmax) {
   // 64-bit one without the 64-bit conversion (a binary64-pipe instruction).
   return (uint64_t)(uint32_t)Ar<R>::mul(Ar<R>::div(r, rmax), (R)2147483648.0);
 }
+
+// The FP64 form keeps Q (at most 2^31) in the prefix array between its two passes: a
+// binary64 quotient per cell costs 16 us of the slow pipe per 1e6 cells.
+template <class R> constexpr bool kKeepQ = sizeof(R) == 8;
 
 // Inclusive block scan of 64-bit counts (thread order); returns the block total.
 __device__ __forceinline__ uint64_t block_scan_incl(uint64_t v, uint64_t* incl) {
@@ -367,7 +372,8 @@ struct Tiles {
   __device__ __forceinline__ uint32_t tile_of(uint32_t ix, uint32_t iy, uint32_t iz) const {
     return ((iz >> tlg) * nt + (iy >> tlg)) * nt + (ix >> tlg);
   }
-  __device__ __forceinline__ uint32_t of(uint32_t cell) const { return at<false>(cell); }
+  // lg = 0: no power of two (or one cell, which the divisions take as well)
+  __device__ __forceinline__ uint32_t of(uint32_t cell) const { return lg ? at<true>(cell) : at<false>(cell); }
 };
 
 // Multiplier ceil(2^64 / d) of the exact 32-bit division by d >= 2.
@@ -390,6 +396,50 @@ inline Tiles make_tiles(int n, int tile) {
   return t;
 }
 
+// The sum S > 0 of the weights as a divisor, prepared once per call: its
+// normalised form d = S 2^shift (top bit set) with the reciprocal word
+// v = floor((2^128 - 1) / d) - 2^64 of Moeller & Granlund, "Improved division by
+// invariant integers" (IEEE Trans. Comput. 60, 165 (2011)), and m = floor((2^64 - 1) / S).
+__device__ __forceinline__ void set_divisor(DevScalars* sc, uint64_t S) {
+  sc->sumQ = S;
+  if (S == 0) return;
+  const int k = __clzll((long long)S);
+  const uint64_t d = S << k;
+  // v = floor((2^128 - 1 - 2^64 d) / d): long division of (2^64 - 1 - d) 2^64 + (2^64 - 1) by d, bit by bit
+  uint64_t r = ~0ull - d, v = 0;
+  for (int i = 0; i < 64; ++i) {
+    const uint64_t top = r >> 63;
+    r = (r << 1) | 1ull;
+    v <<= 1;
+    if (top || r >= d) { r -= d; v |= 1ull; }
+  }
+  sc->div_shift = k;
+  sc->div_v = v;
+  sc->div_m = ~0ull / S;
+}
+struct Divisor {
+  uint64_t S, v, m;
+  int shift;
+};
+
+// floor((N * pre + u) / S) and the remainder, for N < 2^32, pre <= S < 2^63, u < S:
+// their algorithm 4 (two words by one) in integers.
+__device__ __forceinline__ uint32_t sys_floor(uint64_t N, uint64_t pre, uint64_t u, const Divisor& dv, uint64_t* rem) {
+  uint64_t lo = N * pre, hi = __umul64hi(N, pre);
+  lo += u;
+  hi += lo < u;
+  const int k = dv.shift;  // >= 1: S < 2^63
+  const uint64_t d = dv.S << k, u1 = (hi << k) | (lo >> (64 - k)), u0 = lo << k;
+  uint64_t q0 = dv.v * u1, q1 = __umul64hi(dv.v, u1);
+  q0 += u0;
+  q1 += u1 + (q0 < u0) + 1ull;
+  uint64_t r = u0 - q1 * d;
+  if (r > q0) { --q1; r += d; }
+  if (r >= d) { ++q1; r -= d; }
+  *rem = r >> k;
+  return (uint32_t)q1;
+}
+
 // Compact copy of the velocities of AT * IT consecutive cells (one block).
 template <class R, int IT, class V>
 __device__ __forceinline__ void velq_write(const V* vel, int64_t n3, int64_t c0, float u, uint32_t* velq, uint32_t bx,
@@ -402,7 +452,8 @@ __device__ __forceinline__ void velq_write(const V* vel, int64_t n3, int64_t c0,
     if (i >= n3) break;
     const V U = vel[i];
     uint32_t ix, iy, iz;
-    tl.template coords<false>((uint32_t)i, &ix, &iy, &iz);
+    if (tl.lg) tl.template coords<true>((uint32_t)i, &ix, &iy, &iz);
+    else tl.template coords<false>((uint32_t)i, &ix, &iy, &iz);
     velq[velq_x(ix) | velq_y(iy, bx) | velq_z(iz, bx)] =
         velq_pack(velq_value(U.x), velq_value(U.y), velq_value(U.z), qs);
   }
@@ -443,9 +494,14 @@ __global__ void __launch_bounds__(AT) k_alloc_sum(const R* emis, const typename 
   uint64_t acc = 0;
   if (rmax > (R)0) {
     R v[IT];
-    load_items<R, IT>(emis, (int64_t)blockIdx.x * (AT * IT) + (int64_t)threadIdx.x * IT, n3, v);
+    const int64_t c0 = (int64_t)blockIdx.x * (AT * IT) + (int64_t)threadIdx.x * IT;
+    load_items<R, IT>(emis, c0, n3, v);
 #pragma unroll
-    for (int k = 0; k < IT; ++k) acc += quantised<R>(v[k], rmax);
+    for (int k = 0; k < IT; ++k) {
+      const uint64_t q = quantised<R>(v[k], rmax);
+      acc += q;
+      if (kKeepQ<R> && c0 + k < n3) P[c0 + k] = (uint32_t)q;
+    }
   }
   uint64_t incl;
   uint64_t tot = block_scan_incl(acc, &incl);
@@ -468,7 +524,7 @@ __global__ void __launch_bounds__(AT) k_alloc_sum(const R* emis, const typename 
     U4 r = draw(strm, 0u, 0u, kAllocBlock);
     uint64_t w = ((uint64_t)r.b << 32) | r.a;
     uint64_t npk = (sumQ > 0) ? n_packets : 0;
-    sc->sumQ = sumQ;
+    set_divisor(sc, sumQ);
     sc->alloc_u = sumQ > 0 ? w % sumQ : 0;
     P[n3] = (uint32_t)npk;
     sc->emitted = npk;
@@ -479,28 +535,6 @@ __global__ void __launch_bounds__(AT) k_alloc_sum(const R* emis, const typename 
     sc->alloc_counter = 0;
     if (sumQ == 0 && n_packets > 0) sc->flags |= 4;
   }
-}
-
-// floor((N * pre + u) / S) and the remainder, for N < 2^32, pre <= S < 2^64,
-// u < S: a binary64 estimate corrected with exact 128-bit products.
-__device__ __forceinline__ uint32_t sys_floor(uint64_t N, uint64_t pre, uint64_t u, uint64_t S, uint64_t* rem) {
-  uint64_t lo = N * pre, hi = __umul64hi(N, pre);
-  uint64_t lo2 = lo + u;
-  hi += (lo2 < lo);
-  lo = lo2;
-  double est = ((double)hi * 18446744073709551616.0 + (double)lo) / (double)S;
-  uint64_t q = (uint64_t)est;
-  if (q > N) q = N;
-  for (;;) {  // q S > X ?
-    uint64_t plo = q * S, phi = __umul64hi(q, S);
-    if (phi > hi || (phi == hi && plo > lo)) { --q; continue; }
-    // X - q S >= S ?
-    uint64_t rlo = lo - plo, rhi = hi - phi - (lo < plo);
-    if (rhi > 0 || rlo >= S) { ++q; continue; }
-    *rem = rlo;
-    break;
-  }
-  return (uint32_t)q;
 }
 
 // floor(t / S) and t mod S for t < 2^64, given m = floor((2^64 - 1) / S): the
@@ -523,13 +557,20 @@ __device__ __forceinline__ uint64_t div_small(uint64_t t, uint64_t S, uint64_t m
 // range, so a warp of 32 consecutive packets finds its first cell with one
 // load) and the packets per super-tile (the capacity of its march-queue bucket).
 template <class R, int IT>
-__device__ __forceinline__ void alloc_prefix_block(const R* emis, int64_t n3, uint64_t n_packets, uint64_t S,
+__device__ __forceinline__ void alloc_prefix_block(const R* emis, int64_t n3, uint64_t n_packets, const Divisor& dv,
                                                    uint64_t u, R rmax, uint64_t pre_block, int64_t c0, uint32_t* P,
                                                    uint32_t* first, const Tiles& tl, uint32_t bk0,
                                                    unsigned long long* bcap) {
+  const uint64_t S = dv.S;
   uint64_t Q[IT];
   uint64_t acc = 0;
-  {
+  if (kKeepQ<R>) {  // left in P by the pass before
+#pragma unroll
+    for (int k = 0; k < IT; ++k) {
+      Q[k] = (rmax > (R)0 && c0 + k < n3) ? __ldcg(P + c0 + k) : 0u;
+      acc += Q[k];
+    }
+  } else {
     R v[IT];
     load_items<R, IT>(emis, c0, n3, v);
 #pragma unroll
@@ -547,8 +588,8 @@ __device__ __forceinline__ void alloc_prefix_block(const R* emis, int64_t n3, ui
     for (int k = 0; k < IT; ++k) out[k] = 0u;
   } else {
     uint64_t rem;
-    uint32_t pk = sys_floor(n_packets, pre_block + incl - acc, u, S, &rem);
-    const uint64_t minv = ~0ull / S;
+    uint32_t pk = sys_floor(n_packets, pre_block + incl - acc, u, dv, &rem);
+    const uint64_t minv = dv.m;
 #pragma unroll
     for (int k = 0; k < IT; ++k) {
       out[k] = pk;
@@ -652,13 +693,13 @@ __device__ __forceinline__ void bucket_scan_block(const unsigned long long* bfil
 }
 // The last block to finish turns the bucket capacities into offsets.
 template <class R, int IT>
-__global__ void __launch_bounds__(AT) k_alloc_prefix(const R* emis, int64_t n3, uint64_t n_packets, DevScalars* sc,
+__global__ void __launch_bounds__(AT, 3) k_alloc_prefix(const R* emis, int64_t n3, uint64_t n_packets, DevScalars* sc,
                                                      const unsigned long long* partQ, uint32_t* P, uint32_t* first,
                                                      Tiles tl, unsigned long long* bcap, unsigned long long* bfill,
                                                      int nb) {
   const int64_t c0 = (int64_t)blockIdx.x * (AT * IT) + (int64_t)threadIdx.x * IT;
-  alloc_prefix_block<R, IT>(emis, n3, n_packets, sc->sumQ, sc->alloc_u, (R)sc->rmax, partQ[blockIdx.x], c0, P, first,
-                            tl, 0u, bcap);
+  alloc_prefix_block<R, IT>(emis, n3, n_packets, Divisor{sc->sumQ, sc->div_v, sc->div_m, sc->div_shift}, sc->alloc_u,
+                            (R)sc->rmax, partQ[blockIdx.x], c0, P, first, tl, 0u, bcap);
   if (!last_block_done(&sc->alloc_counter)) return;
   bucket_offsets_block<AT>(bcap, bfill, nb);
   if (threadIdx.x == 0) sc->alloc_counter = 0;
@@ -1961,7 +2002,11 @@ __device__ __forceinline__ void alloc_sum_batch(const BoxDev* bxs, int B, uint32
     R v[kAllocItems];
     load_items<R, kAllocItems>((const R*)d.emis, c0, d.n3, v);
 #pragma unroll
-    for (int k = 0; k < kAllocItems; ++k) acc += quantised<R>(v[k], rmax);
+    for (int k = 0; k < kAllocItems; ++k) {
+      const uint64_t q = quantised<R>(v[k], rmax);
+      acc += q;
+      if (kKeepQ<R> && c0 + k < d.n3) d.P[c0 + k] = (uint32_t)q;
+    }
   }
   uint64_t incl;
   uint64_t tot = block_scan_incl(acc, &incl);
@@ -1992,7 +2037,7 @@ __device__ __forceinline__ void alloc_sum_batch(const BoxDev* bxs, int B, uint32
       U4 r = draw(Stream{k0, k1, (uint32_t)i}, 0u, 0u, kAllocBlock);
       uint64_t w = ((uint64_t)r.b << 32) | r.a;
       uint64_t npk = (sumQ > 0) ? e.npk : 0;
-      sc->sumQ = sumQ;
+      set_divisor(sc, sumQ);
       sc->alloc_u = sumQ > 0 ? w % sumQ : 0;
       e.P[e.n3] = (uint32_t)npk;
       sc->emitted = npk;
@@ -2018,8 +2063,10 @@ __device__ __forceinline__ void alloc_prefix_batch(const BoxDev* bxs, int B, con
   const BoxDev& d = bxs[b];
   const DevScalars* sc = d.sc;
   const int64_t c0 = (int64_t)(g - d.ablk0) * kAllocChunk + (int64_t)threadIdx.x * kAllocItems;
-  alloc_prefix_block<R, kAllocItems>((const R*)d.emis, d.n3, d.npk, __ldcg(&sc->sumQ), __ldcg(&sc->alloc_u), (R)__ldcg(&sc->rmax),
-                        __ldcg(&partQ[g]), c0, d.P, d.first, Tiles{d.n, d.nt, d.lg, d.mn, d.mn2, d.tlg}, d.bk0, bcap);
+  const Divisor dv{__ldcg(&sc->sumQ), __ldcg(&sc->div_v), __ldcg(&sc->div_m), __ldcg(&sc->div_shift)};
+  alloc_prefix_block<R, kAllocItems>((const R*)d.emis, d.n3, d.npk, dv, __ldcg(&sc->alloc_u), (R)__ldcg(&sc->rmax),
+                                     __ldcg(&partQ[g]), c0, d.P, d.first,
+                                     Tiles{d.n, d.nt, d.lg, d.mn, d.mn2, d.tlg}, d.bk0, bcap);
 }
 template <class R>
 __global__ void __launch_bounds__(AT) k_alloc_prefix_batch(const BoxDev* bxs, int B, const unsigned long long* partQ,
