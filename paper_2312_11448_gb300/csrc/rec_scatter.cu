@@ -389,7 +389,9 @@ __device__ __forceinline__ CellCoords cell_coords(const double p[3]) {
   return CellCoords{floor_bits(p[0]), floor_bits(p[1]), floor_bits(p[2])};
 }
 
-constexpr int kSteps = 4;  // steps of a photon between votes of its warp
+// Steps of a photon between votes of its warp: 3 / 4 / 6 / 8 steps, mixed 57.1 / 54.8 / 53.9 / 52.5 ms,
+// binary64 49.3 / 48.9 / 48.9 / 49.2 ms (the runs below).
+constexpr int kSteps = 4, kStepsMixed = 8;
 
 // Measured: 16,384 photons, 6,000 steps each at most, z = 1700: 111 -> 49 ms
 // (111 -> 61 ms from spreading the warps over all SMs and 18 waiting lanes).
@@ -560,8 +562,8 @@ __global__ void __launch_bounds__(ST) k_scatter(McArgs A) {
 // cached in registers until the photon changes cell.  Statistically equivalent
 // to the binary64 form; not operation-for-operation equal to it.
 // Bound by instruction issue in divergent warps: 65,536 photons, 30,000 steps
-// each at most, z = 1700: 79.5 -> 54.8 ms, mostly from drawing the random words
-// with whole warps (McWords) and from four steps between votes.
+// each at most, z = 1700: 79.5 -> 52.5 ms, mostly from drawing the random words
+// with whole warps (McWords) and from eight steps between votes.
 __device__ __forceinline__ void df_add(float& hi, float& lo, float b) {
   const float s = hi + b;
   const float bb = s - hi;
@@ -828,9 +830,9 @@ __global__ void __launch_bounds__(ST) k_scatter_mixed(McArgs A) {
     if (__ballot_sync(kFull, active) == 0) break;
 
     // a few steps between votes
-    if (active && !pend) rng.ensure(kSteps);
+    if (active && !pend) rng.ensure(kStepsMixed);
 #pragma unroll 1
-    for (int it = 0; it < kSteps; ++it) {
+    for (int it = 0; it < kStepsMixed; ++it) {
       if (!active || pend) break;
       const float y = (xh - up) + xl;
       if (y < -A.x_lostf) {

@@ -1020,17 +1020,13 @@ __global__ void __launch_bounds__(kTmaThreads, kTmaCtasPerSm) k_substep_tma(Pass
 // side h in m); k_local then updates every cell on its own (no global lambda).
 template <bool MIXED>
 __global__ void __launch_bounds__(NT) k_divergence(const void* vel4, int n, double fac, void* div) {
-  const int64_t n3 = (int64_t)n * n * n;
-  const int64_t stride = (int64_t)gridDim.x * NT;
-  for (int64_t c = (int64_t)blockIdx.x * NT + threadIdx.x; c < n3; c += stride) {
-    const int ix = (int)(c % n), iy = (int)((c / n) % n), iz = (int)(c / ((int64_t)n * n));
-    const int xp = ix + 1 == n ? 0 : ix + 1, xm = ix == 0 ? n - 1 : ix - 1;
-    const int yp = iy + 1 == n ? 0 : iy + 1, ym = iy == 0 ? n - 1 : iy - 1;
-    const int zp = iz + 1 == n ? 0 : iz + 1, zm = iz == 0 ? n - 1 : iz - 1;
-    const int64_t nn = (int64_t)n * n, row = (int64_t)iz * nn + (int64_t)iy * n;
-    const int64_t cxp = row + xp, cxm = row + xm;
-    const int64_t cyp = (int64_t)iz * nn + (int64_t)yp * n + ix, cym = (int64_t)iz * nn + (int64_t)ym * n + ix;
-    const int64_t czp = (int64_t)zp * nn + (int64_t)iy * n + ix, czm = (int64_t)zm * nn + (int64_t)iy * n + ix;
+  // 32-bit cell indices (n <= 1024): 64-bit remainders cost more than the stencil's loads
+  const uint32_t n1 = (uint32_t)n, nn = n1 * n1, n3 = nn * n1;
+  for (uint32_t c = blockIdx.x * NT + threadIdx.x; c < n3; c += gridDim.x * NT) {
+    const uint32_t iz = c / nn, in = c - iz * nn, iy = in / n1, ix = in - iy * n1;
+    const uint32_t cxp = ix + 1 == n1 ? c - ix : c + 1, cxm = ix == 0 ? c + n1 - 1 : c - 1;
+    const uint32_t cyp = iy + 1 == n1 ? c - iy * n1 : c + n1, cym = iy == 0 ? c + nn - n1 : c - n1;
+    const uint32_t czp = iz + 1 == n1 ? in : c + nn, czm = iz == 0 ? c + n3 - nn : c - nn;
     if (MIXED) {
       const float4* U = (const float4*)vel4;
       const float d = (U[cxp].x - U[cxm].x) + (U[cyp].y - U[cym].y) + (U[czp].z - U[czm].z);
