@@ -21,7 +21,7 @@
 // Every pass but the last is bound by the binary64 pipe (two operations per
 // cycle and SM), so coefficients are computed once and read back (40 bytes per
 // cell), quotients by a common divisor share its reciprocal, and quotients by sums
-// are taken of the sums.  256^3: 50.2 -> 17.7 ms per reversed step.
+// are taken of the sums.  256^3: 50.2 -> 14.5 ms per reversed step.
 
 #include <cmath>
 
@@ -73,12 +73,12 @@ __device__ __forceinline__ Fwd forward_cell(const AdjArgs& a, int64_t i, double 
     f.al = q.x; f.w = q.y; f.Tn = q.z; f.tpd = q.w;
   } else {
     const double T = a.T[i];
-    const double opx = 1.0 + k.fHe + x, g = k.kc * x / opx, hh = k.hq / (d * opx);
-    f.Tn = (T + k.dt * (g * k.Tg + hh)) / (1.0 + k.dt * (2.0 * k.H + g));
+    const double opx = 1.0 + k.fHe + x, kx = k.kc * x;
+    f.Tn = (T * opx + k.dt * (kx * k.Tg + k.hq / d)) / (opx * (1.0 + 2.0 * k.H * k.dt) + k.dt * kx);
     const double lt = log(f.Tn * 1.0e-4);
     f.tpd = exp(k.pd * lt);
     f.al = k.fa * exp(k.pb * lt) / (1.0 + k.pc * f.tpd);
-    f.w = f.wt ? ((double)(a.tally ? a.tally[i] : 0u) / tot) * S1s / n1s_rel : 1.0;
+    f.w = f.wt ? (double)(a.tally ? a.tally[i] : 0u) * (S1s / tot) / n1s_rel : 1.0;
   }
   f.n = k.nH * d;
   f.A = k.dt * f.al * f.n;

@@ -1304,8 +1304,9 @@ __global__ void __launch_bounds__(TT, emit_occupancy<R>()) k_emit(TransportArgs<
 // ones take new packets, so that both run with many lanes at once.
 // Cells a lane walks per round, with their words in flight together (256^3 mixed: 3 / 4 /
 // 5 / 6 cells 4.07 / 3.57 / 3.60 / 3.43 ms, 8 cells 3.69 at three blocks per SM; FP64: 4 / 6
-// cells 7.97 / 8.28 ms).
-template <class R> struct MarchAhead { static constexpr int value = sizeof(R) == 4 ? 6 : 4; };
+// cells 7.97 / 8.28 ms; region sweeps of 512^3, 1e9 packets: 6 / 8 / 10 cells 76.3 / 72.0 /
+// 70.5 ms, 12 spill).
+template <class R, bool RS> struct MarchAhead { static constexpr int value = sizeof(R) == 4 ? (RS ? 10 : 6) : 4; };
 
 // Resident blocks per SM of the march (register budget per thread; a batch
 // keeps the box of each lane's packet in registers).
@@ -1457,7 +1458,7 @@ __global__ void __launch_bounds__(TT, (march_occupancy<R, MB, RS>())) k_march(Tr
   static_assert(!RS || (P2 && !MB), "region sweeps: single box of power-of-two side");
   static_assert(!MB || !P2, "a batch mixes sides");
   using V = typename Vec4<R>::T;
-  constexpr int kA = MarchAhead<R>::value;
+  constexpr int kA = MarchAhead<R, RS>::value;
   const int lane = threadIdx.x & 31;
   const uint32_t n = (uint32_t)a.n;
   // region sweeps: bucket of the open chunk (its super-tile); path length at
