@@ -77,7 +77,8 @@ int early_nodes(const rec_params& p) {
   const bool mixed = p.precision == REC_PREC_MIXED;
   auto q = [&](int i) { return mixed ? (double)(float)p.emission_quantiles[i] : p.emission_quantiles[i]; };
   int k = 0;
-  while (k + 1 < p.n_quantiles && (q(k + 1) == 0.0 || q(k + 1) <= -0x1p-20 * std::fabs(q(k)))) ++k;
+  // (a table value beyond the binary32 range becomes infinite there, and interpolation from it is no number)
+  while (k + 1 < p.n_quantiles && is_finite(q(k)) && (q(k + 1) == 0.0 || q(k + 1) <= -0x1p-20 * std::fabs(q(k)))) ++k;
   return k;
 }
 
