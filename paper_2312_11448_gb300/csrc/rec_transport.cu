@@ -10,18 +10,22 @@
 // resonance.
 //
 // Kernels (one lya_transport call):
-//   k_alloc_max     r_max over the emission weights (and a validity check)
-//   k_alloc_sum     Q_i = floor(2^31 r_i / r_max); block sums; last block scans
-//                   them and draws the systematic-sampling offset u
+//   k_alloc_max     r_max over the emission weights (and a validity check), largest
+//                   speeds
+//   k_alloc_sum     Q_i = floor(2^31 r_i / r_max); compact velocity copy; block
+//                   sums; last block scans them and draws the systematic-sampling
+//                   offset u
 //   k_alloc_prefix  packet prefix P_i = floor((N prefixQ_i + u) / sum Q), exact
 //                   integer arithmetic; cell of every 32nd packet; packets per
-//                   32^3 super-tile
-//   k_emit          one packet per thread: warp-cooperative cell lookup in P,
-//                   Philox draws, emission, resonance test in the home cell
-//                   (warp-aggregated tally); the others step once and are queued
-//                   in their home super-tile's bucket
+//                   super-tile; last block: bucket offsets
+//   k_emit          64 packets per warp and iteration: cell lookup in P, Philox
+//                   draws; packets that are home by their quantile word are tallied,
+//                   the others finished 32 at a time (resonance test in the home
+//                   cell, warp-aggregated tally) or queued in their home
+//                   super-tile's bucket; last block: chunks of the buckets
 //   k_march         persistent warps march the queued packets (Amanatides-Woo),
-//                   refilling idle lanes from the queue; tally atomics
+//                   refilling idle lanes from the queue; tally atomics; last block
+//                   closes the call
 // The march is written operation by operation with round-to-nearest
 // intrinsics (never contracted into FMA), in binary32 for the mixed form and
 // binary64 for the FP64 form, so its integer results are reproducible.
@@ -1263,6 +1267,10 @@ __device__ __forceinline__ void emit_window64(const TransportArgs<R>& a, const E
   while (count >= 32u) emit_finish32<R, P2>(a, e, st, head, count, my_abs, my_cross);
 }
 
+// What bounds the emission: the half-rate integer pipe (wide multiplies of Philox) and
+// issue in binary32, 1.65 -> 1.59 ms at 256^3 with 1e8 packets when the packets
+// settled by their quantile word skip the table; the binary64 pipe in the FP64
+// form, 15.1 -> 8.8 ms with those packets, the ring and quotients saved.
 // Resident blocks per SM of the emission (registers and the shared-memory ring:
 // with the ring a sixth block measured slower, 1.83 against 1.74 ms at 256^3).
 template <class R> constexpr int emit_occupancy() { return sizeof(R) == 4 ? 5 : 4; }
@@ -1302,10 +1310,14 @@ __global__ void __launch_bounds__(TT, emit_occupancy<R>()) k_emit(TransportArgs<
 // parked ones read the exact velocity of their candidate and take the exact
 // resonance test (tally and done, or on to the rest of the round), and the idle
 // ones take new packets, so that both run with many lanes at once.
+// What bounds it: requests from L1 to L2 (72 % busy), instruction issue (68 %) and the
+// integer pipe (66 %) together.  With the velocity vector read in every cell it was
+// the requests alone (87 %): 256^3, 1e8 packets 5.34 -> 3.38 ms, FP64 47.4 -> 8.0 ms;
+// 512^3, 1e9 packets with sweeps 111 -> 65.3 ms.
 // Cells a lane walks per round, with their words in flight together (256^3 mixed: 3 / 4 /
 // 5 / 6 cells 4.07 / 3.57 / 3.60 / 3.43 ms, 8 cells 3.69 at three blocks per SM; FP64: 4 / 6
-// cells 7.97 / 8.28 ms; region sweeps of 512^3, 1e9 packets: 6 / 8 / 10 cells 76.3 / 72.0 /
-// 70.5 ms, 12 spill).
+// cells 7.97 / 8.28 ms; region sweeps of 512^3, 1e9 packets, leaving packets queued after every
+// round: 6 / 8 / 10 cells 76.3 / 72.0 / 70.5 ms, 12 spill).
 template <class R, bool RS> struct MarchAhead { static constexpr int value = sizeof(R) == 4 ? (RS ? 10 : 6) : 4; };
 
 // Resident blocks per SM of the march (register budget per thread; a batch
@@ -1465,6 +1477,7 @@ __global__ void __launch_bounds__(TT, (march_occupancy<R, MB, RS>())) k_march(Tr
   // which the lane's packet leaves the region around it (+inf: no limit)
   uint32_t cbk = 0;
   float leave = 0.0f;
+  bool gone = false;  // it has left, and waits to be queued again
   __shared__ BoxCounters cnt;
   if (MB) box_counters_clear(cnt, B);
   // box of the lane's packet and of the open chunk
@@ -1493,10 +1506,9 @@ __global__ void __launch_bounds__(TT, (march_occupancy<R, MB, RS>())) k_march(Tr
   uint32_t my_abs = 0, my_cap = 0, my_cross = 0;
   for (;;) {
     const unsigned stop = __ballot_sync(0xffffffffu, !active || parked);
-    bool fresh = false;  // region sweeps: a round was completed, check the region
     if (__popc(stop) >= a.refill || stop == 0xffffffffu) {
       // exact test of the parked lanes' first candidate cell
-      if (parked) {
+      if (parked && !(RS && gone)) {
         uint32_t cand = 0;
 #pragma unroll
         for (int k = 0; k < kA; ++k) {
@@ -1506,7 +1518,6 @@ __global__ void __launch_bounds__(TT, (march_occupancy<R, MB, RS>())) k_march(Tr
         cand &= 0xffffffffu << kfrom;
         if (cand == 0) {
           parked = false;
-          fresh = true;
         } else {
           const uint32_t k = (uint32_t)__ffs((int)cand) - 1u;
           uint32_t c = cl[0];
@@ -1537,8 +1548,45 @@ __global__ void __launch_bounds__(TT, (march_occupancy<R, MB, RS>())) k_march(Tr
           } else {
             kfrom = k + 1u;
             parked = (cand >> kfrom) != 0u;
-            fresh = !parked;
           }
+        }
+        if (RS) gone = active && !parked && bound_exit(se[kA - 1]) >= leave;
+      }
+      if (RS) {
+        // packets that left their region: appended to the second queue as full
+        // states (the current cell is the next to test), counted in the bucket
+        // of the super-tile they have reached
+        const unsigned rm = __ballot_sync(0xffffffffu, gone);
+        if (rm) {
+          uint32_t ix, iy, iz;
+          velq_coords(X | Y | Z, bx, &ix, &iy, &iz);
+          const uint32_t cell = (((iz << a.tl.lg) | iy) << a.tl.lg) | ix;
+          // the warp's part of the second queue
+          const uint32_t part = (blockIdx.x * (TT / 32) + (threadIdx.x >> 5)) & (uint32_t)(kRqParts - 1);
+          unsigned long long qb = 0;
+          const int leader = __ffs(rm) - 1;
+          if (lane == leader) qb = atomicAdd(&a.rqn[part], (unsigned long long)__popc(rm));
+          qb = __shfl_sync(0xffffffffu, qb, leader);
+          const uint64_t k = qb + __popc(rm & ((1u << lane) - 1u));
+          const bool stored = gone && k < a.rq_part;
+          if (stored) {
+            const uint64_t slot = (uint64_t)part * a.rq_part + k;
+            V q0v, q1v, q2v;
+            q0v.x = bits_to<R>(cell); q0v.y = tMx; q0v.z = tMy; q0v.w = tMz;
+            q1v.x = copysign(tDx, knx); q1v.y = copysign(tDy, kny); q1v.z = copysign(tDz, knz); q1v.w = u0;
+            q2v.x = knx; q2v.y = kny; q2v.z = knz; q2v.w = bits_to<R>(kc);
+            a.rq[3 * slot] = q0v;
+            a.rq[3 * slot + 1] = q1v;
+            a.rq[3 * slot + 2] = q2v;
+            active = false;
+          }
+          const unsigned sm = __ballot_sync(0xffffffffu, stored);
+          const uint32_t bk = stored ? a.tl.template at<true>(cell) : 0xffffffffu;
+          const unsigned gm = __match_any_sync(0xffffffffu, bk) & sm;
+          if (stored && lane == __ffs(gm) - 1) atomicAdd(&a.rcount[bk], (unsigned long long)__popc(gm));
+          if (gone && !stored) leave = __int_as_float(0x7f800000);  // the second queue is full: march on without a limit
+          if (__any_sync(0xffffffffu, gone && !stored) && lane == 0) atomicOr(&a.sc->flags, 16);
+          if (gone) gone = parked = false;
         }
       }
       // refill idle lanes in lane order from the warp's chunks
@@ -1658,7 +1706,7 @@ __global__ void __launch_bounds__(TT, (march_occupancy<R, MB, RS>())) k_march(Tr
       }
     }
     if (!__any_sync(0xffffffffu, active)) break;  // no packet left in the warp
-    if (active && !parked && !(RS && fresh)) {
+    if (active && !parked) {
       // one round: walk kA cells, loading the words that matter, then ask the bound
 #pragma unroll
       for (int k = 0; k < kA; ++k) {
@@ -1676,48 +1724,10 @@ __global__ void __launch_bounds__(TT, (march_occupancy<R, MB, RS>())) k_march(Tr
 #pragma unroll
       for (int k = 0; k < kA; ++k)
         parked |= velq_dot(qw[k], vp.m, kVelqBiasBits) >= __float_as_int(fmaf(-bound_exit(se[k]), vp.c1, vp.c2));
-      fresh = !parked;
-    }
-    if (RS) {
-      bool rqp = false;  // the lane's packet left its region: queue it again
-      uint32_t cell = 0;
-      if (fresh && bound_exit(se[kA - 1]) >= leave) {
-        rqp = true;
-        uint32_t ix, iy, iz;
-        velq_coords(X | Y | Z, bx, &ix, &iy, &iz);
-        cell = (((iz << a.tl.lg) | iy) << a.tl.lg) | ix;
-      }
-      // packets that left their region: appended to the second queue as full
-      // states (the current cell is the next to test), counted in the bucket
-      // of the super-tile they have reached
-      const unsigned rm = __ballot_sync(0xffffffffu, rqp);
-      if (rm) {
-        // the warp's part of the second queue
-        const uint32_t part = (blockIdx.x * (TT / 32) + (threadIdx.x >> 5)) & (uint32_t)(kRqParts - 1);
-        unsigned long long qb = 0;
-        const int leader = __ffs(rm) - 1;
-        if (lane == leader) qb = atomicAdd(&a.rqn[part], (unsigned long long)__popc(rm));
-        qb = __shfl_sync(0xffffffffu, qb, leader);
-        const uint64_t k = qb + __popc(rm & ((1u << lane) - 1u));
-        const bool stored = rqp && k < a.rq_part;
-        const uint64_t slot = (uint64_t)part * a.rq_part + k;
-        if (stored) {
-          V q0v, q1v, q2v;
-          q0v.x = bits_to<R>(cell); q0v.y = tMx; q0v.z = tMy; q0v.w = tMz;
-          q1v.x = copysign(tDx, knx); q1v.y = copysign(tDy, kny); q1v.z = copysign(tDz, knz); q1v.w = u0;
-          q2v.x = knx; q2v.y = kny; q2v.z = knz; q2v.w = bits_to<R>(kc);
-          a.rq[3 * slot] = q0v;
-          a.rq[3 * slot + 1] = q1v;
-          a.rq[3 * slot + 2] = q2v;
-          active = false;
-        }
-        const unsigned sm = __ballot_sync(0xffffffffu, stored);
-        const uint32_t bk = stored ? a.tl.template at<true>(cell) : 0xffffffffu;
-        const unsigned gm = __match_any_sync(0xffffffffu, bk) & sm;
-        if (stored && lane == __ffs(gm) - 1) atomicAdd(&a.rcount[bk], (unsigned long long)__popc(gm));
-        if (rqp && !stored) leave = __int_as_float(0x7f800000);  // the second queue is full: march on without a limit
-        if (__any_sync(0xffffffffu, rqp && !stored) && lane == 0) atomicOr(&a.sc->flags, 16);
-      }
+      // a packet that left its region waits for the warp's next stop, so that the
+      // append runs with many lanes: with one or two lanes after each round
+      // the sweeps of 512^3, 1e9 packets took 70.9 ms, with this 65.3
+      if (RS && !parked && bound_exit(se[kA - 1]) >= leave) gone = parked = true;
     }
   }
   if (MB) {
