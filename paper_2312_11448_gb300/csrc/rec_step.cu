@@ -18,7 +18,8 @@
 // converged; then the final pass: x, T, U, emission weights, tallies zeroed and the sums
 // of the new state.  (One launch per evaluation, ten of them with those after
 // convergence returning at once, was 40 us per substep slower: 256^3 mixed substep
-// 379 -> 339 us, two partial-mixing substeps of 128^3 443 -> 289 us.)
+// 379 -> 339 us, two partial-mixing substeps of 128^3 443 -> 289 us, 234 with block sums that
+// add two values per step of the tree and a divergence with 32-bit indices.)
 // Two forms: FP64 (all binary64) and MIXED (binary32 per-cell coefficients and
 // root, binary64 state x, net-rate residual correction and volume sums).
 
