@@ -528,20 +528,20 @@ def time_batched(W, K, prep=60, n_boxes=64):
 # Roofline of the Monte-Carlo kernels (profiles/k_scatter_mc_z1700.md): ncu
 # counts on one launch of the bench workload (8192 photons capped at 2e4 steps,
 # 1.57e8 photon steps, one scattering per 10.5 steps), amortised per photon
-# step.  The binary64 kernel is bound by its binary64 pipe (127.8 SM-cycles of
+# step.  The binary64 kernel is bound by its binary64 pipe (94.2 SM-cycles of
 # that pipe per step: sm__pipe_fp64_cycles_active x sm__cycles_active / steps);
-# the mixed kernel by instruction issue (24.7 warp instructions per step:
+# the mixed kernel by instruction issue (17.6 warp instructions per step:
 # smsp__inst_executed / steps).  Peaks: every SM's binary64 pipe busy every
 # cycle, and one warp instruction per cycle per SM sub-partition, at the
 # 2070 MHz maximum SM clock of the 152 SMs.
 _SM_CYCLES_PER_S = 152 * 2.070e9
 MC_PROFILE = {
-    "fp64": {"bound": "fp64-pipe", "kernel": "k_scatter (binary64)", "per_step": 127.8, "per_scatter": 0.0,
+    "fp64": {"bound": "fp64-pipe", "kernel": "k_scatter (binary64)", "per_step": 94.2, "per_scatter": 0.0,
              "peak": _SM_CYCLES_PER_S, "unit": "G SM-cycles/s of the binary64 pipe",
-             "note": "127.8 binary64-pipe SM-cycles per photon step (ncu), peak = every SM's pipe every cycle"},
-    "mixed": {"bound": "issue", "kernel": "k_scatter_mixed (binary32 + double-float)", "per_step": 24.7,
+             "note": "94.2 binary64-pipe SM-cycles per photon step (ncu), peak = every SM's pipe every cycle"},
+    "mixed": {"bound": "issue", "kernel": "k_scatter_mixed (binary32 + double-float)", "per_step": 17.6,
               "per_scatter": 0.0, "peak": 4 * _SM_CYCLES_PER_S, "unit": "G warp instructions/s",
-              "note": "24.7 warp instructions per photon step (ncu), peak = one per cycle per SM sub-partition"},
+              "note": "17.6 warp instructions per photon step (ncu), peak = one per cycle per SM sub-partition"},
 }
 
 

@@ -1310,9 +1310,10 @@ __global__ void __launch_bounds__(TT, emit_occupancy<R>()) k_emit(TransportArgs<
 // parked ones read the exact velocity of their candidate and take the exact
 // resonance test (tally and done, or on to the rest of the round), and the idle
 // ones take new packets, so that both run with many lanes at once.
-// What bounds it: requests from L1 to L2 (72 % busy), instruction issue (68 %) and the
-// integer pipe (66 %) together.  With the velocity vector read in every cell it was
-// the requests alone (87 %): 256^3, 1e8 packets 5.34 -> 3.38 ms, FP64 47.4 -> 8.0 ms;
+// What bounds it: with flows of 1 km/s, requests from L1 to L2 (72 % busy), instruction
+// issue (68 %) and the integer pipe (66 %) together; once Compton drag has slowed the
+// flow most cells need no load, and it is issue (74 %) and the integer pipe (73 %).  With
+// the velocity vector read in every cell it was the requests alone (87 %): 256^3, 1e8 packets 5.34 -> 3.38 ms, FP64 47.4 -> 8.0 ms;
 // 512^3, 1e9 packets with sweeps 111 -> 65.3 ms.
 // Cells a lane walks per round, with their words in flight together (256^3 mixed: 3 / 4 /
 // 5 / 6 cells 4.07 / 3.57 / 3.60 / 3.43 ms, 8 cells 3.69 at three blocks per SM; FP64: 4 / 6
