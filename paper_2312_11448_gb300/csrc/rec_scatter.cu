@@ -1126,9 +1126,13 @@ cudaError_t run_scatter_mc(rec_ctx* c, const McSetup& S, const lya_mc_params* mp
                                 : (fmix ? k_scatter<float> : k_scatter<double>);
   int per_sm = 0;
   const size_t ring = sizeof(uint32_t) * kRingWords * threads;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, ring);
+  // With ST threads the ring and the binary64 Voigt table are 52 KB, beyond the 48 KB
+  // that a kernel has unless it asks for more (the most, whatever this call takes:
+  // the setting is the kernel's, and other threads' calls rely on it).
+  e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(sizeof(uint32_t) * kRingWords * ST));
+  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, ring);
   if (e != cudaSuccess) return e;
-  if (per_sm < 1) per_sm = 1;
+  if (per_sm < 1) return cudaErrorLaunchOutOfResources;
   uint64_t blocks = (uint64_t)c->sm_count * per_sm;
   const uint64_t max_useful = (warps + (threads / 32) - 1) / (threads / 32);
   if (blocks > max_useful) blocks = max_useful;
