@@ -126,7 +126,7 @@ typedef struct {
   int32_t newton_passes; /* Newton evaluations of the last substep */
   int32_t flags;         /* bit 0: Newton did not converge; bit 1: packets hit the crossing cap;
                             bit 2: non-finite or negative emission weight; bit 3: a bounded
-                            device-side wait expired (copy pipeline of a Newton pass); bit 4:
+                            device-side wait expired (copy pipeline or grid barrier); bit 4:
                             region sweeps found their second queue full (the packets concerned
                             marched on without a region limit: results unchanged, speed only) */
   uint64_t requeued;     /* region sweeps (rec_tuning.march_halo > 0): packets queued again for a
@@ -313,10 +313,11 @@ rec_status rec_volume_stats(rec_ctx* ctx, rec_stats* dev_stats);
  * 2^22, about a second); past that the block records the expiry (rec_stats
  * flags bit 3) and returns without finishing its share of the pass.  The wait
  * for its copies still in flight before such a return keeps the default bound.
- * The grid barriers between the phases of the persistent batched launches
- * (see rec_init) poll at most `polls` times as well.  0 makes every such wait
- * give up at once, which is how the error path is tested.  Host-side only: takes effect from the next call
- * enqueued.  Errors: REC_EINVAL (NULL context). */
+ * The grid barriers between the phases of the persistent launches (a substep of
+ * rec_step, the evaluations of rec_step_adjoint, the allocation and emission of a
+ * batch) poll at most `polls` times as well.  0 makes every such wait give up at
+ * once, which is how the error path is tested.  Host-side only: takes effect from
+ * the next call enqueued.  Errors: REC_EINVAL (NULL context). */
 rec_status rec_set_wait_limit(rec_ctx* ctx, uint32_t polls);
 
 /* Waits for the context stream and reports the device-side failures of the
@@ -325,7 +326,8 @@ rec_status rec_set_wait_limit(rec_ctx* ctx, uint32_t polls);
  * incomplete: re-initialise it (zero the tallies; rec_state_init, or write x_e
  * and T and call rec_refresh) before stepping again; rec_sync clears the expiry and the
  * device counters a pass that gave up may have left part-way, so the context
- * stays usable.  Errors: REC_ETIMEOUT, REC_ECUDA. */
+ * stays usable.  A single box that is re-initialised before this call steps on
+ * from there, and the expiry is still reported here.  Errors: REC_ETIMEOUT, REC_ECUDA. */
 rec_status rec_sync(rec_ctx* ctx);
 
 /* Objective on an X_e history over node redshifts zs[0..n_nodes-1] (decreasing),

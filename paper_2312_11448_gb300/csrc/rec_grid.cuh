@@ -1,8 +1,8 @@
 // Grid-wide barrier of a persistent cooperative launch, with a bounded wait.
 //
-// The batched step runs its phases (allocation, emission; the Newton passes
-// and the final pass) as phases of one persistent launch each.  Between two
-// phases every block arrives at this barrier: thread 0 of a block adds itself
+// A substep (the evaluations of lambda and the final pass, of one box or of a batch)
+// and the allocation and emission of a batch run as phases of one persistent launch
+// each.  Between two phases every block arrives at this barrier: thread 0 of a block adds itself
 // to the arrival count; the last block to arrive resets the count and opens the
 // barrier by advancing its generation; the others poll the generation, each
 // poll bounded (at most `limit` polls, about a second at the default), and

@@ -62,6 +62,7 @@ struct DevScalars {
   unsigned long long requeued;     // region sweeps: packets queued again in this transport call
   uint32_t alloc_counter;
   int32_t emis_valid;
+  int32_t expired;  // a wait expired (flags bit 3) in a state that a refresh has since replaced; until rec_sync reports it
   GridBarrier bar;  // grid barrier of the persistent launches (of a batch: in the batch-wide record)
   // binary32 copies of the current iterate for the mixed form's passes (set
   // with lam, so that no pass converts binary64 scalars per thread)

@@ -1200,6 +1200,7 @@ __global__ void __launch_bounds__(NT) k_refresh(PassArgs a, const BoxDev* bxs, i
     sc->lam_state = S[4] > 0.0 ? S[3] / S[4] : 0.0;
     sc->lam_prev = -1.0;
     sc->tally_total = (unsigned long long)(S[5] + 0.5);
+    if (sc->flags & 8) sc->expired = 1;  // the new state steps on, the report stays due
     sc->flags = 0;
     sc->bar.arrived = 0;  // a substep that gave up may have left arrivals
     sc->emis_valid = 1;
@@ -1278,10 +1279,17 @@ cudaError_t enqueue_newton_passes(rec_ctx* c, DevScalars* sc, const StepCoef& k,
               : launch_substep<false, false, false, false>(c, a, nullptr);
 }
 
+// The boxes' block counters, which a final pass that gave up may have left part-way.
+static cudaError_t clear_counters(rec_ctx* c) {
+  return cudaMemset2DAsync(&c->sc->counter, sizeof(DevScalars), 0, sizeof(c->sc->counter), c->n_boxes, c->stream);
+}
+
 cudaError_t launch_refresh(rec_ctx* c, double z) {
   StepCoef k = step_coef(c->cosmo, c->params, z + 1e-6 * (1.0 + z), z, 0);
   PassArgs a = pass_args(c, k);
   GroupTimer t(c, kTOther, 1);
+  cudaError_t e = clear_counters(c);
+  if (e != cudaSuccess) return e;
   if (c->params.precision == REC_PREC_MIXED) k_refresh<true, false><<<c->grid, NT, 0, c->stream>>>(a, nullptr, 1);
   else k_refresh<false, false><<<c->grid, NT, 0, c->stream>>>(a, nullptr, 1);
   return cudaGetLastError();
@@ -1392,8 +1400,8 @@ cudaError_t launch_volume_stats(rec_ctx* c, rec_stats* st) {
   return cudaGetLastError();
 }
 
-// Expired bounded waits (flags bit 3) of every box: reported in *out and
-// cleared, with the counters a pass that gave up may have left part-way.
+// Expired bounded waits (flags bit 3, or an expiry before the last refresh) of every
+// box: reported in *out and cleared, with the counters a pass that gave up may have left part-way.
 __global__ void k_check_waits(DevScalars* sc, const BoxDev* bxs, int B, DevScalars* gsc, DevScalars* adj, int* out) {
   if (threadIdx.x != 0) return;
   // a batch-wide expiry (a grid barrier gave up) may have left any box part-way
@@ -1401,9 +1409,10 @@ __global__ void k_check_waits(DevScalars* sc, const BoxDev* bxs, int B, DevScala
   int any = all ? 1 : 0;
   for (int b = -1; b < B; ++b) {
     DevScalars* s = b < 0 ? adj : (bxs ? bxs[b].sc : sc);
-    if ((all && b >= 0) || (s->flags & 8)) {
+    if ((all && b >= 0) || (s->flags & 8) || s->expired) {
       any = 1;
       s->flags &= ~8;
+      s->expired = 0;
       s->counter = 0;
       s->alloc_counter = 0;
       s->bar.arrived = 0;
@@ -1433,6 +1442,8 @@ cudaError_t launch_refresh_batch(rec_ctx* c, double z) {
   StepCoef k = step_coef(c->cosmo, c->params, z + 1e-6 * (1.0 + z), z, 0);
   PassArgs a = batch_args(c, k);
   GroupTimer t(c, kTOther, 1);
+  cudaError_t e = clear_counters(c);
+  if (e != cudaSuccess) return e;
   if (c->params.precision == REC_PREC_MIXED) k_refresh<true, true><<<c->tot_pblk, NT, 0, c->stream>>>(a, c->bx, c->n_boxes);
   else k_refresh<false, true><<<c->tot_pblk, NT, 0, c->stream>>>(a, c->bx, c->n_boxes);
   return cudaGetLastError();
