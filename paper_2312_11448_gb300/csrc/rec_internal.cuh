@@ -174,8 +174,8 @@ struct rec_ctx {
   int grid;                  // blocks of the streaming passes
   int alloc_blocks;
   int newton_tma = 0;        // TMA-staged substep usable (0: not yet queried, 1 / -1)
-  int substep_resident[16] = {};  // resident blocks per SM of the persistent substeps (0: not queried), and of
-  int tma_resident = 0;           // the TMA-staged one
+  int substep_resident[16] = {};  // resident blocks per SM of the persistent substeps (0: not queried, -1: none),
+  int tma_resident = 0;           // and of the TMA-staged one
   int batch_step_grid = 0;   // resident blocks of the persistent batched substep (0: not queried, -1: none)
   int batch_front_grid = 0;  // resident blocks of the persistent batched transport front (same)
   void* queue;               // queued packets of the march (2 x 16 B binary32, 3 x 32 B binary64) [n_packets]
@@ -276,9 +276,10 @@ cudaError_t launch_check_waits(rec_ctx* c, int* timed_out);
 // Context-free FP64 step on static device scratch; no device allocation.
 rec_status launch_rec_step_noalloc(const rec_params& p, const rec_box& b, double z_from, double z_to,
                                    cudaStream_t stream, rec_stats* st, std::string* why);
-// Newton passes for lambda of a substep on an arbitrary FP64 state (used by the adjoint).
+// Newton passes for lambda of a substep on an arbitrary FP64 state (used by the adjoint); the cells'
+// coefficients are left in the context's cellcache where it has one.
 cudaError_t enqueue_newton_passes(rec_ctx* c, DevScalars* sc, const StepCoef& k, const double* x, const double* T,
-                           const uint32_t* tally);
+                                  const uint32_t* tally);
 
 // rec_transport.cu
 cudaError_t launch_transport(rec_ctx* c, int step, double z, rec_stats* st);

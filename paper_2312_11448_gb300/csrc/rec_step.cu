@@ -606,7 +606,7 @@ __device__ __forceinline__ void pass_view(PassArgs& a, const BoxDev* bxs, int B,
   *box = lo;
 }
 
-template <bool MIXED, bool MB>
+template <bool MIXED, bool MB, bool PART = false, int CACHE = kNoCache>
 __global__ void __launch_bounds__(NT) k_newton(PassArgs a, const BoxDev* bxs, int B) {
   int blk = blockIdx.x, nblk = gridDim.x, box = 0;
   if (MB) pass_view(a, bxs, B, &blk, &nblk, &box, blockIdx.x);
@@ -615,9 +615,9 @@ __global__ void __launch_bounds__(NT) k_newton(PassArgs a, const BoxDev* bxs, in
   const double lam = sc->lam;
   constexpr int K = NSums<MIXED>::value;
   double v[5];
-  newton_block_sums<MIXED>(a, lam, sc->omC * lam + sc->G0,
-                           MIXED ? 0.0 : weight_factor((double)sc->tally_total, sc->S1s), mixed_scal(sc, false), blk,
-                           nblk, v);
+  newton_block_sums<MIXED, PART, CACHE>(a, lam, sc->omC * lam + sc->G0,
+                                        MIXED ? 0.0 : weight_factor((double)sc->tally_total, sc->S1s),
+                                        mixed_scal(sc, false), blk, nblk, v);
   if (threadIdx.x == 0) {
     double* p = a.part + (size_t)blk * kMaxSums;
     for (int j = 0; j < K; ++j) p[j] = v[j];
@@ -698,15 +698,15 @@ __device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t b
 
 // Final pass: new state at the converged lambda, emission weights, sums.
 // st: statistics record (one per box in a batch) or NULL.
-template <bool MIXED, bool MB>
+template <bool MIXED, bool MB, bool PART = false>
 __global__ void __launch_bounds__(NT) k_final(PassArgs a, rec_stats* st, const BoxDev* bxs, int B) {
   int blk = blockIdx.x, nblk = gridDim.x, box = 0;
   if (MB) pass_view(a, bxs, B, &blk, &nblk, &box, blockIdx.x);
   DevScalars* sc = a.sc;
   const double lam = sc->lam;
   double v[3];
-  final_block<MIXED>(a, sc->omC * lam + sc->G0, MIXED ? 0.0 : weight_factor((double)sc->tally_total, sc->S1s),
-                     mixed_scal(sc, false), blk, nblk, v);
+  final_block<MIXED, PART>(a, sc->omC * lam + sc->G0, MIXED ? 0.0 : weight_factor((double)sc->tally_total, sc->S1s),
+                           mixed_scal(sc, false), blk, nblk, v);
   if (threadIdx.x == 0) {
     double* p = a.part + (size_t)blk * kMaxSums;
     p[0] = v[0]; p[1] = v[1]; p[2] = v[2];
@@ -1243,33 +1243,55 @@ PassArgs pass_args(rec_ctx* c, const StepCoef& k) {
   return a;
 }
 
-// Launches one persistent substep kernel; resident: blocks per SM looked up once per context and kernel.
+// Resident blocks per SM of a persistent substep kernel, looked up once per context
+// and kernel; -1: it cannot run (no cooperative launch, or REC_NEWTON=passes).
 template <class F>
-cudaError_t launch_resident(rec_ctx* c, F kernel, int threads, size_t smem, int* resident, int blocks, void** args) {
+int substep_resident(rec_ctx* c, F kernel, int threads, size_t smem, int* resident) {
   if (*resident == 0) {
-    cudaError_t e = smem ? cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) : cudaSuccess;
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(resident, kernel, threads, smem);
-    if (e != cudaSuccess) { *resident = 0; return e; }
-    if (*resident < 1) return cudaErrorCooperativeLaunchTooLarge;
+    int per_sm = 0, coop = 0, dev = 0;
+    const char* sel = std::getenv("REC_NEWTON");
+    bool ok = !(sel && std::strcmp(sel, "passes") == 0) && cudaGetDevice(&dev) == cudaSuccess &&
+              cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) == cudaSuccess && coop != 0;
+    if (ok && smem)
+      ok = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) == cudaSuccess;
+    ok = ok && cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, smem) == cudaSuccess;
+    cudaGetLastError();
+    *resident = ok && per_sm > 0 ? per_sm : -1;
   }
-  const int grid = std::min(blocks, *resident * c->sm_count);
+  return *resident;
+}
+template <class F>
+cudaError_t launch_resident(rec_ctx* c, F kernel, int threads, size_t smem, int resident, int blocks, void** args) {
+  const int grid = std::min(blocks, resident * c->sm_count);
   return cudaLaunchCooperativeKernel((const void*)kernel, dim3(grid), dim3(threads), args, smem, c->stream);
 }
 
+// The substep as one persistent launch, or, where that cannot run, as a launch per
+// pass (ten evaluations; those after convergence return at once): the same sums in the
+// same order.
 template <bool MIXED, bool PART, bool CACHE, bool FINAL>
 cudaError_t launch_substep(rec_ctx* c, PassArgs a, rec_stats* st) {
-  int nvb = c->grid;
-  uint32_t limit = c->wait_limit;
-  void* args[] = {&a, &st, &nvb, &limit};
-  return launch_resident(c, k_substep<MIXED, PART, CACHE, FINAL>, NT, 0,
-                         &c->substep_resident[(MIXED ? 8 : 0) + (PART ? 4 : 0) + (CACHE ? 2 : 0) + (FINAL ? 1 : 0)], nvb,
-                         args);
+  int* slot = &c->substep_resident[(MIXED ? 8 : 0) + (PART ? 4 : 0) + (CACHE ? 2 : 0) + (FINAL ? 1 : 0)];
+  const int resident = substep_resident(c, k_substep<MIXED, PART, CACHE, FINAL>, NT, 0, slot);
+  if (resident > 0) {
+    int nvb = c->grid;
+    uint32_t limit = c->wait_limit;
+    void* args[] = {&a, &st, &nvb, &limit};
+    return launch_resident(c, k_substep<MIXED, PART, CACHE, FINAL>, NT, 0, resident, nvb, args);
+  }
+  k_substep_begin<<<1, 32, 0, c->stream>>>(a.sc, a.k, (double)c->n3);
+  constexpr int keep = CACHE && !FINAL ? kFillCache : kNoCache;  // the adjoint reads the coefficients back
+  for (int it = 0; it < kNewtonMaxPasses; ++it)
+    k_newton<MIXED, false, PART, keep><<<c->grid, NT, 0, c->stream>>>(a, nullptr, 1);
+  if (FINAL) k_final<MIXED, false, PART><<<c->grid, NT, 0, c->stream>>>(a, st, nullptr, 1);
+  c->launches[FINAL ? kTStep : kTAdj] += kNewtonMaxPasses + (FINAL ? 1 : 0);  // beyond the one the caller counts
+  return cudaGetLastError();
 }
 
 }  // namespace
 
 cudaError_t enqueue_newton_passes(rec_ctx* c, DevScalars* sc, const StepCoef& k, const double* x, const double* T,
-                           const uint32_t* tally) {
+                                  const uint32_t* tally) {
   PassArgs a = pass_args(c, k);
   a.sc = sc;
   a.x = const_cast<double*>(x);
@@ -1308,12 +1330,13 @@ cudaError_t launch_state_init(rec_ctx* c, double z) {
   return launch_refresh(c, z);
 }
 
-// The TMA-staged substep needs 16-byte aligned streams (bulk copies);
-// REC_NEWTON=plain selects the grid-stride one.
+// The TMA-staged substep needs 16-byte aligned streams (bulk copies) and a cooperative
+// launch; REC_NEWTON=plain selects the grid-stride one, REC_NEWTON=passes a launch per pass.
 bool newton_tma_ok(rec_ctx* c, const PassArgs& a) {
   if (c->newton_tma == 0) {
     const char* sel = std::getenv("REC_NEWTON");
     bool ok = !(sel && std::strcmp(sel, "plain") == 0);
+    ok = ok && substep_resident(c, k_substep_tma, kTmaThreads, kTmaSmem, &c->tma_resident) > 0;
     ok = ok && kTmaCtasPerSm * c->sm_count <= 2 * c->grid;  // its blocks fit the partials (2 x grid entries)
     c->newton_tma = ok ? 1 : -1;
   }
@@ -1359,7 +1382,7 @@ cudaError_t launch_rec_step(rec_ctx* c, double z_from, double z_to, rec_stats* s
     } else if (newton_tma_ok(c, a)) {
       uint32_t limit = c->wait_limit;
       void* args[] = {&a, &st, &limit};
-      e = launch_resident(c, k_substep_tma, kTmaThreads, kTmaSmem, &c->tma_resident, kTmaCtasPerSm * c->sm_count, args);
+      e = launch_resident(c, k_substep_tma, kTmaThreads, kTmaSmem, c->tma_resident, kTmaCtasPerSm * c->sm_count, args);
     } else {
       e = launch_substep<true, false, false, true>(c, a, st);
     }
