@@ -71,12 +71,16 @@ struct DevScalars {
   float Ghi, Glo;    // G as a double-float pair
   float wscale;      // S1s / tally_total (0 without tallies)
   // compact velocity copy of the march (rec_velq.cuh): the velocity that maps to
-  // 127, km/s (0: no usable copy), and the largest speed
+  // 127, km/s (0: no usable copy), the largest speed, whether cells are beyond the scale,
+  // and whether every velocity is finite and below 1e15 km/s
   float vq_u, vq_v;
+  int32_t vq_out, vel_plain;
   // running maxima of the allocation's first pass as ordered bits (weight, velocity
-  // component, squared speed) and what was invalid (bit 0 weight, bit 1 velocity); 0 between calls
+  // component, squared speed), the sum of |component| and what was invalid (bit 0 weight,
+  // bit 1 velocity); 0 between calls
   unsigned long long mx_w;
   unsigned int mx_u, mx_v2, mx_bad;
+  float mx_sum;
 };
 
 // Batched contexts (several boxes in one context, one launch per phase for

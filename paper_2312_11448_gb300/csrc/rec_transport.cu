@@ -216,15 +216,17 @@ __device__ __forceinline__ float velq_value(double v) {
 }
 __device__ __forceinline__ float velq_upper(double v) { return __uint_as_float(velq_abs_bits(v) + 1u); }
 
-// Largest |component| and squared speed of a velocity vector, running maxima;
-// anything not finite marks the box as unusable for the compact copy.
+// Largest |component| and squared speed of a velocity vector, running maxima, and the
+// sum of |component| over the cells that are finite.
 struct VelMax {
-  float u = 0.0f, v2 = 0.0f;
+  float u = 0.0f, v2 = 0.0f, sum = 0.0f;
   int bad = 0;
   template <class V>
   __device__ __forceinline__ void add(const V& U) {
     const float x = velq_upper(U.x), y = velq_upper(U.y), z = velq_upper(U.z);
-    bad |= !(x < 3e38f) || !(y < 3e38f) || !(z < 3e38f);
+    const bool fin = x < 3e38f && y < 3e38f && z < 3e38f;
+    bad |= !fin;
+    sum += fin ? x + y + z : 0.0f;
     u = fmaxf(u, fmaxf(x, fmaxf(y, z)));
     v2 = fmaxf(v2, x * x + y * y + z * z);
   }
@@ -244,6 +246,7 @@ __device__ __forceinline__ double from_order_bits(uint64_t b, double) { return _
 template <int NTH>
 __device__ __forceinline__ void block_maxima(DevScalars* sc, uint64_t w, const VelMax& vm, bool bad) {
   __shared__ uint32_t sm[NTH / 32][5];
+  __shared__ float part[NTH / 32];
   const unsigned full = 0xffffffffu;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   auto max64 = [&](uint32_t hi, uint32_t lo, uint32_t* h, uint32_t* l) {
@@ -255,8 +258,11 @@ __device__ __forceinline__ void block_maxima(DevScalars* sc, uint64_t w, const V
   const uint32_t u = __reduce_max_sync(full, __float_as_uint(vm.u));
   const uint32_t v2 = __reduce_max_sync(full, __float_as_uint(vm.v2));
   const uint32_t b = __reduce_or_sync(full, (bad ? 1u : 0u) | (vm.bad ? 2u : 0u));
+  float sum = vm.sum;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(full, sum, o);
   __syncthreads();  // sm may still be read by a previous call
-  if (lane == 0) { sm[warp][0] = h; sm[warp][1] = l; sm[warp][2] = u; sm[warp][3] = v2; sm[warp][4] = b; }
+  if (lane == 0) { sm[warp][0] = h; sm[warp][1] = l; sm[warp][2] = u; sm[warp][3] = v2; sm[warp][4] = b; part[warp] = sum; }
   __syncthreads();
   if (warp == 0) {
     const bool in = lane < NTH / 32;
@@ -265,6 +271,8 @@ __device__ __forceinline__ void block_maxima(DevScalars* sc, uint64_t w, const V
     const uint32_t bv = __reduce_max_sync(full, in ? sm[lane][3] : 0u);
     const uint32_t bb = __reduce_or_sync(full, in ? sm[lane][4] : 0u);
     if (lane == 0) {
+      for (int w = 1; w < NTH / 32; ++w) sum += part[w];
+      atomicAdd(&sc->mx_sum, sum);  // in any order: the scale of the copy changes no result
       atomicMax(&sc->mx_w, ((unsigned long long)h << 32) | l);
       atomicMax(&sc->mx_u, bu);
       atomicMax(&sc->mx_v2, bv);
@@ -274,13 +282,18 @@ __device__ __forceinline__ void block_maxima(DevScalars* sc, uint64_t w, const V
 }
 // The box's maxima once every block has added its own (one thread); ready for the next call.
 template <class R>
-__device__ __forceinline__ void take_maxima(DevScalars* sc, float kappa) {
+__device__ __forceinline__ void take_maxima(DevScalars* sc, int64_t n3, float kappa) {
   const uint32_t bad = __ldcg(&sc->mx_bad);
   sc->rmax = bad & 1u ? 0.0 : (double)from_order_bits(__ldcg(&sc->mx_w), (R)0);  // invalid weights: emit nothing
   sc->flags &= ~(2 | 4 | 16);                                                    // transport flags describe this call only
   if (bad & 1u) sc->flags |= 4;
-  sc->vq_u = velq_scale(__uint_as_float(__ldcg(&sc->mx_u)), (bad & 2u) != 0u, kappa);
-  sc->vq_v = sqrtf(__uint_as_float(__ldcg(&sc->mx_v2))) * 1.00001f;
+  const float umax = __uint_as_float(__ldcg(&sc->mx_u));
+  const float u = velq_scale(umax, __ldcg(&sc->mx_sum) / (3.0f * (float)n3), kappa);
+  sc->vq_u = u;
+  sc->vq_v = bad & 2u ? __int_as_float(0x7f800000) : sqrtf(__uint_as_float(__ldcg(&sc->mx_v2))) * 1.00001f;
+  sc->vq_out = (bad & 2u) || umax > u;
+  sc->vel_plain = !(bad & 2u) && umax < 1e15f;
+  sc->mx_sum = 0.0f;
   sc->mx_w = 0;
   sc->mx_u = sc->mx_v2 = sc->mx_bad = 0;
 }
@@ -305,7 +318,7 @@ __global__ void __launch_bounds__(kPassThreads) k_alloc_max(const R* emis, const
   block_maxima<kPassThreads>(sc, order_bits(m), vm, bad);
   if (!last_block_done(&sc->counter)) return;
   if (threadIdx.x == 0) {
-    take_maxima<R>(sc, kappa);
+    take_maxima<R>(sc, n3, kappa);
     sc->counter = 0;
   }
 }
@@ -458,8 +471,9 @@ __device__ __forceinline__ void velq_write(const V* vel, int64_t n3, int64_t c0,
     uint32_t ix, iy, iz;
     if (tl.lg) tl.template coords<true>((uint32_t)i, &ix, &iy, &iz);
     else tl.template coords<false>((uint32_t)i, &ix, &iy, &iz);
+    const bool in = velq_upper(U.x) <= u && velq_upper(U.y) <= u && velq_upper(U.z) <= u;
     velq[velq_x(ix) | velq_y(iy, bx) | velq_z(iz, bx)] =
-        velq_pack(velq_value(U.x), velq_value(U.y), velq_value(U.z), qs);
+        in ? velq_pack(velq_value(U.x), velq_value(U.y), velq_value(U.z), qs) : kVelqOut;
   }
 }
 
@@ -961,7 +975,7 @@ struct EmitBox {
   uint32_t box;  // fourth Philox counter word
   Tiles tl;
   uint32_t bk0;
-  uint32_t early;  // TransportArgs::early, or 0 where the box's velocities are not all finite
+  uint32_t early;  // TransportArgs::early, or 0 where not all velocities are plain (DevScalars::vel_plain)
 };
 
 // Emission of one packet, in three parts: the cell of each of a warp's 32
@@ -1163,9 +1177,15 @@ __device__ __forceinline__ void emit_rest(const TransportArgs<R>& a, const EmitB
 // - xi: the packet's quantile deviate u lies below a bound known to the host
 //   (early_word), so the word that leads u's bits decides, without the table.
 // - v_t = sqrt(T cth): T in [0, 1e15] by its bits, with cth <= 1e15 (early_word is 0 otherwise).
-// - d: the box's velocities are finite (EmitBox::early is 0 otherwise).
+// - d: kappa < 1e15 (early_word is 0 otherwise) and |U| components below 1e15 km/s: the whole
+//   box's (EmitBox::early), or the home cell's (256^3, 1e8 packets with one infinite cell:
+//   1.73 ms of emission, 2.54 with the direction of every packet drawn, 1.65 where the box is plain).
 __device__ __forceinline__ bool temperature_plain(float T) { return __float_as_uint(T) <= 0x58635fa9u; }
 __device__ __forceinline__ bool temperature_plain(double T) { return (uint32_t)__double2hiint(T) < 0x430c6bf5u; }
+template <class V>
+__device__ __forceinline__ bool velocity_plain(const V& U) {
+  return velq_upper(U.x) < 1e15f && velq_upper(U.y) < 1e15f && velq_upper(U.z) < 1e15f;
+}
 
 // Emission in 64-packet windows.  The first Philox block of every packet
 // gives its frequency; the packets with xi <= 0 (about half) are absorbed at
@@ -1247,6 +1267,7 @@ __device__ __forceinline__ void emit_window64(const TransportArgs<R>& a, const E
     if (act) {
       r = draw(KStream{a.ks, e.box}, cell, j, Draws<R>::kQuantBlock);
       early = r.d < e.early && temperature_plain(__ldg(e.T + cell));
+      if (e.early == 0u) early = r.d < a.early && temperature_plain(__ldg(e.T + cell)) && velocity_plain(e.vel[cell]);
     }
     // home tally of the early packets (warp-aggregated)
     const unsigned em = __ballot_sync(0xffffffffu, early);
@@ -1278,7 +1299,7 @@ template <class R> constexpr int emit_occupancy() { return sizeof(R) == 4 ? 5 : 
 template <class R, bool P2>
 __global__ void __launch_bounds__(TT, emit_occupancy<R>()) k_emit(TransportArgs<R> a) {
   const EmitBox<R> e{a.P, a.first, (uint32_t)a.n3, (uint32_t)a.n, a.vel, a.T, a.tally, a.kappa, a.cth, 0u, a.tl, 0u,
-                     a.sc->vq_u > 0.0f ? a.early : 0u};
+                     a.sc->vel_plain ? a.early : 0u};
   const uint32_t N = __ldg(a.P + a.n3);  // packets actually allocated
   __shared__ EmitStash<R> stash[TT / 32];
   EmitStash<R>& st = stash[threadIdx.x >> 5];
@@ -1464,10 +1485,11 @@ __device__ __forceinline__ void transport_end_batch(const BoxDev* bxs, int B, co
 
 // P2: the box side is a power of two (periodic wrap by masks).
 // MB: batched context; the lanes of a warp may hold packets of different boxes.
-template <class R, bool P2, bool MB, bool RS = false>
-__global__ void __launch_bounds__(TT, (march_occupancy<R, MB, RS>())) k_march(TransportArgs<R> a, const BoxDev* bxs,
-                                                                              int B, const BoxStep* bst,
-                                                                              rec_stats* st) {
+// OUT: cells beyond the scale of the copy exist, which are candidates whatever their
+// threshold (a body of its own: the test costs the others 2 %).
+template <class R, bool P2, bool MB, bool RS, bool OUT>
+__device__ __forceinline__ void march_body(const TransportArgs<R>& a, const BoxDev* bxs, int B, const BoxStep* bst,
+                                           BoxCounters& cnt) {
   static_assert(!RS || (P2 && !MB), "region sweeps: single box of power-of-two side");
   static_assert(!MB || !P2, "a batch mixes sides");
   using V = typename Vec4<R>::T;
@@ -1479,8 +1501,6 @@ __global__ void __launch_bounds__(TT, (march_occupancy<R, MB, RS>())) k_march(Tr
   uint32_t cbk = 0;
   float leave = 0.0f;
   bool gone = false;  // it has left, and waits to be queued again
-  __shared__ BoxCounters cnt;
-  if (MB) box_counters_clear(cnt, B);
   // box of the lane's packet and of the open chunk
   int lbox = -1, cbox = 0;
   const uint32_t* q = a.velq;
@@ -1514,7 +1534,9 @@ __global__ void __launch_bounds__(TT, (march_occupancy<R, MB, RS>())) k_march(Tr
 #pragma unroll
         for (int k = 0; k < kA; ++k) {
           const int thr = __float_as_int(fmaf(-bound_exit(se[k]), vp.c1, vp.c2));
-          if (velq_dot(qw[k], vp.m, kVelqBiasBits) >= thr || kc - (uint32_t)(kA - k) >= kMaxCrossings) cand |= 1u << k;
+          if (velq_dot(qw[k], vp.m, kVelqBiasBits) >= thr || (OUT && velq_is_out(qw[k])) ||
+              kc - (uint32_t)(kA - k) >= kMaxCrossings)
+            cand |= 1u << k;
         }
         cand &= 0xffffffffu << kfrom;
         if (cand == 0) {
@@ -1697,7 +1719,7 @@ __global__ void __launch_bounds__(TT, (march_occupancy<R, MB, RS>())) k_march(Tr
           {
             const DevScalars* bsc = MB ? bxs[lbox].sc : a.sc;
             const VelqBox vb = velq_box(q ? bsc->vq_u : 0.0f, bsc->vq_v, (float)lkappa);
-            vp = velq_packet(vb, (float)knx, (float)kny, (float)knz, (float)u0);
+            vp = velq_packet<OUT>(vb, (float)knx, (float)kny, (float)knz, (float)u0);
           }
           active = true;
         }
@@ -1725,14 +1747,36 @@ __global__ void __launch_bounds__(TT, (march_occupancy<R, MB, RS>())) k_march(Tr
 #pragma unroll
       for (int k = 0; k < kA; ++k)
         parked |= velq_dot(qw[k], vp.m, kVelqBiasBits) >= __float_as_int(fmaf(-bound_exit(se[k]), vp.c1, vp.c2));
+      if (OUT) {
+        uint32_t any = 0;
+#pragma unroll
+        for (int k = 0; k < kA; ++k) any |= qw[k];
+        parked |= velq_is_out(any);
+      }
       // a packet that left its region waits for the warp's next stop, so that the
       // append runs with many lanes: with one or two lanes after each round
       // the sweeps of 512^3, 1e9 packets took 70.9 ms, with this 65.3
       if (RS && !parked && bound_exit(se[kA - 1]) >= leave) gone = parked = true;
     }
   }
+  if (!MB) add_counters(a.sc, my_abs, my_cap, my_cross);
+  else if (lbox >= 0) box_counters_add(cnt, lbox, my_abs, my_cap, my_cross);
+}
+
+template <class R, bool P2, bool MB, bool RS = false>
+__global__ void __launch_bounds__(TT, (march_occupancy<R, MB, RS>())) k_march(TransportArgs<R> a, const BoxDev* bxs,
+                                                                              int B, const BoxStep* bst,
+                                                                              rec_stats* st) {
+  __shared__ BoxCounters cnt;
+  bool out = !MB && a.sc->vq_out != 0;
   if (MB) {
-    if (lbox >= 0) box_counters_add(cnt, lbox, my_abs, my_cap, my_cross);
+    box_counters_clear(cnt, B);
+    for (int b = threadIdx.x & 31; b < B; b += 32) out |= bxs[b].sc->vq_out != 0;
+    out = __any_sync(0xffffffffu, out);
+  }
+  if (!out) march_body<R, P2, MB, RS, false>(a, bxs, B, bst, cnt);
+  else march_body<R, P2, MB, RS, true>(a, bxs, B, bst, cnt);
+  if (MB) {
     box_counters_flush(cnt, bxs, B);
     // the last block to finish closes the call: queued counts, tally totals, statistics
     if (last_block_done(&a.sc->counter)) {
@@ -1740,7 +1784,6 @@ __global__ void __launch_bounds__(TT, (march_occupancy<R, MB, RS>())) k_march(Tr
       if (threadIdx.x == 0) a.sc->counter = 0;
     }
   } else {
-    add_counters(a.sc, my_abs, my_cap, my_cross);
     // the last block of the last march closes the call: tally total, statistics
     if (!a.closes || !last_block_done(&a.sc->counter)) return;
     if (threadIdx.x == 0) {
@@ -1852,8 +1895,8 @@ void alloc_launch(rec_ctx* c, int blocks, const typename Vec4<R>::T* vel, const 
 // one rounding (2^-23 relative covers both precisions), and a node is safe if
 // interpolation from it cannot pass zero by rounding: its upper end q1 = 0 (then q1 - q0 is
 // exact), or q1 <= -2^-20 |q0|.
-uint32_t early_word(const rec_ctx* c, double cth) {
-  if (!(cth <= 1e15)) return 0u;
+uint32_t early_word(const rec_ctx* c, double kappa, double cth) {
+  if (!(cth <= 1e15) || !(kappa < 1e15)) return 0u;
   const double w = std::floor((double)c->early_nodes / (double)(c->params.n_quantiles - 1) * (1.0 - 0x1p-22) * 0x1p32) - 258.0;
   return w > 0.0 ? (uint32_t)std::min(w, 4294967295.0) : 0u;
 }
@@ -1890,7 +1933,7 @@ cudaError_t run_transport(rec_ctx* c, int step, double z, rec_stats* st) {
   a.cth = (R)cth;
   a.strm = s;
   a.ks = key_schedule(s.k0, s.k1);
-  a.early = early_word(c, cth);
+  a.early = early_word(c, kappa, cth);
   a.tally = b.tally;
   a.sc = c->sc;
   a.queue = (typename Vec4<R>::T*)c->queue;
@@ -1991,7 +2034,7 @@ __device__ __forceinline__ void alloc_max_batch(const BoxDev* bxs, const BoxStep
   }
   block_maxima<AT>(d.sc, order_bits(m), vm, bad);
   if (!last_block_done(&gsc->counter, ng)) return;
-  for (int i = threadIdx.x; i < B; i += AT) take_maxima<R>(bxs[i].sc, (float)(R)bs.s[i].kappa);
+  for (int i = threadIdx.x; i < B; i += AT) take_maxima<R>(bxs[i].sc, bxs[i].n3, (float)(R)bs.s[i].kappa);
   if (threadIdx.x == 0) gsc->counter = 0;
 }
 template <class R>
@@ -2109,7 +2152,7 @@ __device__ __forceinline__ void emit_batch_body(const TransportArgs<R>& a, const
     return EmitBox<R>{d.P, d.first, (uint32_t)d.n3, d.n, (const V*)d.vel4, (const R*)d.T, d.tally,
                       (R)__ldcg(&bst[b].kappa), (R)__ldcg(&bst[b].cth),
                       (uint32_t)b, Tiles{d.n, d.nt, d.lg, d.mn, d.mn2, d.tlg}, d.bk0,
-                      __ldcg(&d.sc->vq_u) > 0.0f ? a.early : 0u};
+                      __ldcg(&d.sc->vel_plain) ? a.early : 0u};
   };
   const uint64_t warps_total = (uint64_t)gridDim.x * (TT / 32);
   for (uint64_t gbase = ((uint64_t)blockIdx.x * (TT / 32) + (threadIdx.x >> 5)) * 64; gbase < tot_pk;
@@ -2211,9 +2254,12 @@ cudaError_t run_transport_batch(rec_ctx* c, int step, double z, rec_stats* st) {
   a.M = c->params.n_quantiles;
   a.strm = Stream{k0, k1, 0u};
   a.ks = key_schedule(k0, k1);
-  double cth_max = 0.0;
-  for (int b = 0; b < B; ++b) cth_max = std::max(cth_max, bs.s[b].cth);
-  a.early = early_word(c, cth_max);
+  double kappa_max = 0.0, cth_max = 0.0;
+  for (int b = 0; b < B; ++b) {
+    kappa_max = std::max(kappa_max, (double)bs.s[b].kappa);
+    cth_max = std::max(cth_max, (double)bs.s[b].cth);
+  }
+  a.early = early_word(c, kappa_max, cth_max);
   a.sc = c->gsc;
   a.queue = (typename Vec4<R>::T*)c->queue;
   a.nb = nb;
