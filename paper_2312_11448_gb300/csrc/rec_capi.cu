@@ -14,6 +14,7 @@
 #include <vector>
 
 #include "rec_internal.cuh"
+#include "rec_scratch.h"
 #include "rec_velq.cuh"
 
 namespace {
@@ -120,31 +121,34 @@ struct Carver {
     used += round_up(std::max<size_t>(bytes, 1), 256);
   }
 };
-// lay(carver, optional): sets the pointers; optional: with the scratch that only saves
-// time.  That is left out where it would take more than an eighth of the memory
-// that is free, or cannot be had.
+// lay(carver, level): sets the pointers, with the optional scratch of a level
+// (rec_scratch.h).  Less of it where it cannot be had; REC_SCRATCH=least or =copy asks for
+// less from the start.
 template <class F>
 cudaError_t carve_scratch(rec_ctx* c, F lay) {
-  Carver need, with;
-  lay(need, false);
-  lay(with, true);
-  const size_t extra = with.used - need.used;
-  bool optional = extra > 0;
-  if (extra > ((size_t)256 << 20)) {
-    size_t free_bytes = 0, total = 0;
-    optional = cudaMemGetInfo(&free_bytes, &total) == cudaSuccess && extra <= free_bytes / 8;
+  size_t bytes[3];
+  for (int level = 0; level < 3; ++level) {
+    Carver m;
+    lay(m, level);
+    bytes[level] = m.used;
   }
-  cudaError_t e = cudaErrorMemoryAllocation;
-  if (optional) e = cudaMalloc(&c->slab, with.used);
-  if (e == cudaErrorMemoryAllocation) {
+  size_t free_bytes = ~(size_t)0, total = 0;
+  if (bytes[2] - bytes[0] > ((size_t)256 << 20) && cudaMemGetInfo(&free_bytes, &total) != cudaSuccess) free_bytes = 0;
+  int level = rec::scratch_level(bytes[1] - bytes[0], bytes[2] - bytes[1], free_bytes);
+  if (const char* sel = std::getenv("REC_SCRATCH")) {
+    if (std::strcmp(sel, "least") == 0) level = rec::kScratchLeast;
+    if (std::strcmp(sel, "copy") == 0) level = std::min<int>(level, rec::kScratchCopy);
+  }
+  cudaError_t e = cudaMalloc(&c->slab, bytes[level]);
+  while (e == cudaErrorMemoryAllocation && level > 0) {
     cudaGetLastError();
-    optional = false;
-    e = cudaMalloc(&c->slab, need.used);
+    --level;
+    e = cudaMalloc(&c->slab, bytes[level]);
   }
   if (e != cudaSuccess) { c->slab = nullptr; return e; }
   Carver at;
   at.base = (char*)c->slab;
-  lay(at, optional);
+  lay(at, level);
   return cudaSuccess;
 }
 
@@ -234,7 +238,7 @@ rec_status init_batch(const rec_params* params, const rec_box* boxes, int32_t n_
   const size_t qbytes = (size_t)params->n_quantiles * (mixed ? 4 : 8);
   const size_t part_n = std::max<size_t>(2 * (size_t)rec::kMaxSums * c->tot_pblk, (size_t)rec::kMaxSums * c->tot_ablk);
   const size_t qentry = mixed ? 32 : 96;  // two float4 | three double4 per queued packet
-  e = carve_scratch(c, [&](Carver& m, bool optional) {
+  e = carve_scratch(c, [&](Carver& m, int level) {
     m.take(&c->sc, sizeof(rec::DevScalars) * n_boxes);
     m.take(&c->gsc, sizeof(rec::DevScalars));
     m.take(&c->sc_adj, sizeof(rec::DevScalars));
@@ -251,7 +255,7 @@ rec_status init_batch(const rec_params* params, const rec_box* boxes, int32_t n_
     m.take(&c->bx, sizeof(rec::BoxDev) * n_boxes);
     m.take(&c->bstep, sizeof(rec::BoxStep) * n_boxes);
     c->velq = nullptr;
-    if (optional) m.take(&c->velq, sizeof(uint32_t) * nvelq);
+    if (level >= rec::kScratchCopy) m.take(&c->velq, sizeof(uint32_t) * nvelq);
   });
   if (e != cudaSuccess) {
     rec_status r = (e == cudaErrorMemoryAllocation) ? fail(nullptr, REC_ENOMEM, "device allocation failed")
@@ -351,7 +355,7 @@ rec_status rec_init(const rec_params* params, const rec_box* boxes, int32_t n_bo
   const size_t n3 = (size_t)c->n3;
   // super-tiles of the march queue, sized for the smallest tile side
   const size_t nt = (size_t)((b.n + rec::kMinTile - 1) / rec::kMinTile), nb = nt * nt * nt;
-  e = carve_scratch(c, [&](Carver& m, bool optional) {
+  e = carve_scratch(c, [&](Carver& m, int level) {
     m.take(&c->sc, sizeof(rec::DevScalars));
     m.take(&c->sc_adj, sizeof(rec::DevScalars));
     // block partials (two per block: the TMA-staged passes run more blocks than the grid)
@@ -370,10 +374,9 @@ rec_status rec_init(const rec_params* params, const rec_box* boxes, int32_t n_bo
     m.take(&c->queue, (mixed ? 32 : 96) * (size_t)std::max<uint64_t>(b.n_packets, 1));
     c->velq = nullptr;
     c->cellcache = nullptr;
-    if (optional) {
-      m.take(&c->velq, sizeof(uint32_t) * rec::velq_words((uint32_t)b.n));
-      if (!mixed && params->mixing != REC_MIX_LOCAL) m.take(&c->cellcache, 5 * sizeof(double) * n3);
-    }
+    if (level >= rec::kScratchCopy) m.take(&c->velq, sizeof(uint32_t) * rec::velq_words((uint32_t)b.n));
+    if (level >= rec::kScratchAll && !mixed && params->mixing != REC_MIX_LOCAL)
+      m.take(&c->cellcache, 5 * sizeof(double) * n3);
   });
   if (e != cudaSuccess) {
     rec_status r = (e == cudaErrorMemoryAllocation) ? fail(nullptr, REC_ENOMEM, "device allocation failed")
