@@ -104,6 +104,14 @@ rec_tuning default_tuning(bool mixed, bool batch, uint64_t packets, int sm_count
   return t;
 }
 
+// Without the compact velocity copy a lane never waits for its warp's next stop, so
+// a refill pays earlier (256^3, 1e8 packets: 6.39 / 6.25 / 6.51 ms per march at 16 / 8 / 4 idle
+// lanes, 6.18 with chunks of 64).
+void direct_tuning(rec_tuning* t) {
+  t->march_refill = 8;
+  t->march_chunk = std::min(t->march_chunk, 64);
+}
+
 uint32_t log2u(uint32_t v) {
   uint32_t l = 0;
   while ((1u << l) < v) ++l;
@@ -263,6 +271,7 @@ rec_status init_batch(const rec_params* params, const rec_box* boxes, int32_t n_
     rec_free(c);
     return r;
   }
+  if (!c->velq) direct_tuning(&c->tune);
   nvelq = 0;
   for (int i = 0; i < n_boxes; ++i) {
     const rec_box& b = boxes[i];
@@ -384,6 +393,7 @@ rec_status rec_init(const rec_params* params, const rec_box* boxes, int32_t n_bo
     rec_free(c);
     return r;
   }
+  if (!c->velq) direct_tuning(&c->tune);
   // emission-profile table in the working precision of the transport
   std::vector<char> hq(qbytes);
   for (int i = 0; i < params->n_quantiles; ++i) {

@@ -1485,15 +1485,17 @@ __device__ __forceinline__ void transport_end_batch(const BoxDev* bxs, int B, co
 
 // P2: the box side is a power of two (periodic wrap by masks).
 // MB: batched context; the lanes of a warp may hold packets of different boxes.
-// OUT: cells beyond the scale of the copy exist, which are candidates whatever their
-// threshold (a body of its own: the test costs the others 2 %).
-template <class R, bool P2, bool MB, bool RS, bool OUT>
+// F: kCopyOut: cells beyond the scale of the copy exist, which are candidates whatever
+// their threshold (a body of its own: the test costs the others 2 %).  kDirect: a context
+// without the copy reads the velocity of every cell, a few cells ahead of the tests.
+enum MarchForm { kCopy, kCopyOut, kDirect };
+template <class R, bool P2, bool MB, bool RS, MarchForm F>
 __device__ __forceinline__ void march_body(const TransportArgs<R>& a, const BoxDev* bxs, int B, const BoxStep* bst,
                                            BoxCounters& cnt) {
   static_assert(!RS || (P2 && !MB), "region sweeps: single box of power-of-two side");
   static_assert(!MB || !P2, "a batch mixes sides");
   using V = typename Vec4<R>::T;
-  constexpr int kA = MarchAhead<R, RS>::value;
+  constexpr int kA = F != kDirect ? MarchAhead<R, RS>::value : (sizeof(R) == 4 ? 4 : 2);
   const int lane = threadIdx.x & 31;
   const uint32_t n = (uint32_t)a.n;
   // region sweeps: bucket of the open chunk (its super-tile); path length at
@@ -1504,13 +1506,21 @@ __device__ __forceinline__ void march_body(const TransportArgs<R>& a, const BoxD
   // box of the lane's packet and of the open chunk
   int lbox = -1, cbox = 0;
   const uint32_t* q = a.velq;
-  VelqMasks lm = a.vm;
   uint32_t bx = a.vbx, ln = n;
+  // A cell as three parts, one per axis, that a step adds to under a mask: of the copy's
+  // word index, or without the copy of the cell index (power-of-two side) or ten bits per axis.
+  const uint32_t sh = P2 ? a.tl.lg : 10u, low = P2 ? n - 1u : 1023u;
+  auto part_x = [&](uint32_t i) { return F == kDirect ? i : velq_x(i); };
+  auto part_y = [&](uint32_t i) { return F == kDirect ? i << sh : velq_y(i, bx); };
+  auto part_z = [&](uint32_t i) { return F == kDirect ? i << (2u * sh) : velq_z(i, bx); };
+  auto coords = [&](uint32_t c, uint32_t* ix, uint32_t* iy, uint32_t* iz) {
+    if (F != kDirect) return velq_coords(c, bx, ix, iy, iz);
+    *ix = c & low; *iy = (c >> sh) & low; *iz = c >> (2u * sh);
+  };
+  VelqMasks lm = F == kDirect ? VelqMasks{low, low << sh, low << (2u * sh)} : a.vm;
   uint32_t lastx = 0, lasty = 0, lastz = 0;
   R lkappa = a.kappa;
-  if (!MB) {
-    lastx = velq_x(n - 1u); lasty = velq_y(n - 1u, bx); lastz = velq_z(n - 1u, bx);
-  }
+  if (!MB) { lastx = part_x(n - 1u); lasty = part_y(n - 1u); lastz = part_z(n - 1u); }
   uint64_t pos = 0;   // next queue slot of the open chunk
   uint32_t left = 0;  // slots left in it
   bool more = true;
@@ -1529,12 +1539,12 @@ __device__ __forceinline__ void march_body(const TransportArgs<R>& a, const BoxD
     const unsigned stop = __ballot_sync(0xffffffffu, !active || parked);
     if (__popc(stop) >= a.refill || stop == 0xffffffffu) {
       // exact test of the parked lanes' first candidate cell
-      if (parked && !(RS && gone)) {
+      if (F != kDirect && parked && !(RS && gone)) {
         uint32_t cand = 0;
 #pragma unroll
         for (int k = 0; k < kA; ++k) {
           const int thr = __float_as_int(fmaf(-bound_exit(se[k]), vp.c1, vp.c2));
-          if (velq_dot(qw[k], vp.m, kVelqBiasBits) >= thr || (OUT && velq_is_out(qw[k])) ||
+          if (velq_dot(qw[k], vp.m, kVelqBiasBits) >= thr || (F == kCopyOut && velq_is_out(qw[k])) ||
               kc - (uint32_t)(kA - k) >= kMaxCrossings)
             cand |= 1u << k;
         }
@@ -1582,7 +1592,7 @@ __device__ __forceinline__ void march_body(const TransportArgs<R>& a, const BoxD
         const unsigned rm = __ballot_sync(0xffffffffu, gone);
         if (rm) {
           uint32_t ix, iy, iz;
-          velq_coords(X | Y | Z, bx, &ix, &iy, &iz);
+          coords(X | Y | Z, &ix, &iy, &iz);
           const uint32_t cell = (((iz << a.tl.lg) | iy) << a.tl.lg) | ix;
           // the warp's part of the second queue
           const uint32_t part = (blockIdx.x * (TT / 32) + (threadIdx.x >> 5)) & (uint32_t)(kRqParts - 1);
@@ -1622,8 +1632,8 @@ __device__ __forceinline__ void march_body(const TransportArgs<R>& a, const BoxD
           if (lane == 0) nc = atomicAdd(&a.sc->march_next, 1ull);
           const uint64_t chunk = __shfl_sync(0xffffffffu, nc, 0);
           if (chunk >= __ldg(a.cpre + a.nb)) { more = false; break; }
-          // bucket of this chunk: last b with cpre[b] <= chunk (cpre[0] = 0), the lanes
-          // probing 32 places at once, so two rounds of loads for up to 1024 buckets
+          // bucket of this chunk: last b with cpre[b] <= chunk (cpre[0] = 0).  A binary search, the
+          // same in every lane (the lanes probing 32 places at once: 3.60 against 3.43 ms at 256^3)
           uint32_t lo = 0, hi = (uint32_t)a.nb;
           while (hi - lo > 1) {
             uint32_t mid = (lo + hi) >> 1;
@@ -1649,10 +1659,10 @@ __device__ __forceinline__ void march_body(const TransportArgs<R>& a, const BoxD
               const BoxDev& d = bxs[lbox];
               ln = d.n;
               bx = d.vbx;
-              lm = velq_masks(ln, bx, false);
+              if (F != kDirect) lm = velq_masks(ln, bx, false);
               q = d.velq;
               lkappa = (R)bst[lbox].kappa;
-              lastx = velq_x(ln - 1u); lasty = velq_y(ln - 1u, bx); lastz = velq_z(ln - 1u, bx);
+              lastx = part_x(ln - 1u); lasty = part_y(ln - 1u); lastz = part_z(ln - 1u);
             }
           }
           uint32_t cell;
@@ -1695,7 +1705,7 @@ __device__ __forceinline__ void march_body(const TransportArgs<R>& a, const BoxD
           } else {
             a.tl.template coords<P2>(cell, &ix, &iy, &iz);
           }
-          X = velq_x(ix); Y = velq_y(iy, bx); Z = velq_z(iz, bx);
+          X = part_x(ix); Y = part_y(iy); Z = part_z(iz);
           if (RS) {
             // the region: the bucket's super-tile widened by the halo (periodic:
             // offsets from its low corner modulo n).  Along an axis the packet leaves
@@ -1713,13 +1723,13 @@ __device__ __forceinline__ void march_body(const TransportArgs<R>& a, const BoxD
             }
           }
           Sx = sx > 0 ? 0u - lm.x : 0u - 1u;
-          Sy = sy > 0 ? 0u - lm.y : 0u - 2u;
-          Sz = sz > 0 ? 0u - lm.z : 0u - 4u;
+          Sy = sy > 0 ? 0u - lm.y : 0u - (F == kDirect ? 1u << sh : 2u);
+          Sz = sz > 0 ? 0u - lm.z : 0u - (F == kDirect ? 1u << (2u * sh) : 4u);
           if (!P2) { Ex = sx > 0 ? lastx : 0u; Ey = sy > 0 ? lasty : 0u; Ez = sz > 0 ? lastz : 0u; }
-          {
+          if (F != kDirect) {
             const DevScalars* bsc = MB ? bxs[lbox].sc : a.sc;
-            const VelqBox vb = velq_box(q ? bsc->vq_u : 0.0f, bsc->vq_v, (float)lkappa);
-            vp = velq_packet<OUT>(vb, (float)knx, (float)kny, (float)knz, (float)u0);
+            const VelqBox vb = velq_box(bsc->vq_u, bsc->vq_v, (float)lkappa);
+            vp = velq_packet<F == kCopyOut>(vb, (float)knx, (float)kny, (float)knz, (float)u0);
           }
           active = true;
         }
@@ -1729,7 +1739,45 @@ __device__ __forceinline__ void march_body(const TransportArgs<R>& a, const BoxD
       }
     }
     if (!__any_sync(0xffffffffu, active)) break;  // no packet left in the warp
-    if (active && !parked) {
+    if (F == kDirect && active && !parked) {
+      // one round: walk kA cells and read their velocities, then test them in order
+      uint32_t lin[kA];
+      V U[kA];
+      const V* vel = MB ? (const V*)bxs[lbox].vel4 : a.vel;
+#pragma unroll
+      for (int k = 0; k < kA; ++k) {
+        lin[k] = P2 ? X | Y | Z : ((Z >> 20) * ln + (Y >> 10)) * ln + X;
+        U[k] = vel[lin[k]];
+        if (P2)
+          se[k] = walk_step(tMx, tMy, tMz, tDx, tDy, tDz, X, Y, Z, Sx, Sy, Sz, lm.x, lm.y, lm.z);
+        else
+          se[k] = walk_step_any(tMx, tMy, tMz, tDx, tDy, tDz, X, Y, Z, Sx, Sy, Sz, lm.x, lm.y, lm.z, Ex, Ey, Ez, lastx,
+                                lasty, lastz);
+      }
+      Ray<R> r;
+      r.knx = knx; r.kny = kny; r.knz = knz;
+      bool hit = false;
+      uint32_t at = 0, kcell = kc;
+#pragma unroll
+      for (int k = 0; k < kA; ++k) {
+        if (!active) continue;
+        hit = Ar<R>::sub(u0, doppler(r, U[k])) <= se[k];
+        if (hit || kc + (uint32_t)k >= kMaxCrossings) { active = false; at = lin[k]; kcell = kc + (uint32_t)k; }
+      }
+      kc += kA;
+      if (!active) {
+        my_cross += kcell - 1;
+        if (my_cross >= 0x80000000u) {
+          if (MB) box_counters_add(cnt, lbox, 0, 0, my_cross);
+          else atomicAdd(&a.sc->crossings, (unsigned long long)my_cross);
+          my_cross = 0;
+        }
+        if (hit) { atomicAdd((MB ? bxs[lbox].tally : a.tally) + at, 1u); ++my_abs; }
+        else ++my_cap;
+      } else if (RS && bound_exit(se[kA - 1]) >= leave) {
+        gone = parked = true;
+      }
+    } else if (F != kDirect && active && !parked) {
       // one round: walk kA cells, loading the words that matter, then ask the bound
 #pragma unroll
       for (int k = 0; k < kA; ++k) {
@@ -1747,7 +1795,7 @@ __device__ __forceinline__ void march_body(const TransportArgs<R>& a, const BoxD
 #pragma unroll
       for (int k = 0; k < kA; ++k)
         parked |= velq_dot(qw[k], vp.m, kVelqBiasBits) >= __float_as_int(fmaf(-bound_exit(se[k]), vp.c1, vp.c2));
-      if (OUT) {
+      if (F == kCopyOut) {
         uint32_t any = 0;
 #pragma unroll
         for (int k = 0; k < kA; ++k) any |= qw[k];
@@ -1763,19 +1811,21 @@ __device__ __forceinline__ void march_body(const TransportArgs<R>& a, const BoxD
   else if (lbox >= 0) box_counters_add(cnt, lbox, my_abs, my_cap, my_cross);
 }
 
-template <class R, bool P2, bool MB, bool RS = false>
+template <class R, bool P2, bool MB, bool RS, bool COPY>
 __global__ void __launch_bounds__(TT, (march_occupancy<R, MB, RS>())) k_march(TransportArgs<R> a, const BoxDev* bxs,
                                                                               int B, const BoxStep* bst,
                                                                               rec_stats* st) {
   __shared__ BoxCounters cnt;
-  bool out = !MB && a.sc->vq_out != 0;
+  bool out = COPY && !MB && a.sc->vq_out != 0;
   if (MB) {
     box_counters_clear(cnt, B);
-    for (int b = threadIdx.x & 31; b < B; b += 32) out |= bxs[b].sc->vq_out != 0;
+    if (COPY)
+      for (int b = threadIdx.x & 31; b < B; b += 32) out |= bxs[b].sc->vq_out != 0;
     out = __any_sync(0xffffffffu, out);
   }
-  if (!out) march_body<R, P2, MB, RS, false>(a, bxs, B, bst, cnt);
-  else march_body<R, P2, MB, RS, true>(a, bxs, B, bst, cnt);
+  if (!COPY) march_body<R, P2, MB, RS, kDirect>(a, bxs, B, bst, cnt);
+  else if (!out) march_body<R, P2, MB, RS, kCopy>(a, bxs, B, bst, cnt);
+  else march_body<R, P2, MB, RS, kCopyOut>(a, bxs, B, bst, cnt);
   if (MB) {
     box_counters_flush(cnt, bxs, B);
     // the last block to finish closes the call: queued counts, tally totals, statistics
@@ -1890,6 +1940,15 @@ void alloc_launch(rec_ctx* c, int blocks, const typename Vec4<R>::T* vel, const 
                                                       c->bfill, nb);
 }
 
+// Without the copy (256^3, 1e8 packets) the march takes 6.2 ms; as a bound that excludes
+// nothing, so that six cells cost a round and six stops, it took 21.6.
+template <class R, bool P2, bool MB, bool RS>
+void march_launch(rec_ctx* c, const TransportArgs<R>& a, int blocks, const BoxDev* bxs, int B, const BoxStep* bst,
+                  rec_stats* st) {
+  if (c->velq) k_march<R, P2, MB, RS, true><<<blocks, TT, 0, c->stream>>>(a, bxs, B, bst, st);
+  else k_march<R, P2, MB, RS, false><<<blocks, TT, 0, c->stream>>>(a, bxs, B, bst, st);
+}
+
 // Bound of the quantile's leading word w below which xi <= 0 (0: none).  The deviate
 // u < (w + 257) 2^-32 (binary32 keeps the top 23 bits and adds half a unit), the table node k = trunc(u (M - 1)) after
 // one rounding (2^-23 relative covers both precisions), and a node is safe if
@@ -1965,8 +2024,8 @@ cudaError_t run_transport(rec_ctx* c, int step, double z, rec_stats* st) {
   if (!sweeps) {
     GroupTimer t(c, kTMarch, 1);
     const int mb = c->sm_count * tu.march_blocks_per_sm;
-    if (p2) k_march<R, true, false><<<mb, TT, 0, c->stream>>>(a, nullptr, 1, nullptr, st);
-    else k_march<R, false, false><<<mb, TT, 0, c->stream>>>(a, nullptr, 1, nullptr, st);
+    if (p2) march_launch<R, true, false, false>(c, a, mb, nullptr, 1, nullptr, st);
+    else march_launch<R, false, false, false>(c, a, mb, nullptr, 1, nullptr, st);
   } else {
     // region sweeps: each march leaves the packets that stray beyond the halo of
     // their bucket's super-tile in the second queue; those are placed by the
@@ -1988,7 +2047,7 @@ cudaError_t run_transport(rec_ctx* c, int step, double z, rec_stats* st) {
       a.resumed = k > 0;
       a.closes = k + 1 == kMaxSweeps;
       a.halo = a.closes ? 0u : halo;
-      k_march<R, true, false, true><<<mb, TT, 0, c->stream>>>(a, nullptr, 1, nullptr, st);
+      march_launch<R, true, false, true>(c, a, mb, nullptr, 1, nullptr, st);
     }
   }
   return cudaGetLastError();
@@ -2311,8 +2370,7 @@ cudaError_t run_transport_batch(rec_ctx* c, int step, double z, rec_stats* st) {
   }
   {
     GroupTimer t(c, kTMarch, 1);
-    k_march<R, false, true><<<c->sm_count * c->tune.march_blocks_per_sm, TT, 0, c->stream>>>(a, c->bx, B, c->bstep,
-                                                                                             st);
+    march_launch<R, false, true, false>(c, a, c->sm_count * c->tune.march_blocks_per_sm, c->bx, B, c->bstep, st);
   }
   return cudaGetLastError();
 }
