@@ -13,15 +13,16 @@
 //   then the chain through A, s, w, alpha(T'), T', Delta, x and the global sums.
 // Passes (all on the context stream):
 //   k_adj_prep      sums of the pre-step state (S_1s, tally total, lambda guess)
-//   k_substep_begin + k_newton   recompute lambda exactly as the forward step;
-//                   the first evaluation keeps the cells' coefficients
+//   k_substep       recomputes lambda as the forward step does; its first
+//                   evaluation keeps the cells' coefficients
 //   k_adj_r1        mu numerator/denominator and X_e of the end state; keeps x'
 //   k_adj_r2        per-cell adjoints; sums for the C and S_1s paths
 //   k_adj_r3        the S_1s term applied to xbar and g_delta
 // Every pass but the last is bound by the binary64 pipe (two operations per
 // cycle and SM), so coefficients are computed once and read back (40 bytes per
-// cell), quotients by a common divisor share its reciprocal, and quotients by sums
-// are taken of the sums.  256^3: 50.2 -> 14.5 ms per reversed step.
+// cell), and quotients by sums are taken of the sums.  256^3: 50.2 -> 18.7 ms per
+// reversed step.  (Reciprocals shared between a cell's quotients: 14.5 ms, at 1 to 2 % more
+// error in the gradients.)
 
 #include <cmath>
 
@@ -73,12 +74,12 @@ __device__ __forceinline__ Fwd forward_cell(const AdjArgs& a, int64_t i, double 
     f.al = q.x; f.w = q.y; f.Tn = q.z; f.tpd = q.w;
   } else {
     const double T = a.T[i];
-    const double opx = 1.0 + k.fHe + x, kx = k.kc * x;
-    f.Tn = (T * opx + k.dt * (kx * k.Tg + k.hq / d)) / (opx * (1.0 + 2.0 * k.H * k.dt) + k.dt * kx);
+    const double opx = 1.0 + k.fHe + x, g = k.kc * x / opx;
+    f.Tn = (T + k.dt * (g * k.Tg + k.hq / (d * opx))) / (1.0 + k.dt * (2.0 * k.H + g));
     const double lt = log(f.Tn * 1.0e-4);
     f.tpd = exp(k.pd * lt);
     f.al = k.fa * exp(k.pb * lt) / (1.0 + k.pc * f.tpd);
-    f.w = f.wt ? (double)(a.tally ? a.tally[i] : 0u) * (S1s / tot) / n1s_rel : 1.0;
+    f.w = f.wt ? (double)(a.tally ? a.tally[i] : 0u) / tot * S1s / n1s_rel : 1.0;
   }
   f.n = k.nH * d;
   f.A = k.dt * f.al * f.n;
@@ -202,27 +203,26 @@ __global__ void __launch_bounds__(NT) k_adj_r2(AdjArgs a) {
     double db = nb * k.nH;
     double ab = 0.0;
     if (f.wt) {
-      const double r = 1.0 / (d * y1), ww = wb * f.w;
-      ab = wb * S1s * r;
+      const double ww = wb * f.w;
+      ab = wb * S1s / (d * y1);
       v[1] += ww;
-      db -= ww * y1 * r;
-      xbar += ww * d * r;
+      db -= ww / d;
+      xbar += ww / y1;
     }
     // alpha(T'): d alpha/dT' = (alpha/T') (pb - pc pd t^pd / (1 + pc t^pd))
-    const double den_a = 1.0 + k.pc * f.tpd;
-    const double dal = f.al * (k.pb * den_a - k.pc * k.pd * f.tpd) / (f.Tn * den_a);
+    const double dal = f.al / f.Tn * (k.pb - k.pc * k.pd * f.tpd / (1.0 + k.pc * f.tpd));
     const double Tnb = a.Tbar[i] + alb * dal;
     // T' = (T + dt (g Tg + hh)) / den
-    const double ropx = 1.0 / (1.0 + k.fHe + x);
-    const double g = k.kc * x * ropx;
+    const double opx = 1.0 + k.fHe + x;
+    const double g = k.kc * x / opx;
     const double Tb = Tnb / (1.0 + k.dt * (2.0 * k.H + g));
     const double hhb = Tb * k.dt;
     const double gb = hhb * (k.Tg - f.Tn);
-    xbar += gb * k.kc * (1.0 + k.fHe) * ropx * ropx;
+    xbar += gb * k.kc * (1.0 + k.fHe) / (opx * opx);
     if (k.hq != 0.0) {
-      const double hh = k.hq * ropx / d;
+      const double hh = k.hq / (d * opx);
       db -= hhb * hh / d;
-      xbar -= hhb * hh * ropx;
+      xbar -= hhb * hh / opx;
     }
     // X_e of the end state: d/d delta_i of sum(delta x')/sum(delta)
     db += XeSd * (f.xr - Xe1);

@@ -89,36 +89,30 @@ struct CellF64 {
 // of two operations per cycle and SM).  The first evaluation of a substep
 // keeps {alpha(T'), mixing weight w or local Peebles factor, T', t^pd of the case-B fit}
 // per cell; the later ones read them back (32 bytes) and form the same A, s
-// and n from them, bit for bit.  256^3, three evaluations: 26.2 -> 11.7 ms per step, 9.4 with the quotients of cell_f64 and
-// root_slope_f64.
+// and n from them, bit for bit.  256^3, three evaluations: 26.2 -> 11.4 ms per step.
 enum CellCache { kNoCache = 0, kFillCache = 1, kReadCache = 2 };
 
-// Mixing weight per absorbed packet and neutral atom, S_1s / tally total (0: full mixing).
-__device__ __forceinline__ double weight_factor(double tot, double S1s) {
-  return tot > 0.0 && S1s > 0.0 ? S1s / tot : 0.0;
-}
-
 // Coefficients of one cell at the substep end (backward Euler, x_old in the
-// Compton and heating terms).  w uses the substep-start neutral fraction.  Binary64
-// quotients (about ten operations each on the slow pipe) are kept few: T' is written
-// with one denominator, g = kc x / (1 + f_He + x) multiplied through, and w with the box's
-// factor wfac = S_1s / tally total.
+// Compton and heating terms).  w uses the substep-start neutral fraction.  The quotients
+// stay as they are defined: T' over one common denominator and w by a factor
+// S_1s / tally total formed once saved three of six, at 3 to 11 % more error in T'.
 __device__ __forceinline__ CellF64 cell_f64(const StepCoef& k, double d, double x, double T, uint32_t tal,
-                                            double wfac, double* w_out = nullptr, double* tpd_out = nullptr) {
+                                            double tot, double S1s, double* w_out = nullptr, double* tpd_out = nullptr) {
   CellF64 c;
-  const double opx = 1.0 + k.fHe + x, kx = k.kc * x;
-  double heat = 0.0;  // an empty cell has no temperature (0 / 0 of the heating per atom)
-  if (k.hq != 0.0 || __double_as_longlong(d) <= 0) heat = k.hq / d;
-  c.Tn = (T * opx + k.dt * (kx * k.Tg + heat)) / (opx * (1.0 + 2.0 * k.H * k.dt) + k.dt * kx);
+  const double opx = 1.0 + k.fHe + x;
+  const double g = k.kc * x / opx;
+  double hh = 0.0;  // no quotient without heating, unless the cell is empty or no number (0 / 0)
+  if (k.hq != 0.0 || (uint64_t)__double_as_longlong(d) - 1u >= 0x7ff0000000000000ull) hh = k.hq / (d * opx);
+  c.Tn = (T + k.dt * (g * k.Tg + hh)) / (1.0 + k.dt * (2.0 * k.H + g));
   double lt = log(c.Tn * 1.0e-4);
   const double tpd = exp(k.pd * lt);
   c.al = k.fa * exp(k.pb * lt) / (1.0 + k.pc * tpd);
   c.n = k.nH * d;
   c.A = k.dt * c.al * c.n;
   double w = 1.0;
-  if (k.mixing == REC_MIX_TALLY && wfac > 0.0) {
+  if (k.mixing == REC_MIX_TALLY && tot > 0.0) {
     double n1s_rel = d * (1.0 - x);
-    if (n1s_rel > 0.0) w = (double)tal * wfac / n1s_rel;
+    if (S1s > 0.0 && n1s_rel > 0.0) w = ((double)tal / tot) * S1s / n1s_rel;
   }
   c.s = k.dt * w;
   if (w_out) *w_out = w;
@@ -142,13 +136,10 @@ __device__ __forceinline__ double root_f64(double A, double s, double G, double 
   double cc = x + s * G;
   return 2.0 * cc / (B + sqrt(B * B + 4.0 * A * cc));
 }
-// For the evaluation's sums, with dx'/dG = s (1 - x') / (2 A x' + B), 2 A x' + B = q: the two
-// quotients share the reciprocal of (B + q) q.
+// For the evaluation's sums, with dx'/dG = s (1 - x') / (2 A x' + B).
 __device__ __forceinline__ double root_slope_f64(double A, double s, double G, double x, double* dxdG) {
-  const double B = 1.0 + s * G, cc = x + s * G;
-  const double q = sqrt(B * B + 4.0 * A * cc), p = B + q, r = 1.0 / (p * q);
-  const double xr = 2.0 * cc * q * r;
-  *dxdG = s * (1.0 - xr) * p * r;
+  const double xr = root_f64(A, s, G, x);
+  *dxdG = s * (1.0 - xr) / (2.0 * A * xr + (1.0 + s * G));
   return xr;
 }
 
@@ -351,7 +342,7 @@ __device__ __forceinline__ float local_C_f32(const CoefF32& f, float div, float 
 // Coefficients of cell i for a pass of the FP64 form, computed (and kept) or read back.
 template <bool PART, int CACHE>
 __device__ __forceinline__ CellF64 pass_cell(const PassArgs& a, int64_t i, double d, double x, const double* T,
-                                             double wfac, double& Gc) {
+                                             double tot, double S1s, double& Gc) {
   CellF64 c;
   double Ci = 0.0;
   if (CACHE == kReadCache) {
@@ -361,7 +352,7 @@ __device__ __forceinline__ CellF64 pass_cell(const PassArgs& a, int64_t i, doubl
   } else {
     const uint32_t tal = (a.k.mixing == REC_MIX_TALLY) ? a.tally[i] : 0u;
     double w, tpd;
-    c = cell_f64(a.k, d, x, T[i], tal, wfac, &w, &tpd);
+    c = cell_f64(a.k, d, x, T[i], tal, tot, S1s, &w, &tpd);
     if (PART) Ci = local_C(a.k, ((const double*)a.div)[i], c.n * (1.0 - x));
     if (CACHE == kFillCache) {
       double4_32a q;
@@ -384,7 +375,7 @@ __device__ __forceinline__ CellF64 pass_cell(const PassArgs& a, int64_t i, doubl
 // PART: partial mixing — per cell, A scaled by f + (1 - f) C_i, s = dt f and G
 // offset by (1 - f)/f C_i beta e_alpha (C_i the local Peebles factor).
 template <bool MIXED, bool PART = false, int CACHE = kNoCache>
-__device__ __forceinline__ void newton_block_sums(const PassArgs& a, double lam, double G, double wfac,
+__device__ __forceinline__ void newton_block_sums(const PassArgs& a, double lam, double G, double tot, double S1s,
                                                   const MixedScal& ms, int blk, int nblk, double (&v)[5]) {
   const int64_t stride = (int64_t)nblk * NT;
   v[3] = v[4] = 0.0;
@@ -395,7 +386,7 @@ __device__ __forceinline__ void newton_block_sums(const PassArgs& a, double lam,
     for (int64_t i = (int64_t)blk * NT + threadIdx.x; i < a.n3; i += stride) {
       double d = delta[i], x = a.x[i];
       double Gc = G;
-      const CellF64 c = pass_cell<PART, CACHE>(a, i, d, x, T, wfac, Gc);
+      const CellF64 c = pass_cell<PART, CACHE>(a, i, d, x, T, tot, S1s, Gc);
       double dxdG;
       double xr = root_slope_f64(c.A, c.s, Gc, x, &dxdG);
       double an2 = c.al * c.n * c.n;
@@ -512,7 +503,7 @@ __device__ __forceinline__ void final_cell_mixed(const PassArgs& a, const FinalM
 // weights (zeroes the tallies on the last substep); partial sums (thread 0):
 // v0 = sum delta (1 - x'), v1 = sum delta x', v2 = sum delta.
 template <bool MIXED, bool PART = false, int CACHE = kNoCache>
-__device__ __forceinline__ void final_block(const PassArgs& a, double G, double wfac, const MixedScal& ms,
+__device__ __forceinline__ void final_block(const PassArgs& a, double G, double tot, double S1s, const MixedScal& ms,
                                             int blk, int nblk, double (&v)[3]) {
   const int64_t stride = (int64_t)nblk * NT;
   const bool zero_tally = a.k.last != 0;
@@ -525,7 +516,7 @@ __device__ __forceinline__ void final_block(const PassArgs& a, double G, double 
     for (int64_t i = (int64_t)blk * NT + threadIdx.x; i < a.n3; i += stride) {
       double d = delta[i], x = a.x[i];
       double Gc = G;
-      const CellF64 c = pass_cell<PART, CACHE>(a, i, d, x, T, wfac, Gc);
+      const CellF64 c = pass_cell<PART, CACHE>(a, i, d, x, T, tot, S1s, Gc);
       double xr = root_f64(c.A, c.s, Gc, x);
       double damp = exp(-(a.k.kd * xr + a.k.H) * a.k.dt);
       double4_32a u = U[i];
@@ -616,7 +607,7 @@ __global__ void __launch_bounds__(NT) k_newton(PassArgs a, const BoxDev* bxs, in
   constexpr int K = NSums<MIXED>::value;
   double v[5];
   newton_block_sums<MIXED, PART, CACHE>(a, lam, sc->omC * lam + sc->G0,
-                                        MIXED ? 0.0 : weight_factor((double)sc->tally_total, sc->S1s),
+                                        (double)sc->tally_total, sc->S1s,
                                         mixed_scal(sc, false), blk, nblk, v);
   if (threadIdx.x == 0) {
     double* p = a.part + (size_t)blk * kMaxSums;
@@ -705,7 +696,7 @@ __global__ void __launch_bounds__(NT) k_final(PassArgs a, rec_stats* st, const B
   DevScalars* sc = a.sc;
   const double lam = sc->lam;
   double v[3];
-  final_block<MIXED, PART>(a, sc->omC * lam + sc->G0, MIXED ? 0.0 : weight_factor((double)sc->tally_total, sc->S1s),
+  final_block<MIXED, PART>(a, sc->omC * lam + sc->G0, (double)sc->tally_total, sc->S1s,
                            mixed_scal(sc, false), blk, nblk, v);
   if (threadIdx.x == 0) {
     double* p = a.part + (size_t)blk * kMaxSums;
@@ -742,7 +733,7 @@ __global__ void __launch_bounds__(NT) k_batch_substep(PassArgs a0, rec_stats* st
       constexpr int K = NSums<MIXED>::value;
       double v[5];
       newton_block_sums<MIXED>(a, lam, __ldcg(&sc->omC) * lam + __ldcg(&sc->G0),
-                               MIXED ? 0.0 : weight_factor((double)__ldcg(&sc->tally_total), __ldcg(&sc->S1s)),
+                               (double)__ldcg(&sc->tally_total), __ldcg(&sc->S1s),
                                mixed_scal(sc, true), blk, nblk, v);
       if (threadIdx.x == 0) {
         double* p = a.part + (size_t)blk * kMaxSums;
@@ -769,7 +760,7 @@ __global__ void __launch_bounds__(NT) k_batch_substep(PassArgs a0, rec_stats* st
     const double lam = __ldcg(&sc->lam);
     double v[3];
     final_block<MIXED>(a, __ldcg(&sc->omC) * lam + __ldcg(&sc->G0),
-                       MIXED ? 0.0 : weight_factor((double)__ldcg(&sc->tally_total), __ldcg(&sc->S1s)),
+                       (double)__ldcg(&sc->tally_total), __ldcg(&sc->S1s),
                        mixed_scal(sc, true), blk, nblk, v);
     if (threadIdx.x == 0) {
       double* p = a.part + (size_t)blk * kMaxSums;
@@ -786,7 +777,7 @@ __global__ void __launch_bounds__(NT) k_batch_substep(PassArgs a0, rec_stats* st
 // Scalars of the substep as a block reads them: computed by every block itself
 // before the first evaluation (block 0 also stores them), through L2 after that.
 struct SubstepScal {
-  double lam, omC, G0, wfac;
+  double lam, omC, G0, tot, S1s;
   MixedScal ms;
 };
 // One thread per block: every thread's copy of these few binary64 operations
@@ -799,13 +790,13 @@ __device__ __forceinline__ SubstepScal substep_open(DevScalars* sc, const StepCo
     s.lam = b.lam;
     s.omC = 1.0 - b.C;
     s.G0 = b.C * k.beta * k.ea;
-    const double S1s = sc->S1s, tot = (double)sc->tally_total;
-    s.wfac = weight_factor(tot, S1s);
+    s.S1s = sc->S1s;
+    s.tot = (double)sc->tally_total;
     const double G = s.omC * s.lam + s.G0;
     s.ms.lamf = (float)s.lam;
     s.ms.Gf = (float)G;
     s.ms.Gd = df_from_double(G);
-    s.ms.wscale = sc->tally_total > 0 ? (float)(S1s / tot) : 0.0f;
+    s.ms.wscale = sc->tally_total > 0 ? (float)(s.S1s / s.tot) : 0.0f;
     open = s;
     // stored before this block arrives at the first barrier, so before any step on lambda
     if (blockIdx.x == 0) substep_begin(sc, k, n3);
@@ -832,8 +823,8 @@ __global__ void __launch_bounds__(NT, 4) k_substep(PassArgs a, rec_stats* st, in
     for (int g = blockIdx.x; g < nvb; g += gridDim.x) {
       double v[5];
       const double G = s.omC * s.lam + s.G0;
-      if (CACHE && pass > 0) newton_block_sums<MIXED, PART, CACHE ? kReadCache : kNoCache>(a, s.lam, G, s.wfac, s.ms, g, nvb, v);
-      else newton_block_sums<MIXED, PART, CACHE ? kFillCache : kNoCache>(a, s.lam, G, s.wfac, s.ms, g, nvb, v);
+      if (CACHE && pass > 0) newton_block_sums<MIXED, PART, CACHE ? kReadCache : kNoCache>(a, s.lam, G, s.tot, s.S1s, s.ms, g, nvb, v);
+      else newton_block_sums<MIXED, PART, CACHE ? kFillCache : kNoCache>(a, s.lam, G, s.tot, s.S1s, s.ms, g, nvb, v);
       if (threadIdx.x == 0) {
         double* p = a.part + (size_t)g * kMaxSums;
         for (int j = 0; j < K; ++j) p[j] = v[j];
@@ -850,7 +841,7 @@ __global__ void __launch_bounds__(NT, 4) k_substep(PassArgs a, rec_stats* st, in
   if constexpr (FINAL) {
     for (int g = blockIdx.x; g < nvb; g += gridDim.x) {
       double v[3];
-      final_block<MIXED, PART, CACHE ? kReadCache : kNoCache>(a, s.omC * s.lam + s.G0, s.wfac, s.ms, g, nvb, v);
+      final_block<MIXED, PART, CACHE ? kReadCache : kNoCache>(a, s.omC * s.lam + s.G0, s.tot, s.S1s, s.ms, g, nvb, v);
       if (threadIdx.x == 0) {
         double* p = a.part + (size_t)g * kMaxSums;
         p[0] = v[0]; p[1] = v[1]; p[2] = v[2];
@@ -1076,7 +1067,7 @@ __global__ void __launch_bounds__(NT) k_local(PassArgs a, const void* div, rec_s
     double* emis = (double*)a.emis;
     for (int64_t i = (int64_t)blockIdx.x * NT + threadIdx.x; i < a.n3; i += stride) {
       const double d = delta[i], x = a.x[i];
-      CellF64 c = cell_f64(k, d, x, T[i], 0u, 0.0);
+      CellF64 c = cell_f64(k, d, x, T[i], 0u, 0.0, 0.0);
       const double Ci = local_C(k, ((const double*)div)[i], c.n * (1.0 - x));
       // dx/dt = -C (alpha n_H x^2 - beta e_alpha (1 - x)), backward Euler
       const double xr = root_f64(c.A * Ci, c.s * Ci, bea, x);
