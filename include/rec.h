@@ -140,7 +140,8 @@ typedef struct {
   int32_t emit_blocks_per_sm;  /* emission grid, blocks of 256 threads per SM: 1..5 (FP64 form and batch 1..4) */
   int32_t march_blocks_per_sm; /* march grid: 1..4 (FP64 form and batch 1..3); with march_halo > 0
                                   1..3 (FP64 form 1..2) */
-  int32_t march_refill;        /* idle lanes of a warp that trigger a refill from the queue: 1..32 */
+  int32_t march_refill;        /* lanes of a warp that are idle or wait for the exact test of a cell,
+                                  which make it stop for those tests and a refill from the queue: 1..32 */
   int32_t march_chunk;         /* queued packets per unit of march work handed to a warp: 8..4096 */
   int32_t tile;                /* side of the super-tiles that order the march queue: 8, 16, 32 or 64 */
   int32_t march_halo;          /* region sweeps (single box, power-of-two side): 0 = off, every packet

@@ -161,11 +161,6 @@ template <> struct Draws<float> {
   // direction pairs each
   static constexpr int kPairs = 2;
   static constexpr uint32_t kQuantBlock = 0;  // its last word leads the quantile's bits
-  template <class S>
-  static __device__ __forceinline__ void position(const S& s, uint32_t c, uint32_t j, float f[3], float* uq) {
-    U4 r = draw(s, c, j, 0u);
-    f[0] = u01f(r.a); f[1] = u01f(r.b); f[2] = u01f(r.c); *uq = u01f(r.d);
-  }
   using Block = U4;
   static __device__ __forceinline__ bool first_of_block(int t) { return (t & 1) == 0; }
   template <class S>
@@ -753,12 +748,11 @@ struct TransportArgs {
   const R* quant;
   int M;
   R kappa, cth;
-  Stream strm;
-  Keys ks;  // round keys of strm (emission)
+  Keys ks;  // round keys of the step's stream (emission)
   uint32_t early;  // packets whose quantile word is below it have xi <= 0 (early_word)
   uint32_t* tally;
   DevScalars* sc;
-  typename Vec4<R>::T* queue;  // 3 entries per queued packet
+  typename Vec4<R>::T* queue;  // QueueVecs entries per queued packet (3 where a sweep resumes)
   Tiles tl;
   int nb;                          // buckets (super-tiles)
   unsigned long long* boff;        // bucket start in the queue (capacity prefix)
@@ -1990,7 +1984,6 @@ cudaError_t run_transport(rec_ctx* c, int step, double z, rec_stats* st) {
   a.M = c->params.n_quantiles;
   a.kappa = (R)kappa;
   a.cth = (R)cth;
-  a.strm = s;
   a.ks = key_schedule(s.k0, s.k1);
   a.early = early_word(c, kappa, cth);
   a.tally = b.tally;
@@ -2311,7 +2304,6 @@ cudaError_t run_transport_batch(rec_ctx* c, int step, double z, rec_stats* st) {
   std::memset(&a, 0, sizeof(a));
   a.quant = (const R*)c->quant;
   a.M = c->params.n_quantiles;
-  a.strm = Stream{k0, k1, 0u};
   a.ks = key_schedule(k0, k1);
   double kappa_max = 0.0, cth_max = 0.0;
   for (int b = 0; b < B; ++b) {
