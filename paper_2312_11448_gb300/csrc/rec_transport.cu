@@ -279,13 +279,13 @@ __device__ __forceinline__ void block_maxima(DevScalars* sc, uint64_t w, const V
 template <class R>
 __device__ __forceinline__ void take_maxima(DevScalars* sc, int64_t n3, float kappa) {
   const uint32_t bad = __ldcg(&sc->mx_bad);
-  sc->rmax = bad & 1u ? 0.0 : (double)from_order_bits(__ldcg(&sc->mx_w), (R)0);  // invalid weights: emit nothing
-  sc->flags &= ~(2 | 4 | 16);                                                    // transport flags describe this call only
-  if (bad & 1u) sc->flags |= 4;
-  const float umax = __uint_as_float(__ldcg(&sc->mx_u));
+  const unsigned long long w = __ldcg(&sc->mx_w);
+  const float umax = __uint_as_float(__ldcg(&sc->mx_u)), v2 = __uint_as_float(__ldcg(&sc->mx_v2));
   const float u = velq_scale(umax, __ldcg(&sc->mx_sum) / (3.0f * (float)n3), kappa);
+  sc->rmax = bad & 1u ? 0.0 : (double)from_order_bits(w, (R)0);  // invalid weights: emit nothing
+  sc->flags = (sc->flags & ~(2 | 4 | 16)) | (bad & 1u ? 4 : 0);  // transport flags describe this call only
   sc->vq_u = u;
-  sc->vq_v = bad & 2u ? __int_as_float(0x7f800000) : sqrtf(__uint_as_float(__ldcg(&sc->mx_v2))) * 1.00001f;
+  sc->vq_v = bad & 2u ? __int_as_float(0x7f800000) : sqrtf(v2) * 1.00001f;
   sc->vq_out = (bad & 2u) || umax > u;
   sc->vel_plain = !(bad & 2u) && umax < 1e15f;
   sc->mx_sum = 0.0f;
