@@ -878,13 +878,15 @@ def run_ours(args):
         """rec_step against the fixed per-cell-step count of a step with two
         evaluation passes and the final pass (20 + 20 + 64 B mixed): the
         Halley update needs one pass where Newton needed two, which the
-        method-byte fraction above does not credit."""
+        method-byte fraction above does not credit.  The fraction of the
+        passes that run is roofline_other.rec_step."""
         if "rec_step" not in groups:
             return None
         ms_s = groups["rec_step"][0] / k_steps
         b = 104 * n3
         return {"bytes_per_cell_step": 104, "ms_per_step": ms_s, "achieved": b / (ms_s * 1e-3) / 1e9,
-                "frac": b / (ms_s * 1e-3) / 1e9 / peak, "unit": "GB/s", "peak": peak}
+                "frac": b / (ms_s * 1e-3) / 1e9 / peak, "unit": "GB/s", "peak": peak,
+                "rule": "two evaluation passes counted; newton_passes of them run"}
 
     def whole_step(r, k_steps, ms_total):
         ms_s = ms_total / k_steps

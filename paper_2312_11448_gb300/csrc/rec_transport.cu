@@ -1328,8 +1328,8 @@ __global__ void __launch_bounds__(TT, emit_occupancy<R>()) k_emit(TransportArgs<
 // What bounds it: with flows of 1 km/s, requests from L1 to L2 (72 % busy), instruction
 // issue (68 %) and the integer pipe (66 %) together; once Compton drag has slowed the
 // flow most cells need no load, and it is issue (74 %) and the integer pipe (73 %).  With
-// the velocity vector read in every cell it was the requests alone (87 %): 256^3, 1e8 packets 5.34 -> 3.38 ms, FP64 47.4 -> 8.0 ms;
-// 512^3, 1e9 packets with sweeps 111 -> 65.3 ms.
+// the velocity vector read in every cell it was the requests alone (87 %): 256^3, 1e8 packets 5.34 -> 3.36 ms, FP64 47.4 -> 7.9 ms;
+// 512^3, 1e9 packets with sweeps 111 -> 65.7 ms.
 // Cells a lane walks per round, with their words in flight together (256^3 mixed: 3 / 4 /
 // 5 / 6 cells 4.07 / 3.57 / 3.60 / 3.43 ms, 8 cells 3.69 at three blocks per SM; FP64: 4 / 6
 // cells 7.97 / 8.28 ms; region sweeps of 512^3, 1e9 packets, leaving packets queued after every

@@ -39,7 +39,8 @@ __host__ __device__ inline uint32_t velq_y(uint32_t iy, uint32_t bx) {
 __host__ __device__ inline uint32_t velq_z(uint32_t iz, uint32_t bx) {
   return ((iz & 1u) << 2) | ((iz >> 1) << (5u + 2u * bx));
 }
-// Words of the copy of an n^3 box (n <= 1024: at most 2^30).
+// Words of the copy of an n^3 box (n <= 1024: at most 2^30).  x and y are padded to a power of
+// two, so n^3 words for such sides and up to four times as many just above one.
 __host__ __device__ inline uint64_t velq_words(uint32_t n) {
   return (uint64_t)((n + 1u) >> 1) << (5u + 2u * velq_bits(n));
 }
